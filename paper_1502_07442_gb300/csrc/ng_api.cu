@@ -575,21 +575,59 @@ __global__ void k_resident_load(int64_t n, const double* __restrict__ pos,
   }
 }
 
-// The resident state back to the caller's order: positions, velocities and
-// accelerations scattered to their caller indices.
-__global__ void k_resident_store(int64_t n, const uint32_t* __restrict__ rorig,
-                                 const double* __restrict__ rpos, const float* __restrict__ rvel,
-                                 const float* __restrict__ racc, double* __restrict__ pos,
-                                 float* __restrict__ vel, float* __restrict__ acc) {
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n;
-       k += (int64_t)gridDim.x * blockDim.x) {
-    const uint32_t i = rorig[k];
+// The resident state back to the caller's order, in two launches: each body's
+// 48 bytes of positions, velocities and accelerations go to its caller index
+// as one 64-byte record, then the records are unpacked in caller order.
+// Scattering the nine arrays directly writes 4 or 8 bytes of a 32-byte sector
+// at a time (2^24 bodies: 5.6 ms, against 0.72 ms).
+constexpr int kPackTile = 256;
+
+__global__ void __launch_bounds__(kPackTile)
+k_resident_pack(int64_t n, const uint32_t* __restrict__ rorig, const double* __restrict__ rpos,
+                const float* __restrict__ rvel, const float* __restrict__ racc,
+                uint4* __restrict__ rec) {
+  __shared__ uint4 tile[kPackTile][3];
+  __shared__ uint32_t dst[kPackTile];
+  const int tid = threadIdx.x;
+  const int64_t k = blockIdx.x * (int64_t)kPackTile + tid;
+  if (k < n) {
+    double* p = reinterpret_cast<double*>(tile[tid]);
+    float* f = reinterpret_cast<float*>(tile[tid]) + 6;
 #pragma unroll
     for (int e = 0; e < 3; ++e) {
-      pos[e * n + i] = rpos[e * n + k];
-      vel[e * n + i] = rvel[e * n + k];
-      acc[e * n + i] = racc[e * n + k];
+      p[e] = rpos[e * n + k];
+      f[e] = rvel[e * n + k];
+      f[3 + e] = racc[e * n + k];
     }
+    dst[tid] = rorig[k];
+  }
+  __syncthreads();
+  // four lanes write one record (its last 16 bytes stay unused)
+  const int here = (int)min((int64_t)kPackTile, n - blockIdx.x * (int64_t)kPackTile);
+  for (int j = tid; j < 4 * here; j += kPackTile) {
+    const int b = j >> 2, part = j & 3;
+    rec[(size_t)dst[b] * 4 + part] = tile[b][part < 3 ? part : 0];
+  }
+}
+
+__global__ void __launch_bounds__(kPackTile)
+k_resident_unpack(int64_t n, const uint4* __restrict__ rec, double* __restrict__ pos,
+                  float* __restrict__ vel, float* __restrict__ acc) {
+  __shared__ uint4 tile[kPackTile][3];
+  const int tid = threadIdx.x;
+  const int64_t k0 = blockIdx.x * (int64_t)kPackTile, k = k0 + tid;
+  const int here = (int)min((int64_t)kPackTile, n - k0);
+  for (int j = tid; j < 4 * here; j += kPackTile)
+    if ((j & 3) < 3) tile[j >> 2][j & 3] = rec[(size_t)k0 * 4 + j];
+  __syncthreads();
+  if (k >= n) return;
+  const double* p = reinterpret_cast<const double*>(tile[tid]);
+  const float* f = reinterpret_cast<const float*>(tile[tid]) + 6;
+#pragma unroll
+  for (int e = 0; e < 3; ++e) {
+    pos[e * n + k] = p[e];
+    vel[e * n + k] = f[e];
+    acc[e * n + k] = f[3 + e];
   }
 }
 
@@ -612,6 +650,7 @@ int reserve_resident(ng_ctx* c, int64_t n) {
   NG_TRY(ensure(c, c->rorig_alt, (size_t)n * 4));
   NG_TRY(ensure(c, c->racc, (size_t)n * 12));
   NG_TRY(ensure(c, c->rtmp, (size_t)n * 4));
+  NG_TRY(ensure(c, c->rpack, (size_t)n * 64));
   return NG_OK;
 }
 
@@ -643,10 +682,12 @@ int resident_load(ng_ctx* c, int64_t n, const double* pos, const float* vel,
 // bodies of the last step to caller indices, as after ng_build_tree, and the
 // relative criterion's |a_old| returns to caller order.
 int resident_store(ng_ctx* c, int64_t n, double* pos, float* vel, float* acc) {
-  k_resident_store<<<work_grid(c, n, 8), 256, 0, c->stream>>>(
-      n, as<uint32_t>(c->rorig), as<double>(c->spos), as<float>(c->rvel), as<float>(c->racc), pos,
-      vel, acc);
-  c->launches += 1;
+  const int grid = (int)((n + kPackTile - 1) / kPackTile);
+  k_resident_pack<<<grid, kPackTile, 0, c->stream>>>(n, as<uint32_t>(c->rorig), as<double>(c->spos),
+                                                     as<float>(c->rvel), as<float>(c->racc),
+                                                     as<uint4>(c->rpack));
+  k_resident_unpack<<<grid, kPackTile, 0, c->stream>>>(n, as<uint4>(c->rpack), pos, vel, acc);
+  c->launches += 2;
   NG_CUDA(c, cudaGetLastError());
   NG_CUDA(c, cudaMemcpyAsync(c->vals_a.p, c->rorig.p, (size_t)n * 4, cudaMemcpyDeviceToDevice,
                              c->stream));
@@ -758,7 +799,7 @@ int ng_destroy(ng_ctx* c) {
                     &c->status, &c->counter, &c->aold, &c->io_pos, &c->io_vel, &c->io_type, &c->io_mass,
                     &c->io_acc, &c->lattice, &c->rho, &c->rhok, &c->phi,
                     &c->walk_desc, &c->walk_prefix, &c->spos_alt, &c->smass_alt, &c->stype_alt,
-                    &c->rvel, &c->rvel_alt, &c->rorig, &c->rorig_alt, &c->racc, &c->rtmp};
+                    &c->rvel, &c->rvel_alt, &c->rorig, &c->rorig_alt, &c->racc, &c->rtmp, &c->rpack};
   for (DevBuf* b : bufs) release(*b);
   delete c;
   return NG_OK;

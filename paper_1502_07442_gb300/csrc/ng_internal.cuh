@@ -307,7 +307,7 @@ struct ng_ctx {
   // swaps them with their *_alt partners, gathers the previous state into
   // sorted order and writes the forces in that order.
   bool resident = false;
-  ng::DevBuf spos_alt, smass_alt, stype_alt, rvel, rvel_alt, rorig, rorig_alt, racc, rtmp;
+  ng::DevBuf spos_alt, smass_alt, stype_alt, rvel, rvel_alt, rorig, rorig_alt, racc, rtmp, rpack;
   cudaGraphExec_t step_exec_b = nullptr;   // the step with the buffer roles exchanged
   int step_parity = 0;
 
