@@ -791,7 +791,7 @@ int ng_destroy(ng_ctx* c) {
       cufftDestroy(pl.c2r);
     }
   }
-  DevBuf* bufs[] = {&c->d_tab, &c->keys_a, &c->keys_b, &c->vals_a, &c->vals_b, &c->blockhist,
+  DevBuf* bufs[] = {&c->d_tab, &c->keys_a, &c->keys_b, &c->vals_a, &c->vals_b, &c->sort_words, &c->lookback,
                     &c->spos, &c->smass, &c->stype, &c->body, &c->bleaf,
                     &c->tperm, &c->scan_part, &c->n_level, &c->n_prefix, &c->n_first,
                     &c->n_count, &c->n_child, &c->n_nchild, &c->n_tmp, &c->n_m64,
@@ -1178,16 +1178,12 @@ int ng_type_order(ng_ctx* c, int64_t* type_offsets, uint32_t* order_out) {
   if (!c) return NG_EINVAL;
   if (!c->built) return fail(c, NG_ESTATE, "no tree built");
   const int64_t n = c->n;
-  const int nblocks = (int)((n + kRadixTile - 1) / kRadixTile);
   if (type_offsets) {
+    uint32_t cnt[8];
     NG_CUDA(c, cudaStreamSynchronize(c->stream));
-    for (int d = 0; d < c->p.D; ++d) {
-      uint32_t v = 0;
-      NG_CUDA(c, cudaMemcpy(&v, as<uint32_t>(c->blockhist) + (size_t)d * nblocks, 4,
-                            cudaMemcpyDeviceToHost));
-      type_offsets[d] = v;
-    }
-    type_offsets[c->p.D] = n;
+    NG_CUDA(c, cudaMemcpy(cnt, type_counts(c), sizeof(cnt), cudaMemcpyDeviceToHost));
+    type_offsets[0] = 0;
+    for (int d = 0; d < c->p.D; ++d) type_offsets[d + 1] = type_offsets[d] + cnt[d];
   }
   if (order_out) {
     // caller indices in type-major order: perm[tperm[j]]

@@ -174,10 +174,6 @@ __device__ __forceinline__ uint64_t sort_key(double x, double y, double z, uint8
   return (m << 3) | (uint64_t)(type & 7);
 }
 
-// Keys per block of the radix sort; the per-block digit histograms (and the
-// type offsets read back from the last pass's) are laid out by it.
-constexpr int kRadixTile = 2048;
-
 // Entries per row of a single simulation's law table: the passive species
 // count rounded up to a power of two (a row of the table of list species t
 // holds the law of every passive species s; see walk_table).
@@ -278,13 +274,15 @@ struct ng_ctx {
   // particles of the last build
   int64_t n = 0;
   bool built = false;
-  ng::DevBuf keys_a, keys_b, vals_a, vals_b, blockhist;
+  ng::DevBuf keys_a, keys_b, vals_a, vals_b;
+  ng::DevBuf sort_words, lookback;   // histograms and tickets of the sort; tile states (ng_sort.cu)
   ng::DevBuf spos, smass, stype, body, bleaf, tperm, scan_part;
 
   // tree
   int64_t cap_nodes = 0, nnodes = 0;
   int level_cap = ng::kMaxLevel;   // deepest level a build emits (captured steps: depth_seen + 2)
   int depth_seen = ng::kMaxLevel;  // deepest non-empty level of the last checked build
+  bool typed = false;              // tperm holds the type-major order of the last sort
   int sort_passes = 0;             // radix passes of the last key sort
   int64_t ngroups = 0, ngroups_n = -1;   // walk groups of the last checked build, for n = ngroups_n
   ng::DevBuf n_level, n_prefix, n_first, n_count, n_child, n_nchild, n_tmp;
@@ -434,7 +432,8 @@ int reserve_sort(ng_ctx* c, int64_t n);        // sort buffers for n bodies
 // calling thread; the stages that follow then allocate nothing).
 int reserve(ng_ctx* c, int64_t n);
 extern std::mutex g_fft_plan_lock;   // see pm_setup
-int type_order(ng_ctx* c);
+int type_order(ng_ctx* c);                    // needs the gather of the sort
+const uint32_t* type_counts(const ng_ctx* c);  // device: bodies of species 0..7 of the last sort
 
 // Host short-range law tables (double precision closed forms).
 int build_tables(ng_ctx* c);

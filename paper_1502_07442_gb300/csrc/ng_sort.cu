@@ -106,139 +106,397 @@ int scan_u32_flags(ng_ctx* c, const uint32_t* in, uint32_t* out, int64_t len, ui
 
 // --------------------------------------------------------------- keys
 
-__global__ void k_keys(int64_t n, const double* __restrict__ pos, const uint8_t* __restrict__ type,
-                       double L, double invL, bool pow2, int ebox, uint64_t* __restrict__ keys,
-                       uint32_t* __restrict__ idx) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    keys[i] = sort_key(pos[i], pos[n + i], pos[2 * n + i], type[i], L, invL, pow2, ebox);
-    idx[i] = (uint32_t)i;
+struct KeyArgs {
+  int64_t n;
+  const double* pos;
+  const uint8_t* type;
+  double L, invL;
+  bool pow2;
+  int ebox, D;
+};
+
+__device__ __forceinline__ uint64_t body_key(const KeyArgs& a, int64_t i, uint8_t type) {
+  return sort_key(a.pos[i], a.pos[a.n + i], a.pos[2 * a.n + i], type, a.L, a.invL, a.pow2, a.ebox);
+}
+
+// A species as the gather stores it (out of range: 0, flagged there).
+__device__ __forceinline__ uint32_t stored_type(uint8_t t, int D) { return t < D ? t : 0u; }
+
+// Words of the sort (c->sort_words): the digit histograms of the 8 passes,
+// the species counts (kept until the next sort: the starts of the type-major
+// order), and one tile ticket per pass and for the type order.
+constexpr int kSwTypes = 8 * 256, kSwTickets = kSwTypes + 8, kSortWords = kSwTickets + 9;
+
+// Look-back state of one (tile, digit): 0, or a flag in the top bits and a
+// body count below (64 bits: counts up to the largest n).
+constexpr uint64_t kLbAggregate = 1ull << 62, kLbPrefix = 2ull << 62, kLbCount = (1ull << 62) - 1;
+
+__device__ __forceinline__ uint64_t lb_load(const uint64_t* p) {
+  uint64_t v;
+  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ void lb_store(uint64_t* p, uint64_t v) {
+  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+// Polls of one state before a tile stops waiting and counts the digits before
+// it from the input itself. Tiles are numbered by ticket, so the tile waited
+// for always runs and never waits for this one; the limit only bounds the wait.
+constexpr int kLbPolls = 1 << 20;
+
+// Keys of all bodies, the digit histograms of passes first..7 and the species
+// counts; clears the look-back state of the first pass and of the type order.
+__global__ void __launch_bounds__(512)
+k_keys(KeyArgs a, int first, uint64_t* __restrict__ keys, uint32_t* words,
+       uint64_t* __restrict__ lb, int64_t lb_words, uint64_t* __restrict__ lbt, int64_t lbt_words) {
+  __shared__ uint32_t h[8][256];
+  __shared__ uint32_t ht[8];
+  for (int j = threadIdx.x; j < 8 * 256; j += blockDim.x) (&h[0][0])[j] = 0;
+  if (threadIdx.x < 8) ht[threadIdx.x] = 0;
+  __syncthreads();
+  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t j = t; j < lb_words; j += stride) lb[j] = 0;
+  for (int64_t j = t; j < lbt_words; j += stride) lbt[j] = 0;
+  for (int64_t i = t; i < a.n; i += stride) {
+    const uint8_t ty = a.type[i];
+    const uint64_t k = body_key(a, i, ty);
+    keys[i] = k;
+#pragma unroll
+    for (int p = 0; p < 8; ++p)
+      if (p >= first) atomicAdd(&h[p][(uint32_t)(k >> (8 * p)) & 0xffu], 1u);
+    atomicAdd(&ht[stored_type(ty, a.D)], 1u);
   }
+  __syncthreads();
+  for (int j = threadIdx.x; j < 8 * 256; j += blockDim.x)
+    if ((&h[0][0])[j]) atomicAdd(&words[j], (&h[0][0])[j]);
+  if (threadIdx.x < 8 && ht[threadIdx.x]) atomicAdd(&words[kSwTypes + threadIdx.x], ht[threadIdx.x]);
 }
 
 // ---------------------------------------------------------- radix sort
 
+// One stable pass on one 8-bit digit, in one launch: each block takes the
+// next tile of kRsThreads * ITEMS keys, ranks it by digit (each warp its
+// contiguous run in order, ballots group equal digits; then warps in order
+// per digit), publishes the tile's digit counts, adds up those of the tiles
+// before it until it meets one that published its prefix, and writes the keys
+// out through shared memory, so that each digit's run of the tile leaves as
+// one contiguous segment. It reads and writes 12 B a key once and waits mostly
+// on its own phases (ranking, look-back, write-out). A histogram, a scan and a
+// scatter launch per pass read the keys twice and cost two to three launches
+// more (8 passes: 131k bodies 190 -> 75 us, 3 M 470 -> 320 us; 4096 bodies
+// 145 -> 57 us). ITEMS is small for few keys, so that every SM has a tile.
 constexpr int kRsThreads = 256;
-constexpr int kRsItems = 8;                        // keys per lane
 constexpr int kRsWarps = kRsThreads / 32;
-constexpr int kRsTile = kRsThreads * kRsItems;     // 2048 keys per block
-static_assert(kRsTile == kRadixTile, "radix tile and histogram layout disagree");
+constexpr int kRsItemsSmall = 4, kRsItemsLarge = 16;
+// two tiles of the larger kind per SM
+constexpr int64_t kRsLarge = (int64_t)2 * 152 * kRsThreads * kRsItemsLarge;
 
-__global__ void __launch_bounds__(kRsThreads)
-k_rs_hist(const uint64_t* __restrict__ keys, int64_t n, int shift, uint32_t mask,
-          uint32_t* __restrict__ hist, int nblocks) {
-  __shared__ uint32_t cnt[256];
-  cnt[threadIdx.x] = 0;
-  __syncthreads();
-  const int64_t t0 = (int64_t)blockIdx.x * kRsTile;
-  for (int j = threadIdx.x; j < kRsTile; j += kRsThreads) {
-    const int64_t i = t0 + j;
-    if (i < n) atomicAdd(&cnt[(uint32_t)(keys[i] >> shift) & mask], 1u);
+// Look-back state of one pass. Tiles form groups of kRsGroup: a tile adds up
+// the tiles before it in its group (their states loaded together) and the
+// groups before; the last tile of a group publishes the group's counts. The tiles of a wave publish at about the same time, so walking
+// back tile by tile would cost a tile hundreds of loads in a row (3 M bodies:
+// 53 us a pass, 40 us with groups and the tile size below).
+constexpr int kRsGroup = 16;
+struct RsLookback {
+  uint64_t* tile;       // [tile][256]: aggregates
+  uint64_t* group;      // [group][256]: aggregates, then prefixes
+};
+
+template <int ITEMS>
+struct RsSmem {
+  uint32_t wcnt[kRsWarps][256];   // per warp and digit: count, then place in the digit's run
+  uint32_t dstart[256];           // tile position of each digit's run
+  int64_t gdst[256];              // global position of each digit's run less its tile position
+  uint32_t wsum[2][kRsWarps];
+  uint32_t tile;
+  uint64_t tk[kRsThreads * ITEMS];
+  uint32_t tv[kRsThreads * ITEMS];
+};
+
+// Lanes of the warp whose 8-bit digit equals this lane's (of the lanes in
+// `in`): one ballot per bit (match.any, which waits for the memory pipe: 66 us a
+// 3 M pass, ballots 47 us).
+__device__ __forceinline__ uint32_t digit_peers(uint32_t d, uint32_t in) {
+  uint32_t p = in;
+#pragma unroll
+  for (int b = 0; b < 8; ++b) {
+    const uint32_t m = __ballot_sync(0xffffffffu, d >> b & 1u);
+    p &= d >> b & 1u ? m : ~m;
   }
-  __syncthreads();
-  hist[(int64_t)threadIdx.x * nblocks + blockIdx.x] = cnt[threadIdx.x];
+  return p;
 }
 
-// Stable scatter of one digit. Each warp ranks its contiguous sub-tile in
-// order (match_any groups equal digits); warps are ordered per digit. The
-// tile is then reordered by digit in shared memory and written out by
-// consecutive threads, so each digit's run of the tile (16 keys on average)
-// leaves as one contiguous segment instead of one sector per key.
-__global__ void __launch_bounds__(kRsThreads)
-k_rs_scatter(const uint64_t* __restrict__ kin, const uint32_t* __restrict__ vin,
-             uint64_t* __restrict__ kout, uint32_t* __restrict__ vout, int64_t n, int shift,
-             uint32_t mask, const uint32_t* __restrict__ offs, int nblocks) {
-  __shared__ uint32_t wcnt[kRsWarps][256];   // per warp and digit: count, then tile position
-  __shared__ uint32_t dstart[256];           // tile position of each digit's run
-  __shared__ uint32_t gdst[256];             // global position of each digit's run
-  __shared__ uint64_t tk[kRsTile];
-  __shared__ uint32_t tv[kRsTile];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  for (int j = threadIdx.x; j < kRsWarps * 256; j += kRsThreads) (&wcnt[0][0])[j] = 0;
+template <int ITEMS>
+__global__ void __launch_bounds__(kRsThreads, 3)
+k_rs_pass(const uint64_t* __restrict__ kin, const uint32_t* __restrict__ vin,
+          uint64_t* __restrict__ kout, uint32_t* __restrict__ vout, int64_t n, int shift,
+          const uint32_t* __restrict__ hist, uint32_t* ticket, RsLookback lb, RsLookback lb_next) {
+  extern __shared__ __align__(16) unsigned char rs_raw[];
+  RsSmem<ITEMS>& sm = *reinterpret_cast<RsSmem<ITEMS>*>(rs_raw);
+  constexpr int kTile = kRsThreads * ITEMS;
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  if (tid == 0) sm.tile = atomicAdd(ticket, 1u);
+  for (int j = tid; j < kRsWarps * 256; j += kRsThreads) (&sm.wcnt[0][0])[j] = 0;
   __syncthreads();
-  const int64_t t0 = (int64_t)blockIdx.x * kRsTile;
-  const int64_t sub0 = t0 + (int64_t)w * (kRsTile / kRsWarps);
+  const int64_t tile = sm.tile;
+  const int64_t group = tile / kRsGroup, g0 = group * kRsGroup;
+  const int64_t t0 = tile * kTile;
+  const int64_t sub0 = t0 + (int64_t)w * (32 * ITEMS);
   const uint32_t lt = (1u << lane) - 1u;
-  uint64_t k[kRsItems];
-  uint32_t v[kRsItems], rank[kRsItems];
+  uint64_t k[ITEMS];
+  uint32_t rank[ITEMS];
 #pragma unroll
-  for (int it = 0; it < kRsItems; ++it) {
+  for (int it = 0; it < ITEMS; ++it) {
     const int64_t i = sub0 + it * 32 + lane;
-    const bool valid = i < n;
-    k[it] = valid ? kin[i] : 0ull;
-    v[it] = valid ? vin[i] : 0u;
-    const uint32_t d = (uint32_t)(k[it] >> shift) & mask;
-    const uint32_t peers = __match_any_sync(0xffffffffu, valid ? d : 0xffffffffu);
-    uint32_t prior = 0;
-    if (valid) prior = wcnt[w][d];
-    __syncwarp();
-    rank[it] = prior + __popc(peers & lt);
-    if (valid && (peers & lt) == 0) wcnt[w][d] = prior + __popc(peers);
-    __syncwarp();
+    k[it] = i < n ? kin[i] : 0ull;
+  }
+#pragma unroll
+  for (int h = 0; h < ITEMS; h += 4) {
+    // the ballots of four items overlap; their counts follow in order
+    uint32_t peers[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const bool valid = sub0 + (h + j) * 32 + lane < n;
+      peers[j] = digit_peers((uint32_t)(k[h + j] >> shift) & 0xffu, __ballot_sync(0xffffffffu, valid));
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const bool valid = sub0 + (h + j) * 32 + lane < n;
+      const uint32_t d = (uint32_t)(k[h + j] >> shift) & 0xffu;
+      const uint32_t prior = sm.wcnt[w][d];
+      __syncwarp();
+      rank[h + j] = prior + __popc(peers[j] & lt);
+      if (valid && (peers[j] & lt) == 0) sm.wcnt[w][d] = prior + __popc(peers[j]);
+      __syncwarp();
+    }
   }
   __syncthreads();
-  {
-    // thread d: the digit's total in the tile, its run's tile start (block
-    // scan over digits) and the warps' positions inside the run
-    const int d = threadIdx.x;
-    uint32_t total = 0;
-#pragma unroll
-    for (int ww = 0; ww < kRsWarps; ++ww) total += wcnt[ww][d];
-    uint32_t incl = total;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += t;
-    }
-    __shared__ uint32_t wsum[kRsWarps];
-    if (lane == 31) wsum[w] = incl;
-    __syncthreads();
-    uint32_t wbase = 0;
-    for (int ww = 0; ww < w; ++ww) wbase += wsum[ww];
-    uint32_t run = wbase + incl - total;
-    dstart[d] = run;
-    gdst[d] = offs[(int64_t)d * nblocks + blockIdx.x];
+  uint32_t total = 0, incl = 0, gincl = 0, gtot = 0;
+  if (tid < 256) {
+    // thread d: the digit's total in the tile, published at once
 #pragma unroll
     for (int ww = 0; ww < kRsWarps; ++ww) {
-      const uint32_t t = wcnt[ww][d];
-      wcnt[ww][d] = run;
-      run += t;
+      const uint32_t t = sm.wcnt[ww][tid];
+      sm.wcnt[ww][tid] = total;
+      total += t;
     }
-  }
-  __syncthreads();
+    lb_store(&lb.tile[tile * 256 + tid], kLbAggregate | total);
+    lb_next.tile[tile * 256 + tid] = 0;
+    if (tile == g0) lb_next.group[group * 256 + tid] = 0;
+    gtot = hist[tid];
+    incl = total;
+    gincl = gtot;
 #pragma unroll
-  for (int it = 0; it < kRsItems; ++it) {
-    const int64_t i = sub0 + it * 32 + lane;
-    if (i < n) {
-      const uint32_t d = (uint32_t)(k[it] >> shift) & mask;
-      const uint32_t pos = wcnt[w][d] + rank[it];
-      tk[pos] = k[it];
-      tv[pos] = v[it];
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t x = __shfl_up_sync(0xffffffffu, incl, o), y = __shfl_up_sync(0xffffffffu, gincl, o);
+      if (lane >= o) {
+        incl += x;
+        gincl += y;
+      }
+    }
+    if (lane == 31) {
+      sm.wsum[0][w] = incl;
+      sm.wsum[1][w] = gincl;
     }
   }
   __syncthreads();
-  const int valid = (int)((n - t0) < kRsTile ? (n - t0) : kRsTile);
-  for (int p = threadIdx.x; p < valid; p += kRsThreads) {
-    const uint64_t key = tk[p];
-    const uint32_t d = (uint32_t)(key >> shift) & mask;
-    const uint32_t dst = gdst[d] + ((uint32_t)p - dstart[d]);
+  uint32_t base = incl - total, gbase = gincl - gtot;
+  if (tid < 256) {
+    for (int ww = 0; ww < w; ++ww) {
+      base += sm.wsum[0][ww];
+      gbase += sm.wsum[1][ww];
+    }
+    sm.dstart[tid] = base;
+  }
+  __syncthreads();
+  // the tile by digit in shared memory, while the other tiles publish
+#pragma unroll
+  for (int it = 0; it < ITEMS; ++it) {
+    if (sub0 + it * 32 + lane < n) {
+      const uint32_t d = (uint32_t)(k[it] >> shift) & 0xffu;
+      const uint32_t at = sm.dstart[d] + sm.wcnt[w][d] + rank[it];
+      sm.tk[at] = k[it];
+      sm.tv[at] = vin ? vin[sub0 + it * 32 + lane] : (uint32_t)(sub0 + it * 32 + lane);
+    }
+  }
+  if (tid < 256) {
+    // the digit's bodies in the tiles of the group before this one; several
+    // states at a time, so that their loads overlap
+    constexpr int kBatch = 8;
+    uint64_t before = 0;
+    for (int64_t t = g0; t < tile; t += kBatch) {
+      uint64_t st[kBatch];
+#pragma unroll
+      for (int j = 0; j < kBatch; ++j)
+        st[j] = t + j < tile ? lb_load(&lb.tile[(t + j) * 256 + tid]) : kLbAggregate;
+#pragma unroll
+      for (int j = 0; j < kBatch; ++j) {
+        for (int poll = 0; st[j] == 0 && poll < kLbPolls; ++poll)
+          st[j] = lb_load(&lb.tile[(t + j) * 256 + tid]);
+        if (st[j] == 0)
+          for (int64_t i = (t + j) * kTile; i < (t + j + 1) * kTile; ++i)
+            st[j] += ((uint32_t)(kin[i] >> shift) & 0xffu) == (uint32_t)tid;
+        before += st[j] & kLbCount;
+      }
+    }
+    // the last tile of a group publishes the group's count
+    const bool last = tile == g0 + kRsGroup - 1;
+    const uint64_t gsum = before + total;
+    if (last) lb_store(&lb.group[group * 256 + tid], (group == 0 ? kLbPrefix : kLbAggregate) | gsum);
+    // and in the groups before, back to the nearest prefix
+    uint64_t gbefore = 0;
+    bool done = false;
+    for (int64_t t = group - 1; t >= 0 && !done; t -= kBatch) {
+      uint64_t st[kBatch];
+#pragma unroll
+      for (int j = 0; j < kBatch; ++j)
+        st[j] = t - j >= 0 ? lb_load(&lb.group[(t - j) * 256 + tid]) : kLbPrefix;
+#pragma unroll
+      for (int j = 0; j < kBatch; ++j) {
+        if (done) continue;
+        for (int poll = 0; st[j] == 0 && poll < kLbPolls; ++poll)
+          st[j] = lb_load(&lb.group[(t - j) * 256 + tid]);
+        if (st[j] == 0) {
+          for (int64_t i = 0; i < (t - j + 1) * kRsGroup * kTile; ++i)
+            gbefore += ((uint32_t)(kin[i] >> shift) & 0xffu) == (uint32_t)tid;
+          st[j] = kLbPrefix;
+        }
+        gbefore += st[j] & kLbCount;
+        done = (st[j] & kLbPrefix) != 0;
+      }
+    }
+    if (last && group > 0) lb_store(&lb.group[group * 256 + tid], kLbPrefix | (gbefore + gsum));
+    sm.gdst[tid] = (int64_t)gbase + (int64_t)(before + gbefore) - (int64_t)base;
+  }
+  __syncthreads();
+  const int valid = (int)((n - t0) < kTile ? (n - t0) : kTile);
+  for (int p = tid; p < valid; p += kRsThreads) {
+    const uint64_t key = sm.tk[p];
+    const int64_t dst = sm.gdst[(uint32_t)(key >> shift) & 0xffu] + p;
     kout[dst] = key;
-    vout[dst] = tv[p];
+    vout[dst] = sm.tv[p];
   }
 }
 
-static int radix_pass(ng_ctx* c, const uint64_t* kin, const uint32_t* vin, uint64_t* kout,
-                      uint32_t* vout, int64_t n, int shift, uint32_t mask) {
-  const int nblocks = (int)((n + kRsTile - 1) / kRsTile);
-  uint32_t* hist = as<uint32_t>(c->blockhist);
-  k_rs_hist<<<nblocks, kRsThreads, 0, c->stream>>>(kin, n, shift, mask, hist, nblocks);
-  NG_TRY(scan_u32(c, hist, hist, (int64_t)256 * nblocks, nullptr, nullptr));
-  k_rs_scatter<<<nblocks, kRsThreads, 0, c->stream>>>(kin, vin, kout, vout, n, shift, mask, hist,
-                                                     nblocks);
-  c->launches += 2;
+static bool rs_large(int64_t n) { return n >= kRsLarge; }
+static int64_t rs_tiles(int64_t n) {
+  const int64_t tile = kRsThreads * (rs_large(n) ? kRsItemsLarge : kRsItemsSmall);
+  return (n + tile - 1) / tile;
+}
+
+static int64_t rs_groups(int64_t n) { return (rs_tiles(n) + kRsGroup - 1) / kRsGroup; }
+// 64-bit words of one pass's look-back state, and its parts in them
+static int64_t rs_lb_words(int64_t n) { return 256 * (rs_tiles(n) + rs_groups(n)); }
+static RsLookback rs_lookback(uint64_t* w, int64_t n) { return RsLookback{w, w + 256 * rs_tiles(n)}; }
+
+template <int ITEMS>
+static int rs_pass(ng_ctx* c, const uint64_t* kin, const uint32_t* vin, uint64_t* kout, uint32_t* vout,
+                   int64_t n, int pass, RsLookback lb, RsLookback lb_next) {
+  uint32_t* words = as<uint32_t>(c->sort_words);
+  const size_t smem = sizeof(RsSmem<ITEMS>);
+  NG_CUDA(c, cudaFuncSetAttribute(k_rs_pass<ITEMS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  k_rs_pass<ITEMS><<<(int)rs_tiles(n), kRsThreads, smem, c->stream>>>(
+      kin, vin, kout, vout, n, 8 * pass, words + 256 * pass, words + kSwTickets + pass, lb, lb_next);
+  c->launches += 1;
   NG_CUDA(c, cudaGetLastError());
   return NG_OK;
 }
+
+// ------------------------------------------------------ type-major order
+
+// tperm[j] = sorted index of the j-th body in type-major order (each species
+// in key order): a stable partition by the stored species in one launch. A
+// block ranks the bodies of its tile by ballots; one warp per species adds
+// up the counts of the tiles before (32 states per load). 1 B read and 4 B
+// written a body; as a radix pass on the keys' species bits with an index fill
+// and its own histogram and scan it read 24 B and wrote 16 B in four launches.
+constexpr int kToThreads = 512, kToItems = 8, kToTile = kToThreads * kToItems;
+constexpr int kToChunks = kToTile / 32;
+
+__global__ void __launch_bounds__(kToThreads)
+k_type_order(int64_t n, int D, const uint8_t* __restrict__ stype, uint32_t* words, uint64_t* lb,
+             uint32_t* __restrict__ tperm) {
+  __shared__ uint32_t cnt[8][kToChunks];   // per species and chunk: bodies, then output position
+  __shared__ uint32_t tile_s;
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  if (tid == 0) tile_s = atomicAdd(&words[kSwTickets + 8], 1u);
+  __syncthreads();
+  const int64_t tile = tile_s, t0 = tile * kToTile;
+  const uint32_t lt = (1u << lane) - 1u;
+  int ty[kToItems];
+  uint32_t rank[kToItems];
+#pragma unroll
+  for (int it = 0; it < kToItems; ++it) {
+    const int64_t i = t0 + it * kToThreads + tid;
+    ty[it] = i < n ? (int)stype[i] : -1;
+  }
+#pragma unroll
+  for (int it = 0; it < kToItems; ++it) {
+    const int chunk = it * (kToThreads / 32) + w;
+    rank[it] = 0;
+    for (int s = 0; s < D; ++s) {
+      const uint32_t m = __ballot_sync(0xffffffffu, ty[it] == s);
+      if (ty[it] == s) rank[it] = __popc(m & lt);
+      if (lane == 0) cnt[s][chunk] = __popc(m);
+    }
+  }
+  __syncthreads();
+  if (w < D) {
+    // warp w: species w. The chunks' exclusive scan, then the tiles before
+    constexpr int kPer = kToChunks / 32;
+    uint32_t v[kPer], sum = 0;
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) {
+      v[j] = cnt[w][lane * kPer + j];
+      sum += v[j];
+    }
+    uint32_t incl = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t x = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += x;
+    }
+    const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
+    if (lane == 0) lb_store(&lb[tile * 8 + w], (tile == 0 ? kLbPrefix : kLbAggregate) | total);
+    uint64_t before = 0;
+    int polls = 0;
+    for (int64_t t = tile - 1; t >= 0;) {
+      // lane j: the state of tile t - j; add up to the nearest prefix
+      const uint64_t s = t - lane >= 0 ? lb_load(&lb[(t - lane) * 8 + w]) : kLbPrefix;
+      const uint32_t pre = __ballot_sync(0xffffffffu, (s & kLbPrefix) != 0);
+      const uint32_t use = pre ? (pre & -pre) | ((pre & -pre) - 1u) : 0xffffffffu;
+      if (__ballot_sync(0xffffffffu, s == 0) & use) {
+        if (++polls < kLbPolls) continue;
+        before = 0;   // count the species before this tile instead
+        for (int64_t i = lane; i < t0; i += 32) before += stype[i] == w;
+        for (int o = 16; o; o >>= 1) before += __shfl_xor_sync(0xffffffffu, before, o);
+        break;
+      }
+      uint64_t add = (use >> lane & 1u) ? s & kLbCount : 0;
+      for (int o = 16; o; o >>= 1) add += __shfl_xor_sync(0xffffffffu, add, o);
+      before += add;
+      if (pre) break;
+      t -= 32;
+    }
+    if (lane == 0 && tile > 0) lb_store(&lb[tile * 8 + w], kLbPrefix | (before + total));
+    uint32_t run = (uint32_t)before + incl - sum;
+    for (int s = 0; s < w; ++s) run += words[kSwTypes + s];
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) {
+      cnt[w][lane * kPer + j] = run;
+      run += v[j];
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int it = 0; it < kToItems; ++it)
+    if (ty[it] >= 0)
+      tperm[cnt[ty[it]][it * (kToThreads / 32) + w] + rank[it]] =
+          (uint32_t)(t0 + it * kToThreads + tid);
+}
+
+static int64_t to_tiles(int64_t n) { return (n + kToTile - 1) / kToTile; }
 
 // -------------------------------------------------------------- gather
 
@@ -286,13 +544,6 @@ __global__ void k_gather_resident(int64_t n, const uint32_t* __restrict__ perm,
   }
 }
 
-__global__ void k_iota(int64_t n, uint32_t* out) {
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n;
-       k += (int64_t)gridDim.x * blockDim.x)
-    out[k] = (uint32_t)k;
-}
-
-
 int work_grid(ng_ctx* c, int64_t items, int per_sm) {
   const int64_t need = (items + 255) / 256;
   const int64_t most = (int64_t)c->nsm * per_sm;
@@ -308,13 +559,19 @@ bool box_is_pow2(double L) {
   return std::frexp(L, &e) == 0.5;
 }
 
+static KeyArgs key_args(const ng_ctx* c, int64_t n, const double* pos, const uint8_t* type) {
+  const bool pow2 = box_is_pow2(c->L);
+  return KeyArgs{n, pos, type, c->L, 1.0 / c->L, pow2, pow2 ? std::ilogb(c->L) : 0, c->p.D};
+}
+
 int reserve_sort(ng_ctx* c, int64_t n) {
-  const int nblocks = (int)((n + kRsTile - 1) / kRsTile);
   NG_TRY(ensure(c, c->keys_a, n * 8));
   NG_TRY(ensure(c, c->keys_b, n * 8));
   NG_TRY(ensure(c, c->vals_a, n * 4));
   NG_TRY(ensure(c, c->vals_b, n * 4));
-  NG_TRY(ensure(c, c->blockhist, (size_t)256 * nblocks * 4));
+  NG_TRY(ensure(c, c->sort_words, kSortWords * sizeof(uint32_t)));
+  // two radix passes' states (one cleared while the other is in use), then the type order's
+  NG_TRY(ensure(c, c->lookback, (size_t)(2 * rs_lb_words(n) + 8 * to_tiles(n)) * sizeof(uint64_t)));
   NG_TRY(ensure(c, c->spos, n * 24));
   NG_TRY(ensure(c, c->smass, n * 4));
   NG_TRY(ensure(c, c->stype, n));
@@ -328,13 +585,6 @@ int reserve_sort(ng_ctx* c, int64_t n) {
 static int sort_keys(ng_ctx* c, int64_t n, const double* pos, const uint8_t* type) {
   uint64_t *ka = as<uint64_t>(c->keys_a), *kb = as<uint64_t>(c->keys_b);
   uint32_t *va = as<uint32_t>(c->vals_a), *vb = as<uint32_t>(c->vals_b);
-  const int grid = work_grid(c, n, 8);
-  const bool pow2 = box_is_pow2(c->L);
-  stage_mark(c, NG_STAGE_KEYS);
-  k_keys<<<grid, 256, 0, c->stream>>>(n, pos, type, c->L, 1.0 / c->L, pow2,
-                                      pow2 ? std::ilogb(c->L) : 0, ka, va);
-  c->launches += 1;
-  NG_CUDA(c, cudaGetLastError());
   // 8 passes of 8 bits: the result returns to (ka, va). A tree capped at
   // level_cap reads the Morton bits of its levels only (bits >= 3 + 3 (20 -
   // cap)), so the passes below them are skipped, keeping an even number of
@@ -346,11 +596,28 @@ static int sort_keys(ng_ctx* c, int64_t n, const double* pos, const uint8_t* typ
     if ((8 - first) & 1) --first;
   }
   c->sort_passes = 8 - first;
+  c->typed = false;
+  const int64_t lbw = rs_lb_words(n), lbt = 8 * to_tiles(n);
+  uint64_t* lb = as<uint64_t>(c->lookback);
+  stage_mark(c, NG_STAGE_KEYS);
+  NG_CUDA(c, cudaMemsetAsync(c->sort_words.p, 0, kSortWords * sizeof(uint32_t), c->stream));
+  // blocks of at least 2048 bodies, at most two per SM: each adds its
+  // histograms to the global ones
+  const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)c->nsm * 2, (n + 2047) / 2048));
+  k_keys<<<grid, 512, 0, c->stream>>>(key_args(c, n, pos, type), first, ka, as<uint32_t>(c->sort_words),
+                                      lb, lbw, lb + 2 * lbw, lbt);
+  c->launches += 1;
+  NG_CUDA(c, cudaGetLastError());
   stage_mark(c, NG_STAGE_RADIX);
   for (int pass = first; pass < 8; ++pass) {
     const bool even = ((pass - first) & 1) == 0;
-    NG_TRY(radix_pass(c, even ? ka : kb, even ? va : vb, even ? kb : ka, even ? vb : va, n,
-                      8 * pass, 0xffu));
+    const uint64_t* kin = even ? ka : kb;
+    const uint32_t* vin = pass == first ? nullptr : even ? va : vb;   // first pass: the index
+    uint64_t* kout = even ? kb : ka;
+    const RsLookback lin = rs_lookback(even ? lb : lb + lbw, n), lnext = rs_lookback(even ? lb + lbw : lb, n);
+    uint32_t* vout = even ? vb : va;
+    if (rs_large(n)) NG_TRY(rs_pass<kRsItemsLarge>(c, kin, vin, kout, vout, n, pass, lin, lnext));
+    else NG_TRY(rs_pass<kRsItemsSmall>(c, kin, vin, kout, vout, n, pass, lin, lnext));
   }
   return NG_OK;
 }
@@ -383,19 +650,21 @@ int sort_bodies(ng_ctx* c, int64_t n, const double* pos, const uint8_t* type, co
   return NG_OK;
 }
 
-// Type-major order: one stable radix pass on the species bits of the sorted
-// keys. tperm[j] = sorted index of the j-th body in type-major order.
 int type_order(ng_ctx* c) {
   const int64_t n = c->n;
-  const int grid = work_grid(c, n, 8);
-  uint64_t *ka = as<uint64_t>(c->keys_a), *kb = as<uint64_t>(c->keys_b);
-  uint32_t* vb = as<uint32_t>(c->vals_b);
   stage_mark(c, NG_STAGE_TYPE_ORDER);
-  k_iota<<<grid, 256, 0, c->stream>>>(n, vb);
+  // a tree rebuilt on the same sorted bodies keeps their order (the launch
+  // takes its tickets and look-back state as the sort's key kernel left them)
+  if (c->typed) return NG_OK;
+  c->typed = true;
+  k_type_order<<<(int)to_tiles(n), kToThreads, 0, c->stream>>>(
+      n, c->p.D, as<uint8_t>(c->stype), as<uint32_t>(c->sort_words),
+      as<uint64_t>(c->lookback) + 2 * rs_lb_words(n), as<uint32_t>(c->tperm));
   c->launches += 1;
   NG_CUDA(c, cudaGetLastError());
-  NG_TRY(radix_pass(c, ka, vb, kb, as<uint32_t>(c->tperm), n, 0, 7u));
   return NG_OK;
 }
+
+const uint32_t* type_counts(const ng_ctx* c) { return as<uint32_t>(c->sort_words) + kSwTypes; }
 
 }  // namespace ng
