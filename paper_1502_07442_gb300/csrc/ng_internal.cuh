@@ -19,19 +19,17 @@ namespace ng {
 constexpr int kMaxD = NG_MAX_SPECIES;
 constexpr int kMaxLevel = 20;           // 20 Morton bits per axis
 constexpr int kCapturedDepthMargin = 2;  // captured steps build this far below the depth seen
-// Trees of at most kClusterMaxBodies bodies are built, and their monopoles
-// reduced, by one launch each: a cluster of kClusterBlocks blocks that runs
-// every level with the hardware cluster barrier between levels (larger trees:
-// one launch per level and phase, over the whole GPU).
+// The top levels of a tree's monopoles are reduced by one cluster of
+// kClusterBlocks blocks with the hardware cluster barrier between levels.
 constexpr int kClusterBlocks = 8;
-constexpr int64_t kClusterMaxBodies = 32768;
+constexpr int kMonoWords = 1 + kMaxLevel + 1;   // counters of the monopole stage
 // Monopoles of trees of kBinnedMonoBodies bodies or more are reduced in an
 // order binned by the work of a node: leaves by body count (0..64, one more
 // bin for the larger leaves of a tree stopped at a level cap), internal nodes
 // by level and child count.
 constexpr int kLeafBins = 66;
 constexpr int kMonoBins = kLeafBins + (kMaxLevel + 1) * 8;
-constexpr int64_t kBinnedMonoBodies = 1 << 20;   // smaller trees: level order
+constexpr int64_t kBinnedMonoBodies = 1 << 20;
 constexpr int kWarp = 32;
 
 // Status words in device memory (ctx->status).
@@ -287,7 +285,8 @@ struct ng_ctx {
   int64_t ngroups = 0, ngroups_n = -1;   // walk groups of the last checked build, for n = ngroups_n
   ng::DevBuf n_level, n_prefix, n_first, n_count, n_child, n_nchild, n_tmp;
   ng::DevBuf n_m64, n_cnt, n_geo, n_com, n_link, n_mono;
-  ng::DevBuf mono_bins;   // uint32[3 kMonoBins + 1]: nodes, cursors and starts per monopole bin
+  ng::DevBuf mono_words;   // uint32[kMonoWords + 3 kMonoBins + 1]: counters and bins of the monopole stage
+  ng::DevBuf tree_cnt;    // uint32[levels][tiles]: node counts of the tree build
   ng::DevBuf groups;
   ng::DevBuf gsize, grank;          // group size at its first body, rank of each group start
   ng::DevBuf status;     // uint32[ST_COUNT]
@@ -396,6 +395,7 @@ int resident_load(ng_ctx* c, int64_t n, const double* pos, const float* vel, con
 int resident_store(ng_ctx* c, int64_t n, double* pos, float* vel, float* acc);
 int resident_step_once(ng_ctx* c, int64_t n, double dt, bool checked);
 int build_octree(ng_ctx* c);                  // needs sorted bodies
+size_t tree_scratch_bytes(int64_t n);         // tree_cnt for n bodies
 int reduce_monopoles(ng_ctx* c);              // needs octree
 int build_groups(ng_ctx* c);                  // needs octree
 int launch_walk(ng_ctx* c, float* acc, bool accumulate, bool count);
@@ -503,8 +503,6 @@ __device__ __forceinline__ uint32_t block_inclusive_scan(uint32_t v, uint32_t* w
 // Blocks of 256 threads for a grid-stride kernel over `items` items: enough
 // to cover them, at most per_sm blocks per SM, at least one.
 int work_grid(ng_ctx* c, int64_t items, int per_sm);
-// Upper bound on the nodes of tree level l: 8^l and the body count.
-int64_t level_bound(int l, int64_t n);
 
 // Pipeline pieces shared by the single-simulation calls and the batch
 // runtime (ng_api.cu).

@@ -550,10 +550,6 @@ int work_grid(ng_ctx* c, int64_t items, int per_sm) {
   return (int)std::max<int64_t>(1, std::min(need, most));
 }
 
-int64_t level_bound(int l, int64_t n) {
-  return l >= 21 ? n : std::min<int64_t>(n, (int64_t)1 << (3 * l));
-}
-
 bool box_is_pow2(double L) {
   int e = 0;
   return std::frexp(L, &e) == 0.5;

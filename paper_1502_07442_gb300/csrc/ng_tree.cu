@@ -1,16 +1,16 @@
-// Tree stage (Sec. 2.2): canonical Morton-prefix octree built breadth-first
-// one level per launch (node ranges stay on the device, no host round trip),
-// per-node per-species monopoles reduced in double precision (one thread per
-// node: every leaf in one launch, then the internal nodes level by level,
-// bottom-up), and the walk groups.
+// Tree stage (Sec. 2.2): canonical Morton-prefix octree, all levels at once
+// from the sorted keys (node ranges stay on the device, no host round trip),
+// per-node per-species monopoles reduced in double precision (every leaf in
+// one launch, then the internal nodes by subtrees, bottom-up), and the walk
+// groups.
 //
 // Canonical tree: nodes are the non-empty Morton cells reachable from the
 // root; a cell is a leaf iff it holds <= leaf_size bodies or is at level 20;
 // children are the non-empty octants in octant order; nodes are numbered
 // level by level, and within a level in key order. Builds inside captured
 // steps stop at a level cap two below the deepest level seen by the step
-// before the capture (fewer launches per level-free tail); a cell at the cap
-// is then a leaf whatever it holds, and SF_DEPTH says so.
+// before the capture (their sort then orders fewer key bits); a cell at the
+// cap is then a leaf whatever it holds, and SF_DEPTH says so.
 #include <cooperative_groups.h>
 
 #include "ng_internal.cuh"
@@ -26,301 +26,269 @@ __device__ __forceinline__ Levels levels_of(uint32_t* status) {
   return Levels{status + ST_LEVELS, status + ST_LEVELS + kMaxLevel + 2};
 }
 
-__global__ void k_tree_init(uint32_t* status, int64_t n, uint8_t* level, uint64_t* prefix,
-                            uint32_t* first, uint32_t* count) {
-  if (threadIdx.x == 0) {
-    Levels lv = levels_of(status);
-    for (int l = 0; l <= kMaxLevel + 1; ++l) lv.start[l] = 1;
-    for (int l = 0; l <= kMaxLevel; ++l) lv.count[l] = 0;
-    lv.start[0] = 0;
-    lv.start[1] = 1;
-    lv.count[0] = 1;
-    status[ST_NODES_NEEDED] = 1;
-    status[ST_NGROUPS] = 0;
-    level[0] = 0;
-    prefix[0] = 0;
-    first[0] = 0;
-    count[0] = (uint32_t)n;
-  }
+// The tree from the sorted keys in one pass over the bodies, all levels at
+// once. With common(a, b) the number of octal digits two Morton keys share:
+//   delta(i)  = common(key[i - 1], key[i]) (-1 for the first body): body i is
+//               the first body of its cells of level delta(i) + 1 and deeper;
+//   lambda(i) = 1 + the deepest level whose cell around i holds more than
+//               leaf_size bodies (0 if none does), at most lmax. That level is
+//               the largest common(key[j], key[j + leaf_size]) over the windows
+//               j in [i - leaf_size, i], which are the runs of leaf_size + 1
+//               consecutive bodies around i.
+// A cell is a node iff its parent holds more than leaf_size bodies, so the
+// nodes that start at body i are exactly those of levels delta(i) + 1 ..
+// lambda(i); the last of them is a leaf, and the first child of each other
+// one is the next. Nodes are numbered level by level, in key order within a
+// level: the number of a node is the exclusive scan of the per-level start
+// flags laid out level-major, which k_tree_count sums per tile, one device
+// scan turns into offsets, and k_tree_emit completes inside the tile.
+//
+// Bound by reading the keys twice (8 B a body each) and by the launches: four
+// or five for any size, where one launch triple per level took 81 (131k
+// bodies: about 340 -> 33 us of kernels; 3 M: 560 -> 95 us), and a cluster of
+// eight blocks walking the levels of a small tree 92 us at 4096 bodies (now 26).
+constexpr int kTreeThreads = 256;
+constexpr int kTreeItems = 4;
+constexpr int kTreeTile = kTreeThreads * kTreeItems;   // bodies per block
+constexpr int kTreeChunks = kTreeTile / 32;            // warp-wide runs of bodies per tile
+constexpr int kMaxLeaf = 64;
+static_assert(kTreeChunks == 32, "the chunk scan takes one chunk per lane");
+
+// Octal digits that the Morton parts of two keys share (20: the same cell).
+__device__ __forceinline__ int common_levels(uint64_t a, uint64_t b) {
+  const uint64_t x = (a ^ b) >> 3;
+  return x ? 19 - (63 - __clzll((long long)x)) / 3 : kMaxLevel;
 }
 
-// First index in [lo, hi) whose child octant at shift is >= oct.
-__device__ __forceinline__ uint32_t octant_bound(const uint64_t* __restrict__ keys, uint32_t lo,
-                                                 uint32_t hi, int shift, uint32_t oct) {
-  while (lo < hi) {
-    const uint32_t mid = lo + ((hi - lo) >> 1);
-    const uint32_t o = (uint32_t)((keys[mid] >> (3 + shift)) & 7ull);
-    if (o < oct) lo = mid + 1; else hi = mid;
-  }
-  return lo;
-}
-
-// Both kernels give each node of level lvl a team of 8 lanes: lane o finds
-// where octant o of the node's (sorted) body range starts, all 8 binary
-// searches at once, so a level with few large nodes (the top of the tree)
-// waits for one search, not eight in a row. Teams of a warp loop together
-// (every lane runs the same iterations, so the team shuffles are safe).
-struct OctTeam {
-  uint32_t start, end;   // octant `sub` of the node: bodies [start, end)
-  bool nonempty;
-  uint32_t bits;         // non-empty octants of the node, bit o for octant o
+struct TreeTile {
+  uint64_t key[kTreeTile + 2 * kMaxLeaf];
+  int8_t w[2][kTreeTile + kMaxLeaf];
 };
 
-__device__ __forceinline__ OctTeam octant_team(const uint64_t* __restrict__ keys, bool split,
-                                               uint32_t f, uint32_t c, int shift, int sub,
-                                               int lane) {
-  OctTeam t;
-  t.start = (split && sub > 0) ? octant_bound(keys, f, f + c, shift, (uint32_t)sub) : f;
-  const uint32_t nxt = __shfl_down_sync(0xffffffffu, t.start, 1, 8);
-  t.end = sub == 7 ? f + c : nxt;
-  t.nonempty = split && t.end > t.start;
-  const uint32_t m = __ballot_sync(0xffffffffu, t.nonempty);
-  t.bits = (m >> (lane & 24)) & 0xffu;
-  return t;
-}
-
-// Count phase of level lvl: each team of 8 lanes (team of teams, warps'
-// teams looping together) takes nodes of the level and records their child
-// counts in nchild and tmp. lmax: the deepest level the build emits
-// (kMaxLevel unless capped); nodes of level lmax are leaves, and one above
-// the leaf size raises SF_DEPTH.
-__device__ __forceinline__ void tree_count_nodes(int lvl, int lmax, uint32_t* status, int64_t cap,
-                                                 int leaf_size, const uint64_t* __restrict__ keys,
-                                                 const uint32_t* __restrict__ first,
-                                                 const uint32_t* __restrict__ count,
-                                                 uint8_t* nchild, uint32_t* child, uint32_t* tmp,
-                                                 int64_t team, int64_t teams) {
-  Levels lv = levels_of(status);
-  const uint32_t s = lv.start[lvl];
-  uint32_t e = lv.start[lvl + 1];
-  if (e > cap) e = (uint32_t)cap;
-  const int nodes = e > s ? (int)(e - s) : 0;
-  const int shift = 3 * (kMaxLevel - (lvl + 1));
-  const int lane = threadIdx.x & 31, sub = lane & 7;
-  for (int64_t base = team & ~(int64_t)3; base < nodes; base += teams) {
-    const int64_t j = base + (team & 3);
-    const bool valid = j < nodes;
-    const uint32_t k = s + (uint32_t)j;
-    const uint32_t f = valid ? first[k] : 0u, c = valid ? count[k] : 0u;
-    const bool split = valid && (int)c > leaf_size && lvl < lmax;
-    const OctTeam t = octant_team(keys, split, f, c, shift, sub, lane);
-    if (valid && sub == 0) {
-      const uint32_t nch = (uint32_t)__popc(t.bits);
-      nchild[k] = (uint8_t)nch;
-      tmp[k - s] = nch;
-      if (lvl == lmax) {
-        child[k] = 0xffffffffu;   // no emit follows the last level
-        if ((int)c > leaf_size && lmax < kMaxLevel) atomicOr(&status[ST_FLAGS], (uint32_t)SF_DEPTH);
-      }
+// The tile's keys into shared memory and delta, lambda of the thread's bodies
+// (body it: t0 + it * kTreeThreads + threadIdx.x). Returns the keys' offset:
+// body i is sm.key[i - (t0 - leaf)].
+__device__ __forceinline__ void tree_tile(TreeTile& sm, const uint64_t* __restrict__ keys, int64_t n,
+                                          int64_t t0, int leaf, int lmax, int delta[kTreeItems],
+                                          int lambda[kTreeItems]) {
+  const int64_t base = t0 - leaf;
+  for (int j = threadIdx.x; j < kTreeTile + 2 * leaf; j += kTreeThreads) {
+    const int64_t i = base + j;
+    sm.key[j] = i >= 0 && i < n ? keys[i] : 0ull;
+  }
+  __syncthreads();
+  const int nw = kTreeTile + leaf;
+  for (int j = threadIdx.x; j < nw; j += kTreeThreads) {
+    const int64_t i = base + j;
+    sm.w[0][j] = i >= 0 && i + leaf < n ? (int8_t)common_levels(sm.key[j], sm.key[j + leaf])
+                                        : (int8_t)-1;
+  }
+  // maximum over windows of `span` entries, doubled while it fits leaf + 1
+  int cur = 0, span = 1;
+  for (; 2 * span <= leaf + 1; span *= 2) {
+    __syncthreads();
+    for (int j = threadIdx.x; j < nw; j += kTreeThreads) {
+      const int8_t v = sm.w[cur][j];
+      sm.w[cur ^ 1][j] = j + span < nw ? max(v, sm.w[cur][j + span]) : v;
+    }
+    cur ^= 1;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int it = 0; it < kTreeItems; ++it) {
+    const int ii = it * kTreeThreads + threadIdx.x;
+    const int64_t i = t0 + ii;
+    delta[it] = kMaxLevel;
+    lambda[it] = -1;   // no node starts here
+    if (i < n) {
+      delta[it] = i == 0 ? -1 : common_levels(sm.key[ii + leaf - 1], sm.key[ii + leaf]);
+      lambda[it] = min(lmax, 1 + max(sm.w[cur][ii], sm.w[cur][ii + leaf + 1 - span]));
     }
   }
 }
 
-// The start of level lvl + 2 from the child total of level lvl (one thread);
-// a node count beyond the capacity raises SF_NODE_OVERFLOW.
-__device__ __forceinline__ void tree_level_close(int lvl, uint32_t* status, int64_t cap) {
-  Levels lv = levels_of(status);
-  const uint64_t end = (uint64_t)lv.start[lvl + 1] + lv.count[lvl + 1];
-  lv.start[lvl + 2] = (uint32_t)(end < 0xffffffffull ? end : 0xffffffffull);
-  // only levels up to the first overflow are counted correctly: the node
-  // estimate is taken there and never from the truncated levels below it
-  if (!(status[ST_FLAGS] & SF_NODE_OVERFLOW)) {
-    status[ST_NODES_NEEDED] = (uint32_t)(end < 0xffffffffull ? end : 0xffffffffull);
-    if (end > (uint64_t)cap) status[ST_FLAGS] |= (uint32_t)SF_NODE_OVERFLOW;
-  }
-}
-
-// Emit phase of level lvl: the children of each split node, numbered from the
-// level's end (next0) by the exclusive scan of the child counts (off).
-__device__ __forceinline__ void tree_emit_nodes(int lvl, uint32_t next0, uint32_t* status, int64_t cap,
-                                                const uint64_t* __restrict__ keys, uint8_t* level,
-                                                uint64_t* prefix, uint32_t* first, uint32_t* count,
-                                                const uint8_t* __restrict__ nchild, uint32_t* child,
-                                                const uint32_t* __restrict__ off, int64_t team,
-                                                int64_t teams) {
-  Levels lv = levels_of(status);
-  const uint32_t s = lv.start[lvl];
-  uint32_t e = next0;
-  if (e > cap) e = (uint32_t)cap;
-  const int nodes = e > s ? (int)(e - s) : 0;
-  const int shift = 3 * (kMaxLevel - (lvl + 1));
-  const int lane = threadIdx.x & 31, sub = lane & 7;
-  for (int64_t base = team & ~(int64_t)3; base < nodes; base += teams) {
-    const int64_t j = base + (team & 3);
-    const bool valid = j < nodes;
-    const uint32_t k = s + (uint32_t)j;
-    const uint32_t nch = valid ? nchild[k] : 0u;
-    const bool split = nch > 0;
-    const uint32_t f = split ? first[k] : 0u, c = split ? count[k] : 0u;
-    const OctTeam t = octant_team(keys, split, f, c, shift, sub, lane);
-    if (!split) {
-      if (valid && sub == 0) child[k] = 0xffffffffu;
-      continue;
-    }
-    const uint32_t c0 = next0 + off[k - s];
-    if (sub == 0) child[k] = c0;
-    if (t.nonempty) {
-      const uint64_t id = (uint64_t)c0 + (uint32_t)__popc(t.bits & ((1u << sub) - 1u));
-      if (id < (uint64_t)cap) {
-        level[id] = (uint8_t)(lvl + 1);
-        prefix[id] = (prefix[k] << 3) | (uint64_t)sub;
-        first[id] = t.start;
-        count[id] = t.end - t.start;
-      }
+// cnt[l * gridDim.x + block]: nodes of level l that start in the block's tile.
+__global__ void __launch_bounds__(kTreeThreads)
+k_tree_count(const uint64_t* __restrict__ keys, int64_t n, int leaf, int lmax,
+             uint32_t* __restrict__ cnt) {
+  __shared__ TreeTile sm;
+  __shared__ uint32_t total[kMaxLevel + 1];
+  if (threadIdx.x <= kMaxLevel) total[threadIdx.x] = 0;
+  int delta[kTreeItems], lambda[kTreeItems];
+  tree_tile(sm, keys, n, (int64_t)blockIdx.x * kTreeTile, leaf, lmax, delta, lambda);
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int it = 0; it < kTreeItems; ++it) {
+    const bool has = lambda[it] > delta[it];
+    const int lo = __reduce_min_sync(0xffffffffu, has ? delta[it] + 1 : kMaxLevel + 1);
+    const int hi = __reduce_max_sync(0xffffffffu, has ? lambda[it] : -1);
+    for (int l = lo; l <= hi; ++l) {
+      const uint32_t m = __ballot_sync(0xffffffffu, has && delta[it] < l && l <= lambda[it]);
+      if (lane == 0 && m) atomicAdd(&total[l], (uint32_t)__popc(m));
     }
   }
+  __syncthreads();
+  if (threadIdx.x <= lmax) cnt[(size_t)threadIdx.x * gridDim.x + blockIdx.x] = total[threadIdx.x];
 }
 
-__global__ void k_tree_count(int lvl, int lmax, uint32_t* status, int64_t cap, int leaf_size,
-                             const uint64_t* __restrict__ keys, const uint32_t* __restrict__ first,
-                             const uint32_t* __restrict__ count, uint8_t* nchild,
-                             uint32_t* child, uint32_t* tmp) {
-  const int64_t team = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 3;
-  const int64_t teams = ((int64_t)gridDim.x * blockDim.x) >> 3;   // a multiple of 4
-  tree_count_nodes(lvl, lmax, status, cap, leaf_size, keys, first, count, nchild, child, tmp, team,
-                   teams);
-}
-
-__global__ void k_tree_emit(int lvl, uint32_t* status, int64_t cap,
-                            const uint64_t* __restrict__ keys, uint8_t* level, uint64_t* prefix,
-                            uint32_t* first, uint32_t* count, const uint8_t* __restrict__ nchild,
-                            uint32_t* child, const uint32_t* __restrict__ off) {
-  const uint32_t next0 = levels_of(status).start[lvl + 1];
-  if (blockIdx.x == 0 && threadIdx.x == 0) tree_level_close(lvl, status, cap);
-  const int64_t team = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 3;
-  const int64_t teams = ((int64_t)gridDim.x * blockDim.x) >> 3;
-  tree_emit_nodes(lvl, next0, status, cap, keys, level, prefix, first, count, nchild, child, off,
-                  team, teams);
-}
-
-// The whole build of a small tree in one launch: one cluster of
-// kClusterBlocks blocks (co-scheduled; its barrier is the hardware cluster
-// barrier, so no block waits on a flag) runs every level's count, scan and
-// emit phases, each the same code as the per-level kernels, with a cluster
-// barrier between phases. The child-count scan of a level: each block sums
-// its contiguous chunk, the sums go to every block's shared memory, and
-// each block scans its chunk from the sum of the chunks before it.
-__global__ void __cluster_dims__(kClusterBlocks, 1, 1) __launch_bounds__(1024, 1)
-k_tree_cluster(int lmax, uint32_t* status, int64_t n, int64_t cap, int leaf_size,
-               const uint64_t* __restrict__ keys, uint8_t* level, uint64_t* prefix, uint32_t* first,
-               uint32_t* count, uint8_t* nchild, uint32_t* child, uint32_t* tmp) {
-  namespace cg = cooperative_groups;
-  cg::cluster_group cluster = cg::this_cluster();
-  __shared__ uint32_t sums[kClusterBlocks];
-  __shared__ uint32_t warp_tot[32];
-  __shared__ uint32_t tile_total;
-  const int tid = threadIdx.x, nb = (int)gridDim.x, b = (int)blockIdx.x;
-  Levels lv = levels_of(status);
-  if (b == 0 && tid == 0) {
-    for (int l = 0; l <= kMaxLevel + 1; ++l) lv.start[l] = 1;
-    for (int l = 0; l <= kMaxLevel; ++l) lv.count[l] = 0;
-    lv.start[0] = 0;
-    lv.start[1] = 1;
-    lv.count[0] = 1;
-    status[ST_NODES_NEEDED] = 1;
-    status[ST_NGROUPS] = 0;
-    level[0] = 0;
-    prefix[0] = 0;
-    first[0] = 0;
-    count[0] = (uint32_t)n;
-  }
-  cluster.sync();
-  const int64_t team = ((int64_t)b * blockDim.x + tid) >> 3;
-  const int64_t teams = ((int64_t)nb * blockDim.x) >> 3;
-  for (int l = 0; l <= lmax; ++l) {
-    tree_count_nodes(l, lmax, status, cap, leaf_size, keys, first, count, nchild, child, tmp, team,
-                     teams);
-    cluster.sync();
-    if (l == lmax) break;
-    // exclusive scan of the level's child counts (tmp, in place)
-    const uint32_t s = lv.start[l];
-    uint32_t e = lv.start[l + 1];
-    if (e > cap) e = (uint32_t)cap;
-    const int nodes = e > s ? (int)(e - s) : 0;
-    const int chunk = (nodes + nb - 1) / nb;
-    const int c0 = min(nodes, b * chunk), c1 = min(nodes, c0 + chunk);
-    uint32_t part = 0;
-    for (int i = c0 + tid; i < c1; i += blockDim.x) part += tmp[i];
-    block_inclusive_scan<1024>(part, warp_tot, &tile_total);
-    if (tid < nb) *cluster.map_shared_rank(&sums[b], tid) = tile_total;
-    cluster.sync();
-    uint32_t carry = 0;
-    for (int r = 0; r < b; ++r) carry += sums[r];
-    for (int base = c0; base < c1; base += blockDim.x) {
-      const int i = base + tid;
-      const uint32_t v = i < c1 ? tmp[i] : 0u;
-      const uint32_t inc = block_inclusive_scan<1024>(v, warp_tot, &tile_total);
-      if (i < c1) tmp[i] = carry + inc - v;
-      __syncthreads();
-      carry += tile_total;
-      __syncthreads();
-    }
-    if (b == nb - 1 && tid == 0) lv.count[l + 1] = carry;
-    cluster.sync();
-    const uint32_t next0 = lv.start[l + 1];
-    if (b == 0 && tid == 0) tree_level_close(l, status, cap);
-    tree_emit_nodes(l, next0, status, cap, keys, level, prefix, first, count, nchild, child, tmp,
-                    team, teams);
-    cluster.sync();
-  }
-  if (lmax < kMaxLevel && b == 0 && tid == 0) {
-    const uint32_t end = lv.start[lmax + 1];
-    for (int l = lmax + 2; l <= kMaxLevel + 1; ++l) lv.start[l] = end;
-  }
-}
-
-// A build capped at level lmax < kMaxLevel: the levels below it are empty
-// (their starts all equal the end of level lmax), as the node total and the
-// per-level kernels that follow expect.
-__global__ void k_tree_close(uint32_t* status, int lmax) {
-  if (threadIdx.x == 0) {
+// Level, prefix, first body and first child of every node (child: for a leaf
+// the number the next child of its level would have, so that the child
+// counts are differences of neighbours). off: the scanned cnt;
+// status[ST_NODES_NEEDED] holds the node total. Block 0 writes the level
+// table and raises SF_NODE_OVERFLOW if the nodes exceed the capacity.
+__global__ void __launch_bounds__(kTreeThreads)
+k_tree_emit(const uint64_t* __restrict__ keys, int64_t n, int leaf, int lmax,
+            const uint32_t* __restrict__ off, uint32_t* status, int64_t cap,
+            uint8_t* __restrict__ level, uint64_t* __restrict__ prefix,
+            uint32_t* __restrict__ first, uint32_t* __restrict__ child, uint32_t* words) {
+  __shared__ TreeTile sm;
+  __shared__ uint32_t pos[kTreeChunks][kMaxLevel + 2];   // per chunk and level: count, then number
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const uint32_t total = status[ST_NODES_NEEDED];
+  if (blockIdx.x == 0 && tid < kMonoWords) words[tid] = 0;   // the monopoles' counters
+  if (blockIdx.x == 0 && tid <= kMaxLevel + 1) {
     Levels lv = levels_of(status);
-    const uint32_t end = lv.start[lmax + 1];
-    for (int l = lmax + 2; l <= kMaxLevel + 1; ++l) lv.start[l] = end;
+    const uint32_t s = tid <= lmax ? off[(size_t)tid * gridDim.x] : total;
+    const uint32_t e = tid < lmax ? off[(size_t)(tid + 1) * gridDim.x] : total;
+    lv.start[tid] = s;
+    if (tid <= kMaxLevel) lv.count[tid] = e - s;
+    if (tid == 0) {
+      status[ST_NGROUPS] = 0;
+      if ((int64_t)total > cap) atomicOr(&status[ST_FLAGS], (uint32_t)SF_NODE_OVERFLOW);
+    }
   }
+  for (int j = tid; j < kTreeChunks * (kMaxLevel + 2); j += kTreeThreads) (&pos[0][0])[j] = 0;
+  const int64_t t0 = (int64_t)blockIdx.x * kTreeTile;
+  int delta[kTreeItems], lambda[kTreeItems], lo[kTreeItems], hi[kTreeItems];
+  tree_tile(sm, keys, n, t0, leaf, lmax, delta, lambda);
+#pragma unroll
+  for (int it = 0; it < kTreeItems; ++it) {
+    const bool has = lambda[it] > delta[it];
+    lo[it] = __reduce_min_sync(0xffffffffu, has ? delta[it] + 1 : kMaxLevel + 1);
+    hi[it] = __reduce_max_sync(0xffffffffu, has ? lambda[it] : -1);
+    for (int l = lo[it]; l <= hi[it]; ++l) {
+      const uint32_t m = __ballot_sync(0xffffffffu, has && delta[it] < l && l <= lambda[it]);
+      if (lane == 0) pos[it * (kTreeThreads / 32) + warp][l] = (uint32_t)__popc(m);
+    }
+  }
+  __syncthreads();
+  for (int l = warp; l <= lmax; l += kTreeThreads / 32) {
+    const uint32_t v = pos[lane][l];
+    uint32_t inc = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t t = __shfl_up_sync(0xffffffffu, inc, o);
+      if (lane >= o) inc += t;
+    }
+    pos[lane][l] = off[(size_t)l * gridDim.x + blockIdx.x] + inc - v;
+  }
+  __syncthreads();
+  const uint32_t below = (1u << lane) - 1u;
+#pragma unroll
+  for (int it = 0; it < kTreeItems; ++it) {
+    const int chunk = it * (kTreeThreads / 32) + warp;
+    const int ii = it * kTreeThreads + tid;
+    const bool has = lambda[it] > delta[it];
+    const uint64_t key = sm.key[ii + leaf];
+    bool prev = false;
+    uint32_t id = 0;
+    for (int l = lo[it]; l <= hi[it] + 1; ++l) {
+      const bool starts = has && delta[it] < l && l <= lambda[it];
+      const uint32_t m = __ballot_sync(0xffffffffu, starts);
+      const uint32_t r = l <= lmax ? pos[chunk][l] + (uint32_t)__popc(m & below) : total;
+      if (prev) child[id] = r;
+      prev = starts && (int64_t)r < cap;
+      if (prev) {
+        id = r;
+        level[r] = (uint8_t)l;
+        prefix[r] = key >> (3 + 3 * (kMaxLevel - l));
+        first[r] = (uint32_t)(t0 + ii);
+      }
+    }
+  }
+}
+
+// Body and child counts of every node, each leaf's number at its bodies and
+// each child's parent (in its link, for the monopoles' lists). Children are numbered in node order,
+// so a node's child count is the difference of its first child and the next
+// node's. The next node of the level ends a node with the same parent; the
+// last child of a parent finds its end in the keys (doubling steps, then
+// bisection). Nodes of level lmax above the leaf size raise SF_DEPTH (lmax
+// below kMaxLevel).
+__global__ void k_tree_nodes(uint32_t* status, int64_t cap, const uint64_t* __restrict__ keys,
+                             int64_t n, int leaf, int lmax, const uint8_t* __restrict__ level,
+                             const uint64_t* __restrict__ prefix,
+                             const uint32_t* __restrict__ first, const uint32_t* __restrict__ child,
+                             uint32_t* __restrict__ count, uint8_t* __restrict__ nchild,
+                             uint32_t* __restrict__ bleaf, int4* __restrict__ link) {
+  if (status[ST_FLAGS] & SF_NODE_OVERFLOW) return;
+  Levels lv = levels_of(status);
+  const uint32_t total = lv.start[kMaxLevel + 1];
+  for (uint32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < total; k += gridDim.x * blockDim.x) {
+    const int l = level[k];
+    const bool more = k + 1 < lv.start[l + 1];
+    const uint64_t pre = prefix[k];
+    const uint32_t f = first[k];
+    uint32_t end = more ? first[k + 1] : (uint32_t)n;
+    if (l > 0 && !(more && (prefix[k + 1] >> 3) == (pre >> 3))) {
+      const int shift = 3 + 3 * (kMaxLevel - l);
+      uint32_t lo = f, step = 1;   // keys[lo] is in the cell
+      while (step < end - lo && (keys[lo + step] >> shift) == pre) {
+        lo += step;
+        step <<= 1;
+      }
+      uint32_t hi = step < end - lo ? lo + step : end;   // keys[hi] is not (or hi is the bound)
+      while (hi - lo > 1) {
+        const uint32_t mid = lo + ((hi - lo) >> 1);
+        if ((keys[mid] >> shift) == pre) lo = mid; else hi = mid;
+      }
+      end = hi;
+    }
+    count[k] = end - f;
+    const uint32_t nch = l < lmax ? (more ? child[k + 1] : lv.start[l + 2]) - child[k] : 0u;
+    nchild[k] = (uint8_t)nch;
+    if (nch == 0) {
+      for (uint32_t b = f; b < end; ++b) bleaf[b] = k;
+    } else {
+      const uint32_t c0 = child[k];
+      for (uint32_t j = 0; j < nch; ++j) link[c0 + j].w = (int)k;   // until its monopoles are formed
+    }
+    if (l == lmax && lmax < kMaxLevel && end - f > (uint32_t)leaf)
+      atomicOr(&status[ST_FLAGS], (uint32_t)SF_DEPTH);
+  }
+}
+
+// Largest subtree of the monopole stage: about n / 2048 bodies, 256 or more.
+constexpr uint32_t kMaxSub = 512;
+static uint32_t mono_sub(int64_t n) { return n <= 256 * 2048 ? 256 : kMaxSub; }
+
+size_t tree_scratch_bytes(int64_t n) {
+  // node counts per level and tile, later the top nodes of the monopoles
+  const int64_t per = std::max<int64_t>((n + kTreeTile - 1) / kTreeTile, n / mono_sub(n) + 1);
+  return (size_t)per * (kMaxLevel + 1) * sizeof(uint32_t);
 }
 
 int build_octree(ng_ctx* c) {
   const int64_t n = c->n;
   const int64_t cap = c->cap_nodes;
   uint32_t* st = as<uint32_t>(c->status);
-  uint8_t* level = as<uint8_t>(c->n_level);
-  uint64_t* prefix = as<uint64_t>(c->n_prefix);
-  uint32_t* first = as<uint32_t>(c->n_first);
-  uint32_t* count = as<uint32_t>(c->n_count);
-  uint8_t* nchild = as<uint8_t>(c->n_nchild);
-  uint32_t* child = as<uint32_t>(c->n_child);
-  uint32_t* tmp = as<uint32_t>(c->n_tmp);
   const uint64_t* keys = as<uint64_t>(c->keys_a);
+  uint32_t* cnt = as<uint32_t>(c->tree_cnt);
   const int leaf = c->p.leaf_size;
   const int lmax = std::min(std::max(c->level_cap, 0), kMaxLevel);
+  const int tiles = (int)((n + kTreeTile - 1) / kTreeTile);
   stage_mark(c, NG_STAGE_OCTREE);
-  if (n <= kClusterMaxBodies) {
-    k_tree_cluster<<<kClusterBlocks, 1024, 0, c->stream>>>(lmax, st, n, cap, leaf, keys, level,
-                                                          prefix, first, count, nchild, child, tmp);
-    c->launches += 1;
-    NG_CUDA(c, cudaGetLastError());
-    return NG_OK;
-  }
-  k_tree_init<<<1, 32, 0, c->stream>>>(st, n, level, prefix, first, count);
-  c->launches += 1 + (lmax + 1) + lmax;   // init, counts, emits (scans count themselves)
-  for (int l = 0; l <= lmax; ++l) {
-    // grids sized by the most nodes level l can hold (kernels stride over the actual count)
-    const int64_t bound = std::min<int64_t>(cap, level_bound(l, c->n));
-    const int grid = work_grid(c, 8 * bound, 4);   // 8 lanes per node
-    k_tree_count<<<grid, 256, 0, c->stream>>>(l, lmax, st, cap, leaf, keys, first, count, nchild,
-                                              child, tmp);
-    if (l == lmax) break;
-    // children per level: exclusive scan of the per-node child counts
-    uint32_t* lvcount = st + ST_LEVELS + kMaxLevel + 2;
-    NG_TRY(scan_u32(c, tmp, tmp, bound, lvcount + l, lvcount + l + 1));
-    k_tree_emit<<<grid, 256, 0, c->stream>>>(l, st, cap, keys, level, prefix, first, count,
-                                             nchild, child, tmp);
-  }
-  if (lmax < kMaxLevel) {
-    k_tree_close<<<1, 32, 0, c->stream>>>(st, lmax);
-    c->launches += 1;
-  }
+  k_tree_count<<<tiles, kTreeThreads, 0, c->stream>>>(keys, n, leaf, lmax, cnt);
+  NG_TRY(scan_u32(c, cnt, cnt, (int64_t)tiles * (lmax + 1), nullptr, st + ST_NODES_NEEDED));
+  k_tree_emit<<<tiles, kTreeThreads, 0, c->stream>>>(
+      keys, n, leaf, lmax, cnt, st, cap, as<uint8_t>(c->n_level), as<uint64_t>(c->n_prefix),
+      as<uint32_t>(c->n_first), as<uint32_t>(c->n_child),
+      as<uint32_t>(c->mono_words));
+  k_tree_nodes<<<work_grid(c, std::min<int64_t>(cap, 2 * n + 64), 8), 256, 0, c->stream>>>(
+      st, cap, keys, n, leaf, lmax, as<uint8_t>(c->n_level), as<uint64_t>(c->n_prefix),
+      as<uint32_t>(c->n_first), as<uint32_t>(c->n_child), as<uint32_t>(c->n_count),
+      as<uint8_t>(c->n_nchild), as<uint32_t>(c->bleaf), as<int4>(c->n_link));
+  c->launches += 3;   // count, emit, nodes (the scan counts itself)
   NG_CUDA(c, cudaGetLastError());
   return NG_OK;
 }
@@ -347,124 +315,460 @@ struct MonoArgs {
   float4* body;            // [sorted body]
   uint32_t* bleaf;         // [sorted body] leaf index
   uint32_t* status;
-  int64_t n, cap;
+  int64_t n;
   double invL, L;
+  bool unit;               // L == 1: physical and box units are the same
 };
 
-// One thread per node of level lvl (FP64 is ~1/64 of the FP32 rate here, so
-// every FP64 operation counts): a leaf adds each body to its own species
-// (4 FP64 operations per body, in shared-memory slots chosen by the species)
-// and writes the body records (offset from the leaf centre, subtracted in
-// FP64 in physical units, scaled to box units in FP32); an internal node adds
-// its <= 8 children. The FP32 walk records need no FP64 division: the
-// mass-weighted offset sum(m x) - M c is formed with one FP64 FMA and divided
-// by M in FP32.
+// Below kBinnedMonoBodies bodies, leaves are summed from tiles of consecutive
+// bodies in shared memory: the body arrays are read once, coalesced, and every
+// body's record (offset from its leaf's centre, subtracted in FP64 in physical
+// units, scaled to box units in FP32) is written coalesced. A leaf is then summed by one thread
+// (FP64 is ~1/64 of the FP32 rate here, so every FP64 operation counts): it
+// adds each body to its own species, 4 FP64 operations per body, in
+// shared-memory slots chosen by the species. A warp instruction costs the
+// same with idle lanes, so the tile's leaves are taken in the order of their
+// body counts: the threads of a warp then have about equal loop counts. An
+// internal node is summed by one lane per species and component over its <= 8
+// children, in child order. The FP32 walk records need no FP64 division: the mass-weighted
+// offset sum(m x) - M c is formed with one FP64 FMA and divided by M in FP32.
 constexpr int kMonoThreads = 128;
 
-// Sums of node k of level lvl (leaf: its bodies; internal node: its <= 8
-// children) into the node's FP64 monopoles and FP32 walk records. lacc: the
-// calling thread's per-species leaf sums {m, m x, m y, m z} (physical units),
-// addressed by the body's species: no FP64 instruction is spent on the
-// species a body does not have (predicated per-species sums would issue D
-// times as many, and FP64 issues at 1/64 of the FP32 rate here).
+// The walk record {com - centre, mass} of FP64 sums about centre cen.
+__device__ __forceinline__ float4 mono_record(double m, double x, double y, double z,
+                                              const double cen[3]) {
+  if (!(m > 0.0)) return make_float4(0.f, 0.f, 0.f, 0.f);
+  const float mf = (float)m, im = 1.0f / mf;
+  return make_float4((float)fma(-m, cen[0], x) * im, (float)fma(-m, cen[1], y) * im,
+                     (float)fma(-m, cen[2], z) * im, mf);
+}
+
+// Lanes of an internal node's team: 4 components {m, m x, m y, m z} for each
+// of walk_tab_pad(D) species. The children's records are contiguous, so a
+// team reads whole lines, and a warp issues an FP64 instruction per child
+// rather than four.
 template <int D>
-__device__ __forceinline__ void mono_node(int lvl, uint32_t k, const MonoArgs& a,
-                                          double (*lacc)[4][kMonoThreads], int tid) {
+constexpr int kTeam = 4 * walk_tab_pad(D);
+
+// An internal node as its team needs it, loaded ahead of the children's sums.
+struct MonoNode {
+  uint32_t k, nch, c0;   // nch = 0: no node
+  int level;
+  uint64_t prefix;
+};
+__device__ __forceinline__ MonoNode mono_load(bool valid, uint32_t k, const MonoArgs& a) {
+  MonoNode v{k, 0u, 0u, 0, 0ull};
+  if (valid) {
+    v.nch = a.nchild[k];
+    v.c0 = a.child[k];
+    v.level = a.level[k];
+    v.prefix = a.prefix[k];
+  }
+  return v;
+}
+
+// geo of a node, {centre, half side} in box units: exact in FP32 (a centre
+// is an odd number below 2^22 over a power of two).
+__device__ __forceinline__ float4 mono_geo(int level, uint64_t prefix) {
+  const float h = __int_as_float((127 - (level + 1)) << 23);   // 2^-(level + 1)
+  return make_float4((float)(2u * morton_compact3(prefix >> 2) + 1u) * h,
+                     (float)(2u * morton_compact3(prefix >> 1) + 1u) * h,
+                     (float)(2u * morton_compact3(prefix) + 1u) * h, h);
+}
+
+// Sums of internal node v over its children, in child order, by the kTeam<D>
+// lanes of its team. All lanes of the warp call it together.
+template <int D>
+__device__ __forceinline__ void mono_internal(const MonoNode& v, const MonoArgs& a) {
+  constexpr int P = walk_tab_pad(D);
+  const int lane = threadIdx.x & 31, e = lane & 3, q = (lane >> 2) & (P - 1);
+  const bool mine = v.nch > 0 && q < D;
+  double c[8];
+  uint32_t cn = 0;
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    c[j] = 0.0;
+    if (mine && j < (int)v.nch) {
+      const size_t r = (size_t)(v.c0 + j) * D + q;
+      c[j] = a.m64[r * 4 + e];
+      if (e == 0) cn += a.cnt[r];
+    }
+  }
+  // no further than the longest list of the warp
+  const int most = (int)__reduce_max_sync(0xffffffffu, v.nch);
+  double sum = 0.0;
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    if (j >= most) break;
+    sum += c[j];
+  }
+  // over the species (zero in idle lanes), for the node's own centre of mass
+  double all = sum;
+#pragma unroll
+  for (int o = 4; o < kTeam<D>; o <<= 1) all += __shfl_xor_sync(0xffffffffu, all, o);
+  const double m = __shfl_sync(0xffffffffu, sum, 0, 4), mt = __shfl_sync(0xffffffffu, all, 0, 4);
+  if (!mine) return;
   double cen[3], side;
-  node_centre(lvl, a.prefix[k], cen, &side);
+  node_centre(v.level, v.prefix, cen, &side);
+  const double ce = e == 1 ? cen[0] : e == 2 ? cen[1] : cen[2];
+  // records {com - centre, mass}: component e - 1, or the mass for e = 0
+  const size_t r = (size_t)v.k * D + q;
+  const int at = (e + 3) & 3;
+  const float mf = (float)m, f = e == 0 ? mf : (float)fma(-m, ce, sum) * (1.0f / mf);
+  a.m64[r * 4 + e] = sum;
+  reinterpret_cast<float*>(a.mono)[r * 4 + at] = m > 0.0 ? f : 0.f;
+  if (e == 0) a.cnt[r] = cn;
+  if (q == 0) {
+    const float tf = (float)mt, g = e == 0 ? tf : (float)fma(-mt, ce, all) * (1.0f / tf);
+    reinterpret_cast<float*>(a.com)[(size_t)v.k * 4 + at] = mt > 0.0 ? g : 0.f;
+    if (e == 0) a.geo[v.k] = mono_geo(v.level, v.prefix);
+    if (e == 1) a.link[v.k] = make_int4((int)v.c0, (int)v.nch, (int)a.first[v.k], (int)a.count[v.k]);
+  }
+}
+
+// The same sums by the calling lane alone, all species: an FP64 instruction
+// then serves 32 nodes, against 32 / kTeam<D> in teams, for four times as many
+// of them in a row. Taken where the nodes make kLaneLevel rounds of teams.
+constexpr uint32_t kLaneLevel = 4;
+template <int D>
+__device__ __forceinline__ void mono_internal_lane(const MonoNode& v, const MonoArgs& a) {
+  if (v.nch == 0) return;
   double sm[D], sx[D], sy[D], sz[D];
   uint32_t sc[D];
 #pragma unroll
-  for (int t = 0; t < D; ++t) { sm[t] = sx[t] = sy[t] = sz[t] = 0.0; sc[t] = 0; }
-  const uint32_t nch = a.nchild[k];
-  const uint32_t f = a.first[k], c = a.count[k];
-  if (nch == 0) {
-#pragma unroll
-    for (int q = 0; q < D; ++q)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) lacc[q][j][tid] = 0.0;
-    // leaf centre in physical units; body records are offsets from it in box units
-    const double cxL = cen[0] * a.L, cyL = cen[1] * a.L, czL = cen[2] * a.L;
-    const float invLf = (float)a.invL;
-    for (uint32_t b = f; b < f + c; ++b) {
-      const double xp = a.spos[b], yp = a.spos[a.n + b], zp = a.spos[2 * a.n + b];
-      const float m = a.smass[b];
-      const int t = a.stype[b];
-      a.body[b] = make_float4((float)(xp - cxL) * invLf, (float)(yp - cyL) * invLf,
-                              (float)(zp - czL) * invLf, m);
-      a.bleaf[b] = k;
-      const double md = (double)m;
-      lacc[t][0][tid] += md;
-      lacc[t][1][tid] = fma(md, xp, lacc[t][1][tid]);
-      lacc[t][2][tid] = fma(md, yp, lacc[t][2][tid]);
-      lacc[t][3][tid] = fma(md, zp, lacc[t][3][tid]);
-#pragma unroll
-      for (int q = 0; q < D; ++q) sc[q] += t == q ? 1u : 0u;
-    }
-    // to box units (exact when the box is a power of two)
+  for (int q = 0; q < D; ++q) { sm[q] = sx[q] = sy[q] = sz[q] = 0.0; sc[q] = 0; }
+  for (uint32_t j = 0; j < v.nch; ++j) {
+    const size_t r = (size_t)(v.c0 + j) * D;
 #pragma unroll
     for (int q = 0; q < D; ++q) {
-      sm[q] = lacc[q][0][tid];
-      sx[q] = lacc[q][1][tid] * a.invL;
-      sy[q] = lacc[q][2][tid] * a.invL;
-      sz[q] = lacc[q][3][tid] * a.invL;
-    }
-  } else {
-    const uint32_t c0 = a.child[k];
-    for (uint32_t j = 0; j < nch; ++j) {
-      const uint32_t ch = c0 + j;
-#pragma unroll
-      for (int q = 0; q < D; ++q) {
-        const double4_32a v = *reinterpret_cast<const double4_32a*>(a.m64 + ((size_t)ch * D + q) * 4);
-        sm[q] += v.x;
-        sx[q] += v.y;
-        sy[q] += v.z;
-        sz[q] += v.w;
-        sc[q] += a.cnt[(size_t)ch * D + q];
-      }
+      const double4_32a c = *reinterpret_cast<const double4_32a*>(a.m64 + (r + q) * 4);
+      sm[q] += c.x;
+      sx[q] += c.y;
+      sy[q] += c.z;
+      sz[q] += c.w;
+      sc[q] += a.cnt[r + q];
     }
   }
+  double cen[3], side;
+  node_centre(v.level, v.prefix, cen, &side);
   double mt = 0, xt = 0, yt = 0, zt = 0;
 #pragma unroll
   for (int q = 0; q < D; ++q) {
-    // 32-byte records from a cudaMalloc base: one aligned 32-byte access each
-    *reinterpret_cast<double4_32a*>(a.m64 + ((size_t)k * D + q) * 4) =
-        make_double4_32a(sm[q], sx[q], sy[q], sz[q]);
-    a.cnt[(size_t)k * D + q] = sc[q];
-    float4 r = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (sm[q] > 0.0) {
-      const float im = 1.0f / (float)sm[q];
-      r = make_float4((float)fma(-sm[q], cen[0], sx[q]) * im, (float)fma(-sm[q], cen[1], sy[q]) * im,
-                      (float)fma(-sm[q], cen[2], sz[q]) * im, (float)sm[q]);
-    }
-    a.mono[(size_t)k * D + q] = r;
+    const size_t r = (size_t)v.k * D + q;
+    *reinterpret_cast<double4_32a*>(a.m64 + r * 4) = make_double4_32a(sm[q], sx[q], sy[q], sz[q]);
+    a.cnt[r] = sc[q];
+    a.mono[r] = mono_record(sm[q], sx[q], sy[q], sz[q], cen);
     mt += sm[q];
     xt += sx[q];
     yt += sy[q];
     zt += sz[q];
   }
-  a.geo[k] = make_float4((float)cen[0], (float)cen[1], (float)cen[2], (float)(0.5 * side));
-  float4 r = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (mt > 0.0) {
-    const float im = 1.0f / (float)mt;
-    r = make_float4((float)fma(-mt, cen[0], xt) * im, (float)fma(-mt, cen[1], yt) * im,
-                    (float)fma(-mt, cen[2], zt) * im, (float)mt);
-  }
-  a.com[k] = r;
-  a.link[k] = make_int4(nch ? (int)a.child[k] : -1, (int)nch, (int)f, (int)c);
+  a.geo[v.k] = mono_geo(v.level, v.prefix);
+  a.com[v.k] = mono_record(mt, xt, yt, zt, cen);
+  a.link[v.k] = make_int4((int)v.c0, (int)v.nch, (int)a.first[v.k], (int)a.count[v.k]);
 }
 
-// Trees of kBinnedMonoBodies bodies or more: one thread per node, in an
-// order binned by the node's work. A leaf loops over its bodies and an
-// internal node over its children, so a warp runs as long as its longest
-// loop; FP64 issues at 1/64 of the FP32 rate here and a warp instruction
-// costs the same with idle lanes. Taken in level (Morton) order, the leaves
-// of a warp hold 1 to leaf_size bodies and a warp ran 2.5 times the
+// The internal nodes are reduced by subtrees. A subtree is rooted at an
+// internal node of at most `sub` bodies whose parent holds more (or at such a
+// root of the whole tree); one block reduces all its levels bottom-up, with no
+// launch between levels. The nodes above, fewer than n / sub per level, are
+// listed by level and reduced by one thread-block cluster; sub grows with n so
+// that they stay few thousands.
+// One launch per level (21 of them, each waiting for the slowest warp of a
+// level) took 212 us at 131k bodies and three species, the three launches
+// here 121 us.
+//
+// Counters (c->mono_words, zeroed by k_tree_emit): the subtrees and the top
+// nodes per level. Subtree roots are listed in n_tmp, top
+// nodes of level l at top[l * per], top = the tree build's scratch.
+struct MonoLists {
+  uint32_t* words;
+  uint32_t* roots;   // n_tmp
+  uint32_t* top;     // tree_cnt
+  uint32_t sub;      // bodies of the largest subtree
+  uint32_t per;      // top nodes a level can hold
+};
+constexpr int kMlSub = 0, kMlTop = 1;
+static_assert(kMlTop + kMaxLevel + 1 == kMonoWords && kMonoWords <= kTreeThreads, "monopole counters");
+
+// Internal node k into the top list if it is large, into the subtree list if
+// it is small and its parent (left in its link by k_tree_nodes) is not.
+__device__ __forceinline__ void mono_list(uint32_t k, const MonoArgs& a, const MonoLists& m) {
+  if (a.count[k] > m.sub) {
+    const int l = a.level[k];
+    m.top[(size_t)l * m.per + atomicAdd(&m.words[kMlTop + l], 1u)] = k;
+  } else if (k == 0 || a.count[a.link[k].w] > m.sub) {
+    m.roots[atomicAdd(&m.words[kMlSub], 1u)] = k;
+  }
+}
+
+// Tile: bodies whose leaves start in a block's turn (small, so that a small
+// tree's leaves reach many SMs); a leaf may reach kMaxLeaf bodies into the next.
+constexpr int kLeafThreads = 64, kLeafTile = 256, kLeafLoad = kLeafTile + kMaxLeaf;
+template <int D>
+struct LeafSmem {
+  double x[3][kLeafLoad];
+  float m[kLeafLoad];
+  double acc[D][4][kLeafThreads];        // {m, m x, m y, m z} per species, physical units
+  uint32_t start[kLeafTile];             // local start | count class << 16, then in count order
+  uint32_t order[kLeafTile];
+  uint32_t bins[kMaxLeaf + 2];
+  uint32_t warp_tot[kLeafThreads / 32], tile_total;
+  uint8_t t[kLeafLoad];
+};
+
+// Every leaf and body record, one tile of bodies per block and turn; the
+// internal nodes into their lists.
+template <int D>
+__global__ void __launch_bounds__(kLeafThreads) k_mono_tiles(MonoArgs a, MonoLists ml) {
+  __shared__ LeafSmem<D> sm;
+  if (a.status[ST_FLAGS] & SF_NODE_OVERFLOW) return;   // truncated tree: do not read it
+  const int tid = threadIdx.x;
+  const uint32_t total = levels_of(a.status).start[kMaxLevel + 1];
+  for (uint32_t k = blockIdx.x * blockDim.x + tid; k < total; k += gridDim.x * blockDim.x) {
+    if (a.nchild[k]) mono_list(k, a, ml);
+  }
+  const float invLf = (float)a.invL;
+  for (int64_t t0 = (int64_t)blockIdx.x * kLeafTile; t0 < a.n; t0 += (int64_t)gridDim.x * kLeafTile) {
+    __syncthreads();   // the previous tile's readers are done
+    const int held = (int)min((int64_t)kLeafLoad, a.n - t0), own = min(held, kLeafTile);
+    for (int j = tid; j < kMaxLeaf + 2; j += kLeafThreads) sm.bins[j] = 0;
+    uint32_t nleaf = 0;   // leaves that start in the tile (the same in every thread)
+    for (int j0 = 0; j0 < held; j0 += kLeafThreads) {
+      const int j = j0 + tid;
+      bool head = false;
+      if (j < held) {
+        const int64_t b = t0 + j;
+        const double xp = a.spos[b], yp = a.spos[a.n + b], zp = a.spos[2 * a.n + b];
+        const float m = a.smass[b];
+        sm.x[0][j] = xp;
+        sm.x[1][j] = yp;
+        sm.x[2][j] = zp;
+        sm.m[j] = m;
+        sm.t[j] = a.stype[b];
+        if (j < own) {
+          const uint32_t k = a.bleaf[b];
+          head = b == 0 || a.bleaf[b - 1] != k;
+          double cen[3], side;
+          node_centre(a.level[k], a.prefix[k], cen, &side);
+          if (!a.unit) {
+            cen[0] *= a.L;
+            cen[1] *= a.L;
+            cen[2] *= a.L;
+          }
+          a.body[b] = make_float4((float)(xp - cen[0]) * invLf, (float)(yp - cen[1]) * invLf,
+                                  (float)(zp - cen[2]) * invLf, m);
+        }
+      }
+      const uint32_t inc = block_inclusive_scan<kLeafThreads>(head ? 1u : 0u, sm.warp_tot, &sm.tile_total);
+      if (head) sm.start[nleaf + inc - 1] = (uint32_t)j;
+      nleaf += sm.tile_total;
+      __syncthreads();
+    }
+    // the leaves by body count (one class for those above kMaxLeaf)
+    for (uint32_t i = tid; i < nleaf; i += kLeafThreads) {
+      const uint32_t cls = min(a.count[a.bleaf[t0 + sm.start[i]]], (uint32_t)(kMaxLeaf + 1));
+      sm.start[i] |= cls << 16;
+      atomicAdd(&sm.bins[cls], 1u);
+    }
+    __syncthreads();
+    if (tid < 32) {
+      uint32_t run = 0;
+      for (int c = kMaxLeaf + 1; c >= 0; c -= 32) {   // longest first
+        const int j = c - tid;
+        const uint32_t v = j >= 0 ? sm.bins[j] : 0u;
+        uint32_t inc = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const uint32_t x = __shfl_up_sync(0xffffffffu, inc, o);
+          if (tid >= o) inc += x;
+        }
+        if (j >= 0) sm.bins[j] = run + inc - v;
+        run += __shfl_sync(0xffffffffu, inc, 31);
+      }
+    }
+    __syncthreads();
+    for (uint32_t i = tid; i < nleaf; i += kLeafThreads)
+      sm.order[atomicAdd(&sm.bins[sm.start[i] >> 16], 1u)] = sm.start[i] & 0xffffu;
+    __syncthreads();
+    for (uint32_t i = tid; i < nleaf; i += kLeafThreads) {
+      const int j0 = (int)sm.order[i];
+      const uint32_t k = a.bleaf[t0 + j0], c = a.count[k];
+      uint32_t sc[D];
+#pragma unroll
+      for (int q = 0; q < D; ++q) {
+        sc[q] = 0;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) sm.acc[q][e][tid] = 0.0;
+      }
+      for (uint32_t h = 0; h < c; ++h) {
+        const int j = j0 + (int)h;
+        double xp, yp, zp, md;
+        int t;
+        if (j < held) {
+          xp = sm.x[0][j];
+          yp = sm.x[1][j];
+          zp = sm.x[2][j];
+          md = (double)sm.m[j];
+          t = sm.t[j];
+        } else {   // a leaf above kMaxLeaf bodies (a tree stopped at a level cap)
+          const int64_t b = t0 + j;
+          xp = a.spos[b];
+          yp = a.spos[a.n + b];
+          zp = a.spos[2 * a.n + b];
+          md = (double)a.smass[b];
+          t = a.stype[b];
+        }
+        sm.acc[t][0][tid] += md;
+        sm.acc[t][1][tid] = fma(md, xp, sm.acc[t][1][tid]);
+        sm.acc[t][2][tid] = fma(md, yp, sm.acc[t][2][tid]);
+        sm.acc[t][3][tid] = fma(md, zp, sm.acc[t][3][tid]);
+#pragma unroll
+        for (int q = 0; q < D; ++q) sc[q] += t == q ? 1u : 0u;
+      }
+      double cen[3], side;
+      node_centre(a.level[k], a.prefix[k], cen, &side);
+      double mt = 0, xt = 0, yt = 0, zt = 0;
+#pragma unroll
+      for (int q = 0; q < D; ++q) {
+        // to box units (exact when the box is a power of two)
+        const double m = sm.acc[q][0][tid];
+        double x = sm.acc[q][1][tid], y = sm.acc[q][2][tid], z = sm.acc[q][3][tid];
+        if (!a.unit) {
+          x *= a.invL;
+          y *= a.invL;
+          z *= a.invL;
+        }
+        // 32-byte records from a cudaMalloc base: one aligned 32-byte access each
+        *reinterpret_cast<double4_32a*>(a.m64 + ((size_t)k * D + q) * 4) = make_double4_32a(m, x, y, z);
+        a.cnt[(size_t)k * D + q] = sc[q];
+        a.mono[(size_t)k * D + q] = mono_record(m, x, y, z, cen);
+        mt += m;
+        xt += x;
+        yt += y;
+        zt += z;
+      }
+      a.geo[k] = mono_geo(a.level[k], a.prefix[k]);
+      a.com[k] = mono_record(mt, xt, yt, zt, cen);
+      a.link[k] = make_int4(-1, 0, (int)(t0 + j0), (int)c);
+    }
+  }
+}
+
+// One block per subtree: the internal nodes of a level are packed and then
+// summed one per lane where they fill the block's warps, else in teams.
+template <int D>
+__global__ void __launch_bounds__(kMonoThreads) k_mono_subtrees(MonoArgs a, MonoLists m) {
+  constexpr int kTeams = kMonoThreads / kTeam<D>;
+  __shared__ uint2 range[kMaxLevel + 1];
+  __shared__ uint32_t packed[kMaxSub / 2];   // a level's internal nodes hold two bodies or more
+  __shared__ uint32_t held[2];
+  __shared__ int deepest;
+  if (a.status[ST_FLAGS] & SF_NODE_OVERFLOW) return;
+  const int tid = threadIdx.x, lane = tid & 31;
+  Levels lv = levels_of(a.status);
+  const uint32_t roots = m.words[kMlSub];
+  for (uint32_t i = blockIdx.x; i < roots; i += gridDim.x) {
+    const uint32_t k = m.roots[i];
+    const int l0 = a.level[k];
+    if (tid < 32) {
+      // node range of the subtree per level: children are numbered in node order
+      uint32_t s = k, e = k + 1;
+      int l = l0;
+      while (s < e && l <= kMaxLevel) {
+        if (lane == 0) range[l] = make_uint2(s, e);
+        const uint32_t ns = a.child[s];
+        e = l == kMaxLevel ? ns : e < lv.start[l + 1] ? a.child[e] : lv.start[l + 2];
+        s = ns;
+        ++l;
+      }
+      if (lane == 0) {
+        deepest = l - 1;   // this level holds leaves only
+        held[0] = 0;
+      }
+    }
+    __syncthreads();
+    int turn = 0;
+    for (int x = deepest - 1; x >= l0; --x) {
+      const uint2 r = range[x];
+      for (uint32_t b = r.x; b < r.y; b += kMonoThreads) {
+        const uint32_t node = b + tid;
+        if (node < r.y && a.nchild[node]) packed[atomicAdd(&held[turn], 1u)] = node;
+      }
+      if (tid == 0) held[turn ^ 1] = 0;
+      __syncthreads();
+      const uint32_t cnt = held[turn];
+      turn ^= 1;
+      if (cnt >= kLaneLevel * kTeams) {
+        for (uint32_t j = tid; j < cnt; j += kMonoThreads)
+          mono_internal_lane<D>(mono_load(true, packed[j], a), a);
+      } else {
+        for (uint32_t j0 = 0; j0 < cnt; j0 += kTeams) {
+          const uint32_t j = j0 + tid / kTeam<D>;
+          mono_internal<D>(mono_load(j < cnt, j < cnt ? packed[j] : 0u, a), a);
+        }
+      }
+      __syncthreads();   // this level's sums are read by the next
+    }
+  }
+}
+
+// The nodes above the subtrees, level by level, by one cluster of
+// kClusterBlocks blocks (co-scheduled; its barrier is the hardware cluster
+// barrier, so no block waits on a flag).
+template <int D>
+__global__ void __cluster_dims__(kClusterBlocks, 1, 1) __launch_bounds__(512)
+k_mono_top(int lmax, MonoArgs a, MonoLists m) {
+  // the flag and the counts are the same for every block and not written
+  // here: every block returns, or none does
+  if (a.status[ST_FLAGS] & SF_NODE_OVERFLOW) return;
+  namespace cg = cooperative_groups;
+  cg::cluster_group cluster = cg::this_cluster();
+  const int lane = threadIdx.x & 31;
+  const uint32_t team = (blockIdx.x * blockDim.x + threadIdx.x) / kTeam<D>;
+  const uint32_t teams = gridDim.x * blockDim.x / kTeam<D>;
+  const uint32_t counts = m.words[kMlTop + min(lane, kMaxLevel)];   // lane l: level l
+  uint32_t some = __ballot_sync(0xffffffffu, counts != 0 && lane < lmax);   // levels with nodes
+  auto load = [&](int l, uint32_t i, uint32_t cnt) {
+    const bool has = i < cnt;
+    return mono_load(has, has ? m.top[(size_t)l * m.per + i] : 0u, a);
+  };
+  if (!some) return;
+  int l = 31 - __clz(some);
+  uint32_t cnt = __shfl_sync(0xffffffffu, counts, l);
+  MonoNode v = load(l, team, cnt);
+  while (true) {
+    if (cnt >= kLaneLevel * teams) {
+      for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < cnt; i += gridDim.x * blockDim.x)
+        mono_internal_lane<D>(load(l, i, cnt), a);
+    } else {
+      mono_internal<D>(v, a);
+      for (uint32_t i = team + teams; i - lane / kTeam<D> < cnt; i += teams)
+        mono_internal<D>(load(l, i, cnt), a);
+    }
+    some &= ~(1u << l);
+    if (!some) break;
+    // the next level's nodes are loaded before its children's sums are awaited
+    l = 31 - __clz(some);
+    cnt = __shfl_sync(0xffffffffu, counts, l);
+    v = load(l, team, cnt);
+    cluster.sync();
+  }
+}
+
+// Trees of kBinnedMonoBodies bodies or more: the leaves one thread each, all
+// in one launch, then the internal nodes one thread each, one launch per
+// level, bottom-up, both in an order binned by the node's work. A leaf loops
+// over its bodies and an internal node over its children, so a warp runs as
+// long as its longest loop; FP64 issues at 1/64 of the FP32 rate here and a
+// warp instruction costs the same with idle lanes. In Morton order the
+// leaves of a warp hold 1 to leaf_size bodies and a warp ran 2.5 times the
 // iterations its bodies need (2^24 clustered bodies, leaf 32); binned, the
-// threads of a warp have equal loop counts. All leaves are reduced by one
-// launch (a leaf needs no other node), then the internal nodes level by
-// level, bottom-up. Each node is still summed by one thread in its own order,
-// so the results do not depend on the binning.
+// threads of a warp have equal loop counts. Each node is still summed by one
+// thread in its own order, so the results do not depend on the binning. At
+// these sizes a level's launch is filled by its nodes, and the subtrees' blocks
+// above wait on memory between their levels instead (3 M bodies, leaf 8,
+// D = 3: tiles and subtrees 701 us, this path 549 us).
 static_assert(kMonoBins <= 256, "the bin scan takes one bin per thread of a 256-thread block");
 
 __device__ __forceinline__ int mono_bin(uint32_t lvl, uint32_t nch, uint32_t cnt) {
@@ -472,18 +776,14 @@ __device__ __forceinline__ int mono_bin(uint32_t lvl, uint32_t nch, uint32_t cnt
 }
 
 // bins[0, kMonoBins): nodes per bin (zeroed before the launch)
-__global__ void __launch_bounds__(256) k_mono_hist(uint32_t* status, int64_t cap,
-                                                   const uint8_t* __restrict__ level,
-                                                   const uint8_t* __restrict__ nchild,
-                                                   const uint32_t* __restrict__ count, uint32_t* bins) {
+__global__ void __launch_bounds__(256) k_mono_hist(MonoArgs a, uint32_t* bins) {
   __shared__ uint32_t h[kMonoBins];
-  if (status[ST_FLAGS] & SF_NODE_OVERFLOW) return;   // truncated tree: do not read it
+  if (a.status[ST_FLAGS] & SF_NODE_OVERFLOW) return;   // truncated tree: do not read it
   for (int i = threadIdx.x; i < kMonoBins; i += blockDim.x) h[i] = 0;
   __syncthreads();
-  uint32_t total = levels_of(status).start[kMaxLevel + 1];
-  if (total > cap) total = (uint32_t)cap;
+  const uint32_t total = levels_of(a.status).start[kMaxLevel + 1];
   for (uint32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < total; k += gridDim.x * blockDim.x)
-    atomicAdd(&h[mono_bin(level[k], nchild[k], count[k])], 1u);
+    atomicAdd(&h[mono_bin(a.level[k], a.nchild[k], a.count[k])], 1u);
   __syncthreads();
   for (int i = threadIdx.x; i < kMonoBins; i += blockDim.x)
     if (h[i]) atomicAdd(&bins[i], h[i]);
@@ -494,16 +794,12 @@ __global__ void __launch_bounds__(256) k_mono_hist(uint32_t* status, int64_t cap
 // bins[2 kMonoBins, 3 kMonoBins] (the last entry: all nodes). Each block
 // places one contiguous chunk of nodes, reserving its share of every bin with
 // one atomic per bin. Launched with 256 threads.
-__global__ void __launch_bounds__(256) k_mono_order(uint32_t* status, int64_t cap,
-                                                    const uint8_t* __restrict__ level,
-                                                    const uint8_t* __restrict__ nchild,
-                                                    const uint32_t* __restrict__ count, uint32_t* bins,
-                                                    uint32_t* order) {
+__global__ void __launch_bounds__(256) k_mono_order(MonoArgs a, uint32_t* bins, uint32_t* order) {
   __shared__ uint32_t lh[kMonoBins];
   __shared__ uint32_t base[kMonoBins];
   __shared__ uint32_t warp_tot[8];
   __shared__ uint32_t all;
-  if (status[ST_FLAGS] & SF_NODE_OVERFLOW) return;
+  if (a.status[ST_FLAGS] & SF_NODE_OVERFLOW) return;
   const int tid = threadIdx.x;
   // bin starts: exclusive scan of the bin counts
   const uint32_t v = tid < kMonoBins ? bins[tid] : 0u;
@@ -515,33 +811,71 @@ __global__ void __launch_bounds__(256) k_mono_order(uint32_t* status, int64_t ca
   }
   if (blockIdx.x == 0 && tid == 0) bins[3 * kMonoBins] = all;
   __syncthreads();
-  uint32_t total = levels_of(status).start[kMaxLevel + 1];
-  if (total > cap) total = (uint32_t)cap;
+  const uint32_t total = levels_of(a.status).start[kMaxLevel + 1];
   const uint32_t chunk = (total + gridDim.x - 1) / gridDim.x;
   const uint32_t k0 = min(total, blockIdx.x * chunk), k1 = min(total, k0 + chunk);
   for (uint32_t k = k0 + tid; k < k1; k += blockDim.x)
-    atomicAdd(&lh[mono_bin(level[k], nchild[k], count[k])], 1u);
+    atomicAdd(&lh[mono_bin(a.level[k], a.nchild[k], a.count[k])], 1u);
   __syncthreads();
   if (tid < kMonoBins && lh[tid]) base[tid] += atomicAdd(&bins[kMonoBins + tid], lh[tid]);
   __syncthreads();
   for (uint32_t k = k0 + tid; k < k1; k += blockDim.x)
-    order[atomicAdd(&base[mono_bin(level[k], nchild[k], count[k])], 1u)] = k;
+    order[atomicAdd(&base[mono_bin(a.level[k], a.nchild[k], a.count[k])], 1u)] = k;
 }
 
-// Trees below kBinnedMonoBodies bodies: one launch per level, bottom-up, one
-// thread per node of the level in level order. Their levels hold few nodes,
-// so the three launches of the binned order cost more than its convergence
-// saves (batches of 2^12..2^18-body simulations: 7.74 against 8.11 ms).
+// Sums of leaf k: its bodies into the node's FP64 monopoles and FP32 walk
+// records. lacc: the calling thread's per-species sums {m, m x, m y, m z}
+// (physical units), addressed by the body's species: no FP64 instruction is
+// spent on the species a body does not have (predicated per-species sums
+// would issue D times as many).
 template <int D>
-__global__ void __launch_bounds__(kMonoThreads) k_monopoles(int lvl, MonoArgs a) {
-  __shared__ double lacc[D][4][kMonoThreads];
-  if (a.status[ST_FLAGS] & SF_NODE_OVERFLOW) return;   // truncated tree: do not read it
-  Levels lv = levels_of(a.status);
-  const uint32_t s = lv.start[lvl];
-  uint32_t e = lv.start[lvl + 1];
-  if (e > a.cap) e = (uint32_t)a.cap;
-  for (uint32_t k = s + blockIdx.x * blockDim.x + threadIdx.x; k < e; k += gridDim.x * blockDim.x)
-    mono_node<D>(lvl, k, a, lacc, threadIdx.x);
+__device__ __forceinline__ void mono_leaf(uint32_t k, const MonoArgs& a,
+                                          double (*lacc)[4][kMonoThreads], int tid) {
+  double cen[3], side;
+  node_centre(a.level[k], a.prefix[k], cen, &side);
+  uint32_t sc[D];
+#pragma unroll
+  for (int q = 0; q < D; ++q) {
+    sc[q] = 0;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) lacc[q][j][tid] = 0.0;
+  }
+  const uint32_t f = a.first[k], c = a.count[k];
+  // leaf centre in physical units; body records are offsets from it in box units
+  const double cxL = cen[0] * a.L, cyL = cen[1] * a.L, czL = cen[2] * a.L;
+  const float invLf = (float)a.invL;
+  for (uint32_t b = f; b < f + c; ++b) {
+    const double xp = a.spos[b], yp = a.spos[a.n + b], zp = a.spos[2 * a.n + b];
+    const float m = a.smass[b];
+    const int t = a.stype[b];
+    a.body[b] = make_float4((float)(xp - cxL) * invLf, (float)(yp - cyL) * invLf,
+                            (float)(zp - czL) * invLf, m);
+    const double md = (double)m;
+    lacc[t][0][tid] += md;
+    lacc[t][1][tid] = fma(md, xp, lacc[t][1][tid]);
+    lacc[t][2][tid] = fma(md, yp, lacc[t][2][tid]);
+    lacc[t][3][tid] = fma(md, zp, lacc[t][3][tid]);
+#pragma unroll
+    for (int q = 0; q < D; ++q) sc[q] += t == q ? 1u : 0u;
+  }
+  double mt = 0, xt = 0, yt = 0, zt = 0;
+#pragma unroll
+  for (int q = 0; q < D; ++q) {
+    // to box units (exact when the box is a power of two)
+    const double m = lacc[q][0][tid], x = lacc[q][1][tid] * a.invL, y = lacc[q][2][tid] * a.invL,
+                 z = lacc[q][3][tid] * a.invL;
+    // 32-byte records from a cudaMalloc base: one aligned 32-byte access each
+    *reinterpret_cast<double4_32a*>(a.m64 + ((size_t)k * D + q) * 4) = make_double4_32a(m, x, y, z);
+    a.cnt[(size_t)k * D + q] = sc[q];
+    a.mono[(size_t)k * D + q] = mono_record(m, x, y, z, cen);
+    mt += m;
+    xt += x;
+    yt += y;
+    zt += z;
+  }
+  a.geo[k] = mono_geo(a.level[k], a.prefix[k]);
+  a.com[k] = mono_record(mt, xt, yt, zt, cen);
+  a.link[k] = make_int4(-1, 0, (int)f, (int)c);
 }
 
 // Every leaf of the tree: order[0, start of the first internal bin).
@@ -551,10 +885,8 @@ __global__ void __launch_bounds__(kMonoThreads) k_mono_leaves(MonoArgs a, const 
   __shared__ double lacc[D][4][kMonoThreads];
   if (a.status[ST_FLAGS] & SF_NODE_OVERFLOW) return;
   const uint32_t e = bins[2 * kMonoBins + kLeafBins];
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < e; i += gridDim.x * blockDim.x) {
-    const uint32_t k = order[i];
-    mono_node<D>(a.level[k], k, a, lacc, threadIdx.x);
-  }
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < e; i += gridDim.x * blockDim.x)
+    mono_leaf<D>(order[i], a, lacc, threadIdx.x);
 }
 
 // The internal nodes of level lvl (their children are done).
@@ -562,34 +894,51 @@ template <int D>
 __global__ void __launch_bounds__(kMonoThreads) k_mono_internal(int lvl, MonoArgs a,
                                                                 const uint32_t* __restrict__ bins,
                                                                 const uint32_t* __restrict__ order) {
-  __shared__ double lacc[D][4][kMonoThreads];
   if (a.status[ST_FLAGS] & SF_NODE_OVERFLOW) return;
   const uint32_t* start = bins + 2 * kMonoBins + kLeafBins + lvl * 8;
   const uint32_t s = start[0], e = start[8];
   for (uint32_t i = s + blockIdx.x * blockDim.x + threadIdx.x; i < e; i += gridDim.x * blockDim.x)
-    mono_node<D>(lvl, order[i], a, lacc, threadIdx.x);
+    mono_internal_lane<D>(mono_load(true, order[i], a), a);
 }
 
-// Every level of a small tree, bottom-up, in one launch: one cluster of
-// kClusterBlocks blocks with the hardware cluster barrier between levels.
 template <int D>
-__global__ void __cluster_dims__(kClusterBlocks, 1, 1) __launch_bounds__(kMonoThreads)
-k_monopoles_cluster(int lmax, MonoArgs a) {
-  __shared__ double lacc[D][4][kMonoThreads];
-  // the flag is read before any level and never written here: every block
-  // returns, or none does
-  if (a.status[ST_FLAGS] & SF_NODE_OVERFLOW) return;
-  namespace cg = cooperative_groups;
-  cg::cluster_group cluster = cg::this_cluster();
-  Levels lv = levels_of(a.status);
-  for (int l = lmax; l >= 0; --l) {
-    const uint32_t s = lv.start[l];
-    uint32_t e = lv.start[l + 1];
-    if (e > a.cap) e = (uint32_t)a.cap;
-    for (uint32_t k = s + blockIdx.x * blockDim.x + threadIdx.x; k < e; k += gridDim.x * blockDim.x)
-      mono_node<D>(l, k, a, lacc, threadIdx.x);
-    cluster.sync();
+static int launch_monopoles(ng_ctx* c, const MonoArgs& a, const MonoLists& m, int lmax) {
+  if (c->n < kBinnedMonoBodies) {
+    const int64_t tiles = (c->n + kLeafTile - 1) / kLeafTile;
+    k_mono_tiles<D><<<(int)std::min<int64_t>((int64_t)c->nsm * 16, tiles), kLeafThreads, 0, c->stream>>>(a, m);
+    c->launches += 1;
+    if (c->n > c->p.leaf_size) {   // else the root is a leaf
+      // at most eight subtrees under a top node
+      const int64_t subs = 8 * ((c->n + m.sub - 1) / m.sub);
+      k_mono_subtrees<D><<<(int)std::min<int64_t>((int64_t)c->nsm * 16, subs), kMonoThreads, 0, c->stream>>>(a, m);
+      c->launches += 1;
+      if (c->n > m.sub) {
+        k_mono_top<D><<<kClusterBlocks, 512, 0, c->stream>>>(lmax, a, m);
+        c->launches += 1;
+      }
+    }
+    NG_CUDA(c, cudaGetLastError());
+    return NG_OK;
   }
+  uint32_t* bins = as<uint32_t>(c->mono_words) + kMonoWords;
+  uint32_t* order = as<uint32_t>(c->n_tmp);
+  NG_CUDA(c, cudaMemsetAsync(bins, 0, 2 * kMonoBins * sizeof(uint32_t), c->stream));
+  const int64_t cap = std::min<int64_t>(c->cap_nodes, 2 * c->n + 64);
+  const int sgrid = work_grid(c, cap, 4);
+  k_mono_hist<<<sgrid, 256, 0, c->stream>>>(a, bins);
+  k_mono_order<<<sgrid, 256, 0, c->stream>>>(a, bins, order);
+  auto grid = [&](int64_t nodes) {
+    return (int)std::max<int64_t>(
+        1, std::min<int64_t>((int64_t)c->nsm * 16, (nodes + kMonoThreads - 1) / kMonoThreads));
+  };
+  k_mono_leaves<D><<<grid(cap), kMonoThreads, 0, c->stream>>>(a, bins, order);
+  // nodes at level lmax are leaves; a level holds at most 8^l nodes
+  for (int l = lmax - 1; l >= 0; --l)
+    k_mono_internal<D><<<grid(std::min<int64_t>(cap, (int64_t)1 << std::min(3 * l, 40))), kMonoThreads, 0,
+                         c->stream>>>(l, a, bins, order);
+  c->launches += 3 + lmax;
+  NG_CUDA(c, cudaGetLastError());
+  return NG_OK;
 }
 
 int reduce_monopoles(ng_ctx* c) {
@@ -613,77 +962,22 @@ int reduce_monopoles(ng_ctx* c) {
   a.bleaf = as<uint32_t>(c->bleaf);
   a.status = as<uint32_t>(c->status);
   a.n = c->n;
-  a.cap = c->cap_nodes;
   a.invL = 1.0 / c->L;
   a.L = c->L;
+  a.unit = c->L == 1.0;
+  // the per-level tree scratch and the node scratch are free once the tree is built
+  MonoLists m{as<uint32_t>(c->mono_words), as<uint32_t>(c->n_tmp), as<uint32_t>(c->tree_cnt),
+              mono_sub(c->n), (uint32_t)(c->n / mono_sub(c->n) + 1)};
   const int lmax = std::min(std::max(c->level_cap, 0), kMaxLevel);   // deeper levels are empty
   stage_mark(c, NG_STAGE_MONOPOLES);
-  if (c->n <= kClusterMaxBodies) {
-    switch (c->p.D) {
-      case 1: k_monopoles_cluster<1><<<kClusterBlocks, kMonoThreads, 0, c->stream>>>(lmax, a); break;
-      case 2: k_monopoles_cluster<2><<<kClusterBlocks, kMonoThreads, 0, c->stream>>>(lmax, a); break;
-      case 3: k_monopoles_cluster<3><<<kClusterBlocks, kMonoThreads, 0, c->stream>>>(lmax, a); break;
-      case 4: k_monopoles_cluster<4><<<kClusterBlocks, kMonoThreads, 0, c->stream>>>(lmax, a); break;
-      case 5: k_monopoles_cluster<5><<<kClusterBlocks, kMonoThreads, 0, c->stream>>>(lmax, a); break;
-      default: k_monopoles_cluster<6><<<kClusterBlocks, kMonoThreads, 0, c->stream>>>(lmax, a); break;
-    }
-    c->launches += 1;
-    NG_CUDA(c, cudaGetLastError());
-    return NG_OK;
-  }
-  if (c->n < kBinnedMonoBodies) {
-    c->launches += lmax + 1;
-    for (int l = lmax; l >= 0; --l) {
-      const int64_t nodes = std::min<int64_t>(c->cap_nodes, level_bound(l, c->n));
-      const int grid = (int)std::max<int64_t>(
-          1, std::min<int64_t>((int64_t)c->nsm * 16, (nodes + kMonoThreads - 1) / kMonoThreads));
-      switch (c->p.D) {
-        case 1: k_monopoles<1><<<grid, kMonoThreads, 0, c->stream>>>(l, a); break;
-        case 2: k_monopoles<2><<<grid, kMonoThreads, 0, c->stream>>>(l, a); break;
-        case 3: k_monopoles<3><<<grid, kMonoThreads, 0, c->stream>>>(l, a); break;
-        case 4: k_monopoles<4><<<grid, kMonoThreads, 0, c->stream>>>(l, a); break;
-        case 5: k_monopoles<5><<<grid, kMonoThreads, 0, c->stream>>>(l, a); break;
-        default: k_monopoles<6><<<grid, kMonoThreads, 0, c->stream>>>(l, a); break;
-      }
-    }
-    NG_CUDA(c, cudaGetLastError());
-    return NG_OK;
-  }
-  // the tree build's per-level scratch (n_tmp, one word per node) is free
-  // once the tree is built: it holds the binned node order
-  uint32_t* bins = as<uint32_t>(c->mono_bins);
-  uint32_t* order = as<uint32_t>(c->n_tmp);
-  NG_CUDA(c, cudaMemsetAsync(bins, 0, 2 * kMonoBins * sizeof(uint32_t), c->stream));
-  const int sgrid = work_grid(c, c->cap_nodes, 4);
-  k_mono_hist<<<sgrid, 256, 0, c->stream>>>(a.status, a.cap, a.level, a.nchild, a.count, bins);
-  k_mono_order<<<sgrid, 256, 0, c->stream>>>(a.status, a.cap, a.level, a.nchild, a.count, bins, order);
-  const int lgrid = (int)std::max<int64_t>(
-      1, std::min<int64_t>((int64_t)c->nsm * 16, (c->cap_nodes + kMonoThreads - 1) / kMonoThreads));
   switch (c->p.D) {
-    case 1: k_mono_leaves<1><<<lgrid, kMonoThreads, 0, c->stream>>>(a, bins, order); break;
-    case 2: k_mono_leaves<2><<<lgrid, kMonoThreads, 0, c->stream>>>(a, bins, order); break;
-    case 3: k_mono_leaves<3><<<lgrid, kMonoThreads, 0, c->stream>>>(a, bins, order); break;
-    case 4: k_mono_leaves<4><<<lgrid, kMonoThreads, 0, c->stream>>>(a, bins, order); break;
-    case 5: k_mono_leaves<5><<<lgrid, kMonoThreads, 0, c->stream>>>(a, bins, order); break;
-    default: k_mono_leaves<6><<<lgrid, kMonoThreads, 0, c->stream>>>(a, bins, order); break;
+    case 1: return launch_monopoles<1>(c, a, m, lmax);
+    case 2: return launch_monopoles<2>(c, a, m, lmax);
+    case 3: return launch_monopoles<3>(c, a, m, lmax);
+    case 4: return launch_monopoles<4>(c, a, m, lmax);
+    case 5: return launch_monopoles<5>(c, a, m, lmax);
+    default: return launch_monopoles<6>(c, a, m, lmax);
   }
-  // nodes at level lmax are leaves
-  c->launches += 3 + lmax;
-  for (int l = lmax - 1; l >= 0; --l) {
-    const int64_t nodes = std::min<int64_t>(c->cap_nodes, level_bound(l, c->n));
-    const int grid = (int)std::max<int64_t>(
-        1, std::min<int64_t>((int64_t)c->nsm * 16, (nodes + kMonoThreads - 1) / kMonoThreads));
-    switch (c->p.D) {
-      case 1: k_mono_internal<1><<<grid, kMonoThreads, 0, c->stream>>>(l, a, bins, order); break;
-      case 2: k_mono_internal<2><<<grid, kMonoThreads, 0, c->stream>>>(l, a, bins, order); break;
-      case 3: k_mono_internal<3><<<grid, kMonoThreads, 0, c->stream>>>(l, a, bins, order); break;
-      case 4: k_mono_internal<4><<<grid, kMonoThreads, 0, c->stream>>>(l, a, bins, order); break;
-      case 5: k_mono_internal<5><<<grid, kMonoThreads, 0, c->stream>>>(l, a, bins, order); break;
-      default: k_mono_internal<6><<<grid, kMonoThreads, 0, c->stream>>>(l, a, bins, order); break;
-    }
-  }
-  NG_CUDA(c, cudaGetLastError());
-  return NG_OK;
 }
 
 // ------------------------------------------------------------- groups
