@@ -295,6 +295,7 @@ int alloc_nodes(ng_ctx* c, int64_t cap) {
   NG_TRY(ensure(c, c->n_link, cap * 16));
   NG_TRY(ensure(c, c->n_mono, cap * D * 16));
   NG_TRY(ensure(c, c->mono_words, (kMonoWords + 3 * kMonoBins + 1) * sizeof(uint32_t)));
+  if (c->p.pure_tree) NG_TRY(ensure(c, c->exact_node, cap * (2 * D + 1) * 16));
   c->cap_nodes = cap;
   (void)node_bytes;
   return NG_OK;
@@ -305,6 +306,7 @@ int alloc_bodies(ng_ctx* c, int64_t n) {
   NG_TRY(ensure(c, c->bleaf, n * 4));
   NG_TRY(ensure(c, c->groups, n * 8));
   NG_TRY(ensure(c, c->tree_cnt, tree_scratch_bytes(n)));
+  if (c->p.pure_tree) NG_TRY(ensure(c, c->exact_body, n * 32));
   NG_TRY(ensure(c, c->status, ST_COUNT * 4));
   NG_TRY(ensure(c, c->counter, 8));
   return NG_OK;
@@ -796,7 +798,7 @@ int ng_destroy(ng_ctx* c) {
                     &c->spos, &c->smass, &c->stype, &c->body, &c->bleaf,
                     &c->tperm, &c->scan_part, &c->n_level, &c->n_prefix, &c->n_first,
                     &c->n_count, &c->n_child, &c->n_nchild, &c->n_tmp, &c->n_m64,
-                    &c->n_cnt, &c->n_geo, &c->n_com, &c->n_link, &c->n_mono, &c->mono_words,
+                    &c->n_cnt, &c->n_geo, &c->n_com, &c->n_link, &c->n_mono, &c->exact_node, &c->exact_body, &c->mono_words,
                     &c->tree_cnt, &c->groups, &c->gsize, &c->grank,
                     &c->status, &c->counter, &c->aold, &c->io_pos, &c->io_vel, &c->io_type, &c->io_mass,
                     &c->io_acc, &c->lattice, &c->rho, &c->rhok, &c->phi,

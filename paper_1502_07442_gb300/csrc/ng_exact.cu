@@ -3,11 +3,12 @@
 // force depends on the number N_perp of bodies behind a monopole and on the
 // passive mass, so it cannot be read from a table of separations.
 //
-// One thread per sorted body walks the tree with the criterion of the
+// One warp per sorted body walks the tree with the criterion of the
 // per-particle count (geometric or relative, decisions in FP64 as there),
-// and evaluates every accepted species monopole and every body of an opened
-// leaf with the pair's law in FP32 (FP64 offsets rounded once to FP32; the
-// cut-off decided in FP64):
+// a node per lane, and evaluates every accepted species monopole and every
+// body of an opened leaf, a term per lane, with the pair's law in FP32
+// (offsets of positions held as two floats each, rounded to FP32 as the FP64
+// difference would be; the cut-off decided as in FP64):
 //   Newton         f = 1
 //   Yukawa (C=1)   f = 1 + a (1 + r/l) e^{-r/l}
 //   pure Yukawa    f = a (1 + r/l) e^{-r/l}
@@ -30,14 +31,16 @@ namespace ng {
 namespace {
 
 struct ExactArgs {
-  const uint8_t* level;
-  const uint64_t* prefix;
-  const uint32_t* first;
-  const uint32_t* count;
-  const uint8_t* nchild;
-  const uint32_t* child;
+  const float4* geo;       // [node] centre, half side (box units, exact in FP32)
+  const int4* link;        // [node] child_first, nchild, body_first, body_count
   const double* m64;       // [node][D][4]: M, sum m x, sum m y, sum m z (box units)
   const uint32_t* cnt;     // [node][D]: N_perp
+  // positions in box units as two floats, x = hi + lo to 2^-49: bodies
+  // {hi, m}, {lo, species}; node species {com hi, M}, {com lo, N_perp}; and the
+  // centre of mass of all species of a node, hi only
+  float4* brec;            // [body][2]
+  float4* nrec;            // [node][D][2]
+  float4* arec;            // [node]
   const double* spos;      // [3][n] sorted, physical
   const float* smass;      // [n] sorted
   const uint8_t* stype;    // [n] sorted
@@ -66,23 +69,19 @@ struct ExactArgs {
   int accumulate;
   unsigned long long* counter;   // executed terms (optional)
   uint32_t* status;
+  bool unit;               // L == 1
+  float Lh, Ll;            // L = Lh + Ll
+  float theta32, eps2f;
+  float cut_lo2, cut_hi2;  // node cut-off^2 (box units) less and plus the FP32 margin
+  float rc2f;              // rcut2, for the terms' FP32 decision
 };
 
-constexpr int kExactStack = 192;
-
-// One term: passive species s of mass mp, active species t of mass M behind
-// which stand np bodies, offset d (physical, source - target). The cut-off
-// rho < r_cut is decided in FP64 with the oracle's operation order; the law
-// is evaluated in FP32.
+// One term within the cut-off: passive species s of mass mp, active species t
+// of mass M behind which stand np bodies, offset (physical, source - target)
+// and softened separation^2 q; the law is evaluated in FP32.
 __device__ __forceinline__ void exact_term(const ExactArgs& a, int s, int t, float M, float np,
-                                           float mp, const double d[3], float& ax, float& ay,
-                                           float& az) {
-  const double r2 = __dadd_rn(__dadd_rn(__dmul_rn(d[0], d[0]), __dmul_rn(d[1], d[1])),
-                              __dmul_rn(d[2], d[2]));
-  const double q64 = __dadd_rn(r2, a.eps2);
-  if (!(q64 < a.rcut2)) return;
-  const float dx = (float)d[0], dy = (float)d[1], dz = (float)d[2];
-  const float q = (float)q64;
+                                           float mp, float dx, float dy, float dz, float q, float& ax,
+                                           float& ay, float& az) {
   const float rho = sqrtf(q);
   float f;
   const int kind = a.kind[s][t];
@@ -134,122 +133,323 @@ __device__ __forceinline__ void exact_term(const ExactArgs& a, int s, int t, flo
   }
 }
 
-__global__ void __launch_bounds__(128) k_walk_exact(ExactArgs a) {
+// hi + lo of a position (box units)
+__device__ __forceinline__ void split(double p, float* hi, float* lo) {
+  *hi = (float)p;
+  *lo = (float)(p - (double)*hi);
+}
+
+// The two-float records of every body and node.
+__global__ void k_exact_prep(ExactArgs a) {
   if (a.status[ST_FLAGS] & SF_NODE_OVERFLOW) return;
-  unsigned long long mine = 0;
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < a.n;
-       k += (int64_t)gridDim.x * blockDim.x) {
-    const double x[3] = {a.spos[k] * a.invL, a.spos[a.n + k] * a.invL,
-                         a.spos[2 * a.n + k] * a.invL};
-    const int s = a.stype[k];
-    const float mp = a.smass[k];
-    float ax = 0.f, ay = 0.f, az = 0.f;
-    uint32_t stack[kExactStack];
-    int sp = 0;
-    stack[sp++] = 0;
-    long long cnt = 0;
-    uint32_t visits = 0;
-    const uint32_t nnodes = a.status[ST_LEVELS + kMaxLevel + 1];
-    while (sp > 0) {
-      if (++visits > nnodes) {
-        atomicOr(&a.status[ST_FLAGS], (uint32_t)SF_BAD_TREE);
-        break;
-      }
-      const uint32_t nd = stack[--sp];
-      const uint64_t pre = a.prefix[nd];
-      double c[3], side;
-      node_centre(a.level[nd], pre, c, &side);
-      const double half = __dmul_rn(0.5, side);
-      double g2 = 0.0, dcs[3];
-      bool inside = true;
-#pragma unroll
+  const int64_t t0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t b = t0; b < a.n; b += stride) {
+    float h[3], l[3];
+    for (int e = 0; e < 3; ++e) split(a.spos[e * a.n + b] * a.invL, &h[e], &l[e]);
+    a.brec[2 * b] = make_float4(h[0], h[1], h[2], a.smass[b]);
+    a.brec[2 * b + 1] = make_float4(l[0], l[1], l[2], __int_as_float((int)a.stype[b]));
+  }
+  const uint32_t total = a.status[ST_LEVELS + kMaxLevel + 1];
+  for (int64_t k = t0; k < (int64_t)total; k += stride) {
+    double mt = 0.0, st[3] = {0.0, 0.0, 0.0};
+    for (int t = 0; t < a.D; ++t) {
+      const size_t r = (size_t)k * a.D + t;
+      const double* m = a.m64 + r * 4;
+      float h[3] = {0.f, 0.f, 0.f}, l[3] = {0.f, 0.f, 0.f};
+      mt += m[0];
       for (int e = 0; e < 3; ++e) {
-        const double dc = nearest_image_unit(__dsub_rn(c[e], x[e]));
-        dcs[e] = dc;
-        double gap = __dsub_rn(fabs(dc), half);
-        gap = gap > 0.0 ? gap : 0.0;
-        g2 = __dadd_rn(g2, __dmul_rn(gap, gap));
-        if (fabs(dc) > half) inside = false;
+        st[e] += m[1 + e];
+        if (m[0] > 0.0) split(m[1 + e] / m[0], &h[e], &l[e]);
       }
-      if (g2 >= a.rcut2_box) continue;
-      const uint32_t nch = a.nchild[nd];
-      if (!inside) {
-        double mt = 0.0, sx = 0.0, sy = 0.0, sz = 0.0;
-        for (int t = 0; t < a.D; ++t) {
-          const double* m = a.m64 + ((size_t)nd * a.D + t) * 4;
-          mt += m[0];
-          sx += m[1];
-          sy += m[2];
-          sz += m[3];
-        }
-        const double com[3] = {sx / mt, sy / mt, sz / mt};
-        double dd2 = 0.0;
+      // (a positive mass that is zero in FP32 still is a term)
+      const float M = m[0] > 0.0 ? (float)m[0] : -1.f;
+      a.nrec[2 * r] = make_float4(h[0], h[1], h[2], M);
+      a.nrec[2 * r + 1] = make_float4(l[0], l[1], l[2], (float)a.cnt[r]);
+    }
+    a.arec[k] = make_float4((float)(st[0] / mt), (float)(st[1] / mt), (float)(st[2] / mt), 0.f);
+  }
+}
+
+// FP32 offset wrapped to the nearest image (|d| < 1; exact)
+__device__ __forceinline__ float image32(float d) { return fabsf(d) > 0.5f ? d - copysignf(1.f, d) : d; }
+
+// Whether the per-particle walk accepts node nd for the body at x, decided in
+// FP64 as the count decides: 0 beyond the cut-off, 1 accepted, 2 opened.
+__device__ __noinline__ int exact_decide64(const ExactArgs& a, uint32_t nd, int64_t k) {
+  const double x[3] = {a.spos[k] * a.invL, a.spos[a.n + k] * a.invL, a.spos[2 * a.n + k] * a.invL};
+  const float4 ge = a.geo[nd];
+  const double c[3] = {(double)ge.x, (double)ge.y, (double)ge.z};
+  const double half = (double)ge.w, side = 2.0 * half;
+  double g2 = 0.0, dcs[3];
+  bool inside = true;
 #pragma unroll
-        for (int e = 0; e < 3; ++e) {
-          const double v = nearest_image_unit(__dsub_rn(com[e], x[e]));
-          dd2 = __dadd_rn(dd2, __dmul_rn(v, v));
-        }
-        bool accept;
-        if (a.relative) {
-          const double lim = __dmul_rn(0.6, side);
-          bool near = true;
+  for (int e = 0; e < 3; ++e) {
+    const double dc = nearest_image_unit(__dsub_rn(c[e], x[e]));
+    dcs[e] = dc;
+    double gap = __dsub_rn(fabs(dc), half);
+    gap = gap > 0.0 ? gap : 0.0;
+    g2 = __dadd_rn(g2, __dmul_rn(gap, gap));
+    if (fabs(dc) > half) inside = false;
+  }
+  if (g2 >= a.rcut2_box) return 0;
+  if (inside) return 2;
+  double mt = 0.0, sx = 0.0, sy = 0.0, sz = 0.0;
+  for (int t = 0; t < a.D; ++t) {
+    const double* m = a.m64 + ((size_t)nd * a.D + t) * 4;
+    mt += m[0];
+    sx += m[1];
+    sy += m[2];
+    sz += m[3];
+  }
+  const double com[3] = {sx / mt, sy / mt, sz / mt};
+  double dd2 = 0.0;
 #pragma unroll
-          for (int e = 0; e < 3; ++e)
-            if (!(fabs(dcs[e]) < lim)) near = false;
-          const double lhs = __dmul_rn(__dmul_rn(a.gmax, mt), __dmul_rn(side, side));
-          const double rhs = __dmul_rn(__dmul_rn(a.alphaL2, (double)a.aold[a.perm[k]]),
-                                       __dmul_rn(dd2, dd2));
-          accept = !near && lhs <= rhs;
-        } else {
-          accept = side < __dmul_rn(a.theta, sqrt(dd2));
+  for (int e = 0; e < 3; ++e) {
+    const double v = nearest_image_unit(__dsub_rn(com[e], x[e]));
+    dd2 = __dadd_rn(dd2, __dmul_rn(v, v));
+  }
+  if (a.relative) {
+    const double lim = __dmul_rn(0.6, side);
+    bool near = true;
+#pragma unroll
+    for (int e = 0; e < 3; ++e)
+      if (!(fabs(dcs[e]) < lim)) near = false;
+    const double lhs = __dmul_rn(__dmul_rn(a.gmax, mt), __dmul_rn(side, side));
+    const double rhs = __dmul_rn(__dmul_rn(a.alphaL2, (double)a.aold[a.perm[k]]), __dmul_rn(dd2, dd2));
+    return !near && lhs <= rhs ? 1 : 2;
+  }
+  return side < __dmul_rn(a.theta, sqrt(dd2)) ? 1 : 2;
+}
+
+// The same in FP32 where it is certain, else -1 (geometric criterion). Error
+// bounds, box units (coordinates below 1): a node centre is exact, x and the
+// centre of mass are rounded by 2^-25, a difference by 2^-25 more, so that gaps
+// and |offsets| per axis are known to 1e-7, distances to 2e-7 and to a few
+// 2^-24 of themselves; the margins are at least twice that.
+__device__ __forceinline__ int exact_decide32(const ExactArgs& a, const float4 ge, const float4 cm,
+                                              const float xh[3]) {
+  const float gx = fabsf(image32(ge.x - xh[0])) - ge.w, gy = fabsf(image32(ge.y - xh[1])) - ge.w,
+              gz = fabsf(image32(ge.z - xh[2])) - ge.w;
+  const float far = fmaxf(gx, fmaxf(gy, gz));
+  const float px = fmaxf(gx, 0.f), py = fmaxf(gy, 0.f), pz = fmaxf(gz, 0.f);
+  const float g2 = fmaf(px, px, fmaf(py, py, pz * pz));
+  if (g2 > a.cut_hi2) return 0;
+  if (!(g2 < a.cut_lo2)) return -1;
+  if (far < -4e-7f) return 2;          // inside the cube
+  if (!(far > 4e-7f)) return -1;
+  const float ex = image32(cm.x - xh[0]), ey = image32(cm.y - xh[1]), ez = image32(cm.z - xh[2]);
+  const float d = sqrtf(fmaf(ex, ex, fmaf(ey, ey, ez * ez)));
+  const float m = fmaf(2e-6f, d, 6e-7f), side = 2.f * ge.w;
+  if (side < a.theta32 * (d - m) * 0.999999f) return 1;
+  if (side > a.theta32 * (d + m) * 1.000001f) return 2;
+  return -1;
+}
+
+// Whether a term at q64 = |d|^2 + eps^2 (FP64, the count's operation order)
+// lies within the cut-off: for the terms FP32 cannot tell.
+__device__ __noinline__ bool exact_within64(const ExactArgs& a, const double p[3], int64_t k) {
+  double d[3];
+#pragma unroll
+  for (int e = 0; e < 3; ++e)
+    d[e] = nearest_image_unit(__dsub_rn(p[e], a.spos[e * a.n + k] * a.invL)) * a.L;
+  const double r2 = __dadd_rn(__dadd_rn(__dmul_rn(d[0], d[0]), __dmul_rn(d[1], d[1])),
+                              __dmul_rn(d[2], d[2]));
+  return __dadd_rn(r2, a.eps2) < a.rcut2;
+}
+
+// Offset of two-float position (ph, pl) from (xh, xl): the difference of the
+// high parts with its rounding error (Knuth's two-sum), wrapped exactly, plus
+// the low parts; times L. One rounding, up to terms of 2^-48.
+__device__ __forceinline__ float exact_offset(const ExactArgs& a, float ph, float pl, float xh, float xl) {
+  const float s = __fsub_rn(ph, xh);
+  const float bb = __fsub_rn(s, ph);
+  const float err = __fsub_rn(__fsub_rn(ph, __fsub_rn(s, bb)), __fadd_rn(xh, bb));
+  const float w = image32(s), low = __fadd_rn(err, __fsub_rn(pl, xl));
+  return a.unit ? __fadd_rn(w, low) : fmaf(w, a.Lh, fmaf(w, a.Ll, low * a.Lh));
+}
+
+constexpr int kExactWarps = 4;
+
+struct ExactWarp {
+  uint32_t stack[kStackCap];
+  uint32_t node[32];      // accepted nodes of the round
+  uint32_t lfirst[32];    // opened leaves of the round: first body
+  uint32_t loff[32];      // and exclusive prefix of body counts
+};
+
+// One warp per body. A thread per body left the threads of a warp on
+// different nodes and leaves, and few warps in flight (30k bodies: 940); here
+// the lanes of a warp take 32 nodes of the body's stack at a time, then the
+// terms these rounds accept and open, 32 at a time. In FP64 (1/64 of the FP32
+// rate) the decisions and offsets kept that pipe 85 % busy; they are now made
+// in FP32 with error bounds, in FP64 only where FP32 cannot tell, with the same
+// outcome. 30011 bodies, two species, leaf 8: 11.4 ms with a thread per body,
+// 3.4 ms with a warp per body in FP64, 0.52 ms now. The terms and their number
+// are those of the per-particle count; each lane sums its terms in FP32, the
+// lanes' sums are added at the end.
+__global__ void __launch_bounds__(32 * kExactWarps, 8) k_walk_exact(ExactArgs a) {
+  __shared__ ExactWarp sm[kExactWarps];
+  if (a.status[ST_FLAGS] & SF_NODE_OVERFLOW) return;
+  ExactWarp& ws = sm[threadIdx.x >> 5];
+  const int lane = threadIdx.x & 31;
+  const uint32_t lt = (1u << lane) - 1u;
+  const uint32_t nnodes = a.status[ST_LEVELS + kMaxLevel + 1];
+  unsigned long long mine = 0;
+  for (int64_t k = (int64_t)blockIdx.x * kExactWarps + (threadIdx.x >> 5); k < a.n;
+       k += (int64_t)gridDim.x * kExactWarps) {
+    const float4 bh = a.brec[2 * k], bl = a.brec[2 * k + 1];
+    const float xh[3] = {bh.x, bh.y, bh.z};
+    const int s = __float_as_int(bl.w);
+    const float mp = bh.w;
+    float ax = 0.f, ay = 0.f, az = 0.f;
+    uint32_t terms = 0;
+    if (lane == 0) ws.stack[0] = 0;
+    int size = 1;
+    uint32_t visits = 0;
+    uint32_t bad = 0;
+    __syncwarp();
+    while (size > 0) {
+      // the stack of the group walk: up to 32 nodes from the top; opened
+      // nodes whose children do not fit are pushed back (see k_walk)
+      if (size + 7 > kStackCap) { bad = SF_STACK_OVERFLOW; break; }
+      if (visits > nnodes) { bad = SF_BAD_TREE; break; }
+      int kk = min(32, size);
+      int avail = (kStackCap - kStackReserve) - (size - kk);
+      if (avail < 8) {
+        kk = 1;
+        avail = kStackCap - (size - 1);
+      }
+      visits += kk;
+      const bool has = lane < kk;
+      const uint32_t nd = has ? ws.stack[size - kk + lane] : 0u;
+      size -= kk;
+      __syncwarp();
+      int cls = 0;   // 0 skip, 1 accept, 2 leaf, 3 open
+      int4 lk = make_int4(0, 0, 0, 0);
+      if (has) {
+        const float4 ge = a.geo[nd];
+        const float4 cm = a.arec[nd];
+        lk = a.link[nd];
+        int r = a.relative ? -1 : exact_decide32(a, ge, cm, xh);
+        if (r < 0) r = exact_decide64(a, nd, k);
+        cls = r == 2 ? (lk.y == 0 ? 2 : 3) : r;
+      }
+      const uint32_t nch = (uint32_t)lk.y;
+      // opened nodes: children onto the stack
+      {
+        const uint32_t mych = cls == 3 ? nch : 0u;
+        uint32_t incl = mych;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
+          if (lane >= o) incl += t;
         }
-        if (accept) {
-          for (int t = 0; t < a.D; ++t) {
-            const double* m = a.m64 + ((size_t)nd * a.D + t) * 4;
-            if (!(m[0] > 0.0)) continue;
-            const double d[3] = {nearest_image_unit(__dsub_rn(m[1] / m[0], x[0])) * a.L,
-                                 nearest_image_unit(__dsub_rn(m[2] / m[0], x[1])) * a.L,
-                                 nearest_image_unit(__dsub_rn(m[3] / m[0], x[2])) * a.L};
-            exact_term(a, s, t, (float)m[0], (float)a.cnt[(size_t)nd * a.D + t], mp, d, ax, ay,
-                       az);
-            ++cnt;
+        const bool fit = (int)incl <= avail;
+        const uint32_t back = __ballot_sync(0xffffffffu, cls == 3 && !fit);
+        const int used = (int)__reduce_max_sync(0xffffffffu, fit ? incl : 0u);
+        if (cls == 3) {
+          if (fit) {
+            const uint32_t c0 = (uint32_t)lk.x;
+            for (uint32_t j = 0; j < nch; ++j) ws.stack[size + (int)(incl - mych + j)] = c0 + j;
+          } else {
+            ws.stack[size + used + __popc(back & lt)] = nd;
           }
-          continue;
+        }
+        size += used + __popc(back);
+        visits -= __popc(back);
+      }
+      // accepted nodes: a term per species with mass
+      const uint32_t acc = __ballot_sync(0xffffffffu, cls == 1);
+      if (cls == 1) ws.node[__popc(acc & lt)] = nd;
+      // opened leaves: their bodies
+      const uint32_t lm = __ballot_sync(0xffffffffu, cls == 2);
+      uint32_t bodies = 0;
+      if (lm) {
+        const uint32_t nb = cls == 2 ? (uint32_t)lk.w : 0u;
+        uint32_t incl = nb;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
+          if (lane >= o) incl += t;
+        }
+        bodies = __shfl_sync(0xffffffffu, incl, 31);
+        if (cls == 2) {
+          const int at = __popc(lm & lt);
+          ws.lfirst[at] = (uint32_t)lk.z;
+          ws.loff[at] = incl - nb;
         }
       }
-      if (nch == 0) {
-        const uint32_t f = a.first[nd], c2 = a.count[nd];
-        for (uint32_t b = f; b < f + c2; ++b) {
-          if ((int64_t)b == k) continue;
-          const double d[3] = {nearest_image_unit(__dsub_rn(a.spos[b] * a.invL, x[0])) * a.L,
-                               nearest_image_unit(__dsub_rn(a.spos[a.n + b] * a.invL, x[1])) * a.L,
-                               nearest_image_unit(__dsub_rn(a.spos[2 * a.n + b] * a.invL, x[2])) * a.L};
-          exact_term(a, s, a.stype[b], a.smass[b], 1.f, mp, d, ax, ay, az);
-          ++cnt;
+      __syncwarp();
+      // monopole terms, then body terms, in one run of lanes
+      const uint32_t monos = (uint32_t)__popc(acc) * (uint32_t)a.D;
+      const int nl = __popc(lm);
+      for (uint32_t f = lane; f < monos + bodies; f += 32) {
+        float4 ph, pl;
+        float np = 1.f;
+        int t;
+        uint32_t src;   // node species record, or body
+        const bool mono = f < monos;
+        if (mono) {
+          const uint32_t i = f / (uint32_t)a.D;
+          t = (int)(f - i * (uint32_t)a.D);
+          src = ws.node[i] * (uint32_t)a.D + (uint32_t)t;
+          ph = a.nrec[2 * (size_t)src];
+          if (ph.w < 0.f) continue;   // no mass of this species
+          pl = a.nrec[2 * (size_t)src + 1];
+          np = pl.w;
+        } else {
+          const uint32_t h = f - monos;
+          int lo = 0, hi = nl - 1;   // the last leaf that starts at or before h
+          while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (ws.loff[mid] <= h) lo = mid; else hi = mid - 1;
+          }
+          src = ws.lfirst[lo] + (h - ws.loff[lo]);
+          if ((int64_t)src == k) continue;
+          ph = a.brec[2 * (size_t)src];
+          pl = a.brec[2 * (size_t)src + 1];
+          t = __float_as_int(pl.w);
         }
-      } else {
-        if (sp + (int)nch > kExactStack) {
-          atomicOr(&a.status[ST_FLAGS], (uint32_t)SF_STACK_OVERFLOW);
-          break;
+        const float dx = exact_offset(a, ph.x, pl.x, xh[0], bl.x);
+        const float dy = exact_offset(a, ph.y, pl.y, xh[1], bl.y);
+        const float dz = exact_offset(a, ph.z, pl.z, xh[2], bl.z);
+        const float q = fmaf(dx, dx, fmaf(dy, dy, fmaf(dz, dz, a.eps2f)));
+        // q is within 4e-7 of its FP64 value
+        bool within = q < a.rc2f;
+        if (fabsf(q - a.rc2f) <= 2e-6f * a.rc2f && a.rc2f < 3.0e38f) {
+          double p[3];
+#pragma unroll
+          for (int e = 0; e < 3; ++e) {
+            const double* m = a.m64 + (size_t)src * 4;
+            p[e] = mono ? m[1 + e] / m[0] : a.spos[e * a.n + src] * a.invL;
+          }
+          within = exact_within64(a, p, k);
         }
-        for (int ch = (int)nch - 1; ch >= 0; --ch) stack[sp++] = a.child[nd] + ch;
+        if (within) exact_term(a, s, t, ph.w, np, mp, dx, dy, dz, q, ax, ay, az);
+        ++terms;
       }
+      __syncwarp();
     }
-    const uint32_t i = a.out ? a.out[k] : (uint32_t)k;
-    if (a.accumulate) {
-      a.acc[i] += ax;
-      a.acc[a.n + i] += ay;
-      a.acc[2 * a.n + i] += az;
-    } else {
-      a.acc[i] = ax;
-      a.acc[a.n + i] = ay;
-      a.acc[2 * a.n + i] = az;
+    if (bad && lane == 0) atomicOr(&a.status[ST_FLAGS], bad);
+    __syncwarp();
+#pragma unroll
+    for (int o = 16; o; o >>= 1) {
+      ax += __shfl_xor_sync(0xffffffffu, ax, o);
+      ay += __shfl_xor_sync(0xffffffffu, ay, o);
+      az += __shfl_xor_sync(0xffffffffu, az, o);
     }
-    mine += (unsigned long long)cnt;
+    mine += terms;
+    if (lane < 3) {
+      const uint32_t i = a.out ? a.out[k] : (uint32_t)k;
+      const float v = lane == 0 ? ax : lane == 1 ? ay : az;
+      float* o = a.acc + (size_t)lane * a.n + i;
+      *o = a.accumulate ? *o + v : v;
+    }
   }
   if (a.counter) {
     for (int o = 16; o; o >>= 1) mine += __shfl_xor_sync(0xffffffffu, mine, o);
-    if ((threadIdx.x & 31) == 0 && mine) atomicAdd(a.counter, mine);
+    if (lane == 0 && mine) atomicAdd(a.counter, mine);
   }
 }
 
@@ -257,13 +457,12 @@ __global__ void __launch_bounds__(128) k_walk_exact(ExactArgs a) {
 
 int launch_walk_exact(ng_ctx* c, float* acc, bool accumulate, bool count) {
   ExactArgs a{};
-  a.level = as<uint8_t>(c->n_level);
-  a.prefix = as<uint64_t>(c->n_prefix);
-  a.first = as<uint32_t>(c->n_first);
-  a.count = as<uint32_t>(c->n_count);
-  a.nchild = as<uint8_t>(c->n_nchild);
-  a.child = as<uint32_t>(c->n_child);
+  a.geo = as<float4>(c->n_geo);
+  a.link = as<int4>(c->n_link);
   a.m64 = as<double>(c->n_m64);
+  a.brec = as<float4>(c->exact_body);
+  a.nrec = as<float4>(c->exact_node);
+  a.arec = a.nrec + (size_t)c->cap_nodes * c->p.D * 2;
   a.cnt = as<uint32_t>(c->n_cnt);
   a.spos = as<double>(c->spos);
   a.smass = as<float>(c->smass);
@@ -305,9 +504,20 @@ int launch_walk_exact(ng_ctx* c, float* acc, bool accumulate, bool count) {
   a.accumulate = accumulate ? 1 : 0;
   a.counter = count ? as<unsigned long long>(c->counter) : nullptr;
   a.status = as<uint32_t>(c->status);
-  const int blocks = (int)std::min<int64_t>((c->n + 127) / 128, (int64_t)c->nsm * 16);
-  k_walk_exact<<<blocks, 128, 0, c->stream>>>(a);
-  c->launches += 1;
+  a.unit = c->L == 1.0;
+  a.Lh = (float)c->L;
+  a.Ll = (float)(c->L - (double)a.Lh);
+  a.theta32 = (float)a.theta;
+  a.eps2f = (float)a.eps2;
+  a.rc2f = (float)a.rcut2;
+  a.cut_lo2 = (float)((rc - 2e-6) * (rc - 2e-6) * 0.999999);
+  a.cut_hi2 = (float)((rc + 2e-6) * (rc + 2e-6) * 1.000001);
+  if (!(rc > 4e-6)) a.cut_lo2 = -1.f;   // a cut-off near the margin: always in FP64
+  k_exact_prep<<<work_grid(c, c->n, 8), 256, 0, c->stream>>>(a);
+  // one warp a body, eight blocks per SM resident; bodies are taken in turns
+  const int64_t blocks = (c->n + kExactWarps - 1) / kExactWarps;
+  k_walk_exact<<<(int)std::min<int64_t>(blocks, (int64_t)c->nsm * 64), 32 * kExactWarps, 0, c->stream>>>(a);
+  c->launches += 2;
   NG_CUDA(c, cudaGetLastError());
   return NG_OK;
 }

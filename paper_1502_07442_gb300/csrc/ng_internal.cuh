@@ -285,6 +285,7 @@ struct ng_ctx {
   int64_t ngroups = 0, ngroups_n = -1;   // walk groups of the last checked build, for n = ngroups_n
   ng::DevBuf n_level, n_prefix, n_first, n_count, n_child, n_nchild, n_tmp;
   ng::DevBuf n_m64, n_cnt, n_geo, n_com, n_link, n_mono;
+  ng::DevBuf exact_node, exact_body;   // two-float positions of pure tree mode (ng_exact.cu)
   ng::DevBuf mono_words;   // uint32[kMonoWords + 3 kMonoBins + 1]: counters and bins of the monopole stage
   ng::DevBuf tree_cnt;    // uint32[levels][tiles]: node counts of the tree build
   ng::DevBuf groups;

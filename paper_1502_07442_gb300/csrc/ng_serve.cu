@@ -70,8 +70,9 @@ struct Req {
 // buffers for a capacity of `nodes` nodes, PM meshes.
 size_t request_bytes_nodes(const ng_request& q, size_t nodes) {
   const size_t n = (size_t)q.n, D = (size_t)q.params.D, N = (size_t)q.params.pm_mesh;
-  const size_t body = 53 + 100;
-  const size_t node = 74 + 52 * D;
+  const bool pure = q.params.pure_tree != 0;
+  const size_t body = 53 + 100 + (pure ? 32 : 0);
+  const size_t node = 74 + 52 * D + (pure ? 16 * (2 * D + 1) : 0);
   const size_t pm = N ? D * N * N * (N + 2) * 4 * 2 + D * N * N * N * 4 : 0;
   return n * body + nodes * node + pm + (1 << 20);
 }
