@@ -500,22 +500,35 @@ static int64_t to_tiles(int64_t n) { return (n + kToTile - 1) / kToTile; }
 
 // -------------------------------------------------------------- gather
 
-__global__ void k_gather(int64_t n, const uint32_t* __restrict__ perm,
-                         const double* __restrict__ pos, const uint8_t* __restrict__ type,
-                         const float* __restrict__ mass, double L, double invL, bool pow2,
-                         int D, double* __restrict__ spos, float* __restrict__ smass,
-                         uint8_t* __restrict__ stype, uint32_t* status) {
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n;
-       k += (int64_t)gridDim.x * blockDim.x) {
-    const uint32_t i = perm[k];
-    spos[k] = wrap_box(pos[i], L, invL, pow2);
-    spos[n + k] = wrap_box(pos[n + i], L, invL, pow2);
-    spos[2 * n + k] = wrap_box(pos[2 * n + i], L, invL, pow2);
-    smass[k] = mass[i];
-    const uint8_t ti = type[i];
-    if (ti >= D) atomicOr(&status[ST_FLAGS], (uint32_t)SF_BAD_TYPE);
-    stype[k] = ti < D ? ti : 0;    // out-of-range species: flagged, never used as an index
-  }
+struct GatherArgs {
+  int64_t n;
+  // plain: caller arrays, wrapped and checked; resident: the previous state
+  const double* pos;
+  const float* mass;
+  const uint8_t* type;
+  const float* vel;
+  const uint32_t* orig;
+  double* spos;
+  float* smass;
+  uint8_t* stype;
+  float* svel;
+  uint32_t* sorig;
+  double L, invL;
+  bool pow2;
+  int D;
+  uint32_t* status;
+};
+
+// Body i of the input becomes sorted body k.
+__device__ __forceinline__ void gather_plain(const GatherArgs& g, int64_t k, uint32_t i) {
+  const int64_t n = g.n;
+  g.spos[k] = wrap_box(g.pos[i], g.L, g.invL, g.pow2);
+  g.spos[n + k] = wrap_box(g.pos[n + i], g.L, g.invL, g.pow2);
+  g.spos[2 * n + k] = wrap_box(g.pos[2 * n + i], g.L, g.invL, g.pow2);
+  g.smass[k] = g.mass[i];
+  const uint8_t ti = g.type[i];
+  if (ti >= g.D) atomicOr(&g.status[ST_FLAGS], (uint32_t)SF_BAD_TYPE);
+  g.stype[k] = (uint8_t)stored_type(ti, g.D);    // out-of-range species: flagged, never used as an index
 }
 
 // The resident step's gather: the previous state (positions already wrapped
@@ -523,25 +536,186 @@ __global__ void k_gather(int64_t n, const uint32_t* __restrict__ perm,
 // previous step's sorted order) into this step's sorted order. The bodies
 // move little from step to step, so perm is close to the identity and every
 // read is close to sequential.
-__global__ void k_gather_resident(int64_t n, const uint32_t* __restrict__ perm,
-                                  const double* __restrict__ xpos, const float* __restrict__ xmass,
-                                  const uint8_t* __restrict__ xtype, const float* __restrict__ xvel,
-                                  const uint32_t* __restrict__ xorig, double* __restrict__ ypos,
-                                  float* __restrict__ ymass, uint8_t* __restrict__ ytype,
-                                  float* __restrict__ yvel, uint32_t* __restrict__ yorig) {
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n;
+__device__ __forceinline__ void gather_resident(const GatherArgs& g, int64_t k, uint32_t i) {
+  const int64_t n = g.n;
+  g.spos[k] = g.pos[i];
+  g.spos[n + k] = g.pos[n + i];
+  g.spos[2 * n + k] = g.pos[2 * n + i];
+  g.svel[k] = g.vel[i];
+  g.svel[n + k] = g.vel[n + i];
+  g.svel[2 * n + k] = g.vel[2 * n + i];
+  g.smass[k] = g.mass[i];
+  g.stype[k] = g.type[i];
+  g.sorig[k] = g.orig[i];
+}
+
+template <bool RESIDENT>
+__global__ void k_gather(GatherArgs g, const uint32_t* __restrict__ perm) {
+  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < g.n;
        k += (int64_t)gridDim.x * blockDim.x) {
-    const uint32_t i = perm[k];
-    ypos[k] = xpos[i];
-    ypos[n + k] = xpos[n + i];
-    ypos[2 * n + k] = xpos[2 * n + i];
-    yvel[k] = xvel[i];
-    yvel[n + k] = xvel[n + i];
-    yvel[2 * n + k] = xvel[2 * n + i];
-    ymass[k] = xmass[i];
-    ytype[k] = xtype[i];
-    yorig[k] = xorig[i];
+    if (RESIDENT) gather_resident(g, k, perm[k]);
+    else gather_plain(g, k, perm[k]);
   }
+}
+
+// ------------------------------------------------------- small problems
+
+// The whole sort stage of up to 1024 * ITEMS bodies in one launch of one
+// block: keys, the radix passes in shared memory, the gather and the
+// type-major order. At these sizes every launch of the general path costs more
+// than its work (4096 bodies: keys, 8 passes, gather and type order 81 us in 11
+// launches, 46 us here). Bodies past n take the largest key and end last.
+constexpr int kSmThreads = 1024, kSmWarps = kSmThreads / 32;
+constexpr int kSmRow = 257;   // words per warp of digit counts (a bank apart per row)
+constexpr int64_t kSmallSort = 8192;
+
+template <int ITEMS>
+struct SmSmem {
+  uint64_t tk[kSmThreads * ITEMS];
+  uint32_t tv[kSmThreads * ITEMS];
+  uint32_t wcnt[kSmWarps * kSmRow];
+  uint32_t wsum[kSmWarps];
+  uint32_t species[8];
+};
+
+template <int ITEMS, bool RESIDENT>
+__global__ void __launch_bounds__(kSmThreads)
+k_sort_small(KeyArgs a, GatherArgs g, int first, uint64_t* __restrict__ keys,
+             uint32_t* __restrict__ perm, uint32_t* words, uint32_t* __restrict__ tperm) {
+  extern __shared__ __align__(16) unsigned char sm_raw[];
+  SmSmem<ITEMS>& sm = *reinterpret_cast<SmSmem<ITEMS>*>(sm_raw);
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const uint32_t lt = (1u << lane) - 1u;
+  const int i0 = w * (32 * ITEMS) + lane;   // item it of the thread: body i0 + 32 it
+  uint64_t k[ITEMS];
+  uint32_t v[ITEMS], rank[ITEMS];
+#pragma unroll
+  for (int it = 0; it < ITEMS; ++it) {
+    const int i = i0 + it * 32;
+    v[it] = (uint32_t)i;
+    k[it] = i < a.n ? body_key(a, i, a.type[i]) : ~0ull;
+  }
+  for (int p = first; p < 8; ++p) {
+    const int shift = 8 * p;
+    for (int j = tid; j < kSmWarps * kSmRow; j += kSmThreads) sm.wcnt[j] = 0;
+    __syncthreads();
+    uint32_t* cnt = sm.wcnt + w * kSmRow;
+#pragma unroll
+    for (int h = 0; h < ITEMS; h += 4) {
+      uint32_t peers[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) peers[j] = digit_peers((uint32_t)(k[h + j] >> shift) & 0xffu, 0xffffffffu);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const uint32_t d = (uint32_t)(k[h + j] >> shift) & 0xffu;
+        const uint32_t prior = cnt[d];
+        __syncwarp();
+        rank[h + j] = prior + __popc(peers[j] & lt);
+        if ((peers[j] & lt) == 0) cnt[d] = prior + __popc(peers[j]);
+        __syncwarp();
+      }
+    }
+    __syncthreads();
+    {
+      // four threads per digit, eight warps' counts each: the digit's total,
+      // its start (scan over digits) and each warp's place in its run
+      const int d = tid >> 2, seg = tid & 3;
+      uint32_t c[8], sum = 0;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        c[j] = sm.wcnt[(seg * 8 + j) * kSmRow + d];
+        sum += c[j];
+      }
+      uint32_t incl = sum;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += t;
+      }
+      if (lane == 31) sm.wsum[w] = incl;
+      __syncthreads();
+      uint32_t base = sm.wsum[lane];   // exclusive over the warps
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t t = __shfl_up_sync(0xffffffffu, base, o);
+        if (lane >= o) base += t;
+      }
+      base = __shfl_sync(0xffffffffu, base, w) - sm.wsum[w];
+      uint32_t run = base + incl - sum;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        sm.wcnt[(seg * 8 + j) * kSmRow + d] = run;
+        run += c[j];
+      }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int it = 0; it < ITEMS; ++it) {
+      const uint32_t at = cnt[(uint32_t)(k[it] >> shift) & 0xffu] + rank[it];
+      sm.tk[at] = k[it];
+      sm.tv[at] = v[it];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int it = 0; it < ITEMS; ++it) {
+      k[it] = sm.tk[i0 + it * 32];
+      v[it] = sm.tv[i0 + it * 32];
+    }
+  }
+  if (tid < 8) sm.species[tid] = 0;
+  uint32_t* chunk = sm.wcnt;   // [8][32 ITEMS]: bodies per species and chunk, then positions
+  constexpr int kChunks = 32 * ITEMS;
+  __syncthreads();
+  int ty[ITEMS];
+#pragma unroll
+  for (int it = 0; it < ITEMS; ++it) {
+    const int i = i0 + it * 32;
+    ty[it] = -1;
+    if (i < a.n) {
+      keys[i] = k[it];
+      perm[i] = v[it];
+      if (RESIDENT) gather_resident(g, i, v[it]);
+      else gather_plain(g, i, v[it]);
+      ty[it] = (int)stored_type(a.type[v[it]], a.D);
+    }
+    rank[it] = 0;
+    for (int t = 0; t < a.D; ++t) {
+      const uint32_t m = __ballot_sync(0xffffffffu, ty[it] == t);
+      if (ty[it] == t) rank[it] = __popc(m & lt);
+      if (lane == 0) chunk[t * kChunks + w * ITEMS + it] = __popc(m);
+    }
+  }
+  __syncthreads();
+  uint32_t c[ITEMS], incl = 0, sum = 0;
+  if (w < a.D) {   // warp w: species w, chunks in order
+#pragma unroll
+    for (int j = 0; j < ITEMS; ++j) {
+      c[j] = chunk[w * kChunks + lane * ITEMS + j];
+      sum += c[j];
+    }
+    incl = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += t;
+    }
+    if (lane == 31) sm.species[w] = incl;
+  }
+  __syncthreads();
+  if (w < a.D) {
+    uint32_t run = incl - sum;
+    for (int t = 0; t < w; ++t) run += sm.species[t];
+#pragma unroll
+    for (int j = 0; j < ITEMS; ++j) {
+      chunk[w * kChunks + lane * ITEMS + j] = run;
+      run += c[j];
+    }
+  }
+  if (tid < 8) words[kSwTypes + tid] = sm.species[tid];
+  __syncthreads();
+#pragma unroll
+  for (int it = 0; it < ITEMS; ++it)
+    if (ty[it] >= 0) tperm[chunk[ty[it] * kChunks + w * ITEMS + it] + rank[it]] = (uint32_t)(i0 + it * 32);
 }
 
 int work_grid(ng_ctx* c, int64_t items, int per_sm) {
@@ -553,11 +727,6 @@ int work_grid(ng_ctx* c, int64_t items, int per_sm) {
 bool box_is_pow2(double L) {
   int e = 0;
   return std::frexp(L, &e) == 0.5;
-}
-
-static KeyArgs key_args(const ng_ctx* c, int64_t n, const double* pos, const uint8_t* type) {
-  const bool pow2 = box_is_pow2(c->L);
-  return KeyArgs{n, pos, type, c->L, 1.0 / c->L, pow2, pow2 ? std::ilogb(c->L) : 0, c->p.D};
 }
 
 int reserve_sort(ng_ctx* c, int64_t n) {
@@ -576,9 +745,26 @@ int reserve_sort(ng_ctx* c, int64_t n) {
   return NG_OK;
 }
 
-// Keys of the bodies at pos and their stable sort: sorted keys in keys_a,
-// the permutation (sorted index -> input index) in vals_a.
-static int sort_keys(ng_ctx* c, int64_t n, const double* pos, const uint8_t* type) {
+template <int ITEMS, bool RESIDENT>
+static int sort_small(ng_ctx* c, const KeyArgs& a, const GatherArgs& g, int first) {
+  const size_t smem = sizeof(SmSmem<ITEMS>);
+  NG_CUDA(c, cudaFuncSetAttribute(k_sort_small<ITEMS, RESIDENT>,
+                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  k_sort_small<ITEMS, RESIDENT><<<1, kSmThreads, smem, c->stream>>>(
+      a, g, first, as<uint64_t>(c->keys_a), as<uint32_t>(c->vals_a), as<uint32_t>(c->sort_words),
+      as<uint32_t>(c->tperm));
+  c->launches += 1;
+  c->typed = true;
+  NG_CUDA(c, cudaGetLastError());
+  return NG_OK;
+}
+
+// Keys of the bodies at g.pos, their stable sort (sorted keys in keys_a, the
+// permutation sorted index -> input index in vals_a) and the gather into
+// sorted order.
+template <bool RESIDENT>
+static int sort_stage(ng_ctx* c, const GatherArgs& g) {
+  const int64_t n = g.n;
   uint64_t *ka = as<uint64_t>(c->keys_a), *kb = as<uint64_t>(c->keys_b);
   uint32_t *va = as<uint32_t>(c->vals_a), *vb = as<uint32_t>(c->vals_b);
   // 8 passes of 8 bits: the result returns to (ka, va). A tree capped at
@@ -593,6 +779,11 @@ static int sort_keys(ng_ctx* c, int64_t n, const double* pos, const uint8_t* typ
   }
   c->sort_passes = 8 - first;
   c->typed = false;
+  const KeyArgs a{n, g.pos, g.type, g.L, g.invL, g.pow2, g.pow2 ? std::ilogb(c->L) : 0, c->p.D};
+  if (n <= kSmallSort) {
+    stage_mark(c, NG_STAGE_KEYS);
+    return n <= 4 * kSmThreads ? sort_small<4, RESIDENT>(c, a, g, first) : sort_small<8, RESIDENT>(c, a, g, first);
+  }
   const int64_t lbw = rs_lb_words(n), lbt = 8 * to_tiles(n);
   uint64_t* lb = as<uint64_t>(c->lookback);
   stage_mark(c, NG_STAGE_KEYS);
@@ -600,7 +791,7 @@ static int sort_keys(ng_ctx* c, int64_t n, const double* pos, const uint8_t* typ
   // blocks of at least 2048 bodies, at most two per SM: each adds its
   // histograms to the global ones
   const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)c->nsm * 2, (n + 2047) / 2048));
-  k_keys<<<grid, 512, 0, c->stream>>>(key_args(c, n, pos, type), first, ka, as<uint32_t>(c->sort_words),
+  k_keys<<<grid, 512, 0, c->stream>>>(a, first, ka, as<uint32_t>(c->sort_words),
                                       lb, lbw, lb + 2 * lbw, lbt);
   c->launches += 1;
   NG_CUDA(c, cudaGetLastError());
@@ -615,35 +806,46 @@ static int sort_keys(ng_ctx* c, int64_t n, const double* pos, const uint8_t* typ
     if (rs_large(n)) NG_TRY(rs_pass<kRsItemsLarge>(c, kin, vin, kout, vout, n, pass, lin, lnext));
     else NG_TRY(rs_pass<kRsItemsSmall>(c, kin, vin, kout, vout, n, pass, lin, lnext));
   }
-  return NG_OK;
-}
-
-int sort_resident(ng_ctx* c, int64_t n) {
-  NG_TRY(sort_keys(c, n, as<double>(c->spos_alt), as<uint8_t>(c->stype_alt)));
   stage_mark(c, NG_STAGE_GATHER);
-  k_gather_resident<<<work_grid(c, n, 8), 256, 0, c->stream>>>(
-      n, as<uint32_t>(c->vals_a), as<double>(c->spos_alt), as<float>(c->smass_alt),
-      as<uint8_t>(c->stype_alt), as<float>(c->rvel_alt), as<uint32_t>(c->rorig_alt),
-      as<double>(c->spos), as<float>(c->smass), as<uint8_t>(c->stype), as<float>(c->rvel),
-      as<uint32_t>(c->rorig));
+  k_gather<RESIDENT><<<work_grid(c, n, 8), 256, 0, c->stream>>>(g, va);
   c->launches += 1;
   NG_CUDA(c, cudaGetLastError());
   return NG_OK;
 }
 
+static GatherArgs gather_args(ng_ctx* c, int64_t n) {
+  GatherArgs g{};
+  g.n = n;
+  g.spos = as<double>(c->spos);
+  g.smass = as<float>(c->smass);
+  g.stype = as<uint8_t>(c->stype);
+  g.L = c->L;
+  g.invL = 1.0 / c->L;
+  g.pow2 = box_is_pow2(c->L);
+  g.D = c->p.D;
+  g.status = as<uint32_t>(c->status);
+  return g;
+}
+
+int sort_resident(ng_ctx* c, int64_t n) {
+  GatherArgs g = gather_args(c, n);
+  g.pos = as<double>(c->spos_alt);
+  g.mass = as<float>(c->smass_alt);
+  g.type = as<uint8_t>(c->stype_alt);
+  g.vel = as<float>(c->rvel_alt);
+  g.orig = as<uint32_t>(c->rorig_alt);
+  g.svel = as<float>(c->rvel);
+  g.sorig = as<uint32_t>(c->rorig);
+  return sort_stage<true>(c, g);
+}
+
 int sort_bodies(ng_ctx* c, int64_t n, const double* pos, const uint8_t* type, const float* mass) {
   NG_TRY(reserve_sort(c, n));
-  uint32_t* va = as<uint32_t>(c->vals_a);
-  const int grid = work_grid(c, n, 8);
-  const bool pow2 = box_is_pow2(c->L);
-  NG_TRY(sort_keys(c, n, pos, type));
-  c->launches += 1;   // gather
-  stage_mark(c, NG_STAGE_GATHER);
-  k_gather<<<grid, 256, 0, c->stream>>>(n, va, pos, type, mass, c->L, 1.0 / c->L, pow2, c->p.D,
-                                        as<double>(c->spos), as<float>(c->smass),
-                                        as<uint8_t>(c->stype), as<uint32_t>(c->status));
-  NG_CUDA(c, cudaGetLastError());
-  return NG_OK;
+  GatherArgs g = gather_args(c, n);
+  g.pos = pos;
+  g.mass = mass;
+  g.type = type;
+  return sort_stage<false>(c, g);
 }
 
 int type_order(ng_ctx* c) {
