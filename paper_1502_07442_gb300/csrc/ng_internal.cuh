@@ -236,6 +236,8 @@ struct WalkLaunch {
   int ndesc;
   const uint32_t* gprefix;  // [ndesc + 1] group prefix
   uint32_t* work;           // work-queue counter
+  int warps;                // warps of a block that take groups
+  int team, split;          // warps per group, and the tree level their nodes are shared out at
   // law table, segments {c0 - k c1, c1}: single simulations
   // [list species t][ncut + 1][walk_tab_pad(D)] (entry s: passive species s);
   // variable-species launches [law][ncut + 1] (a lane's row: tabid[s][t])

@@ -43,7 +43,18 @@ struct __align__(16) WarpSmem {
   int2 leafb[32];             // opened leaves: first body, body count
   int leafo[32];              // opened leaves: exclusive prefix of body counts
   int stack[kStackCap];
+  uint32_t item;              // team launches: the team's group (its first warp's)
 };
+
+// Team launches: a warp's partial sums, where its team's first warp reads them
+// (the record lists are drained by then).
+template <class Acc, int D, int CAP>
+__device__ __forceinline__ Acc* team_part(WarpSmem<D, CAP>* ws) {
+  return reinterpret_cast<Acc*>(&ws->list[0][0]);
+}
+__device__ __forceinline__ void team_sync(int id, int threads) {
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
 
 constexpr float kMagic = 8388608.0f;   // 2^23
 constexpr int kMagicBits = 0x4B000000;
@@ -89,30 +100,54 @@ __device__ __forceinline__ float2 lds_f2(uint32_t addr) {
 // VARD: the simulations of the launch may have different species counts; D
 // is then the largest (lists for D species, the law table laid out for D),
 // and each work item uses its simulation's own count DESC(D) <= D.
-template <int D, bool ACC64, bool REL, bool VARD>
+// TEAM: L.team warps of a block share a group. Each walks the tree above level
+// L.split alike and takes the nodes of that level, and the accepted nodes and
+// leaves above it, whose number is its own place modulo the team; the team's
+// sums are added in order at the end. For launches with few groups per warp
+// slot, where whole groups per warp leave slots idle or a long tail.
+template <int D, bool ACC64, bool REL, bool VARD, bool TEAM>
 __global__ void __launch_bounds__((VARD ? kVardWarps : walk_warps(D)) * 32, 1) k_walk(WalkLaunch L) {
   using Acc = typename std::conditional<ACC64, double, float>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float2* tab = reinterpret_cast<float2*>(smem_raw);
   const int ntab = L.tab_count;
-  for (int i = threadIdx.x; i < ntab; i += blockDim.x) tab[i] = L.tab[i];
+  {
+    // 16 bytes at a time (the table starts on a cudaMalloc boundary), the odd
+    // entry on its own
+    const float4* src = reinterpret_cast<const float4*>(L.tab);
+    float4* dst = reinterpret_cast<float4*>(tab);
+#pragma unroll 8
+    for (int i = threadIdx.x; i < ntab / 2; i += blockDim.x) dst[i] = src[i];
+    if ((ntab & 1) && threadIdx.x == 0) tab[ntab - 1] = L.tab[ntab - 1];
+  }
   const size_t tab_bytes = ((size_t)ntab * sizeof(float2) + 15) & ~(size_t)15;
   constexpr int CAP = walk_list_cap(D, VARD);
   WarpSmem<D, CAP>* ws = reinterpret_cast<WarpSmem<D, CAP>*>(smem_raw + tab_bytes) + (threadIdx.x >> 5);
   __syncthreads();
+  if ((int)(threadIdx.x >> 5) >= L.warps) return;   // only helped to load the table
 
   const int lane = threadIdx.x & 31;
   const uint32_t lt = (1u << lane) - 1u;
   const uint32_t total_groups = L.gprefix[L.ndesc];
   const int clampbits = kMagicBits + L.ncut;
   unsigned long long nint = 0;
+  // place in the team, and the team's first warp
+  const int tw = TEAM ? (int)(threadIdx.x >> 5) % L.team : 0;
+  WarpSmem<D, CAP>* head = ws - tw;
+  const int bar = TEAM ? 1 + (int)(threadIdx.x >> 5) / L.team : 0;
 
   while (true) {
     // one work item = one group of one simulation (all simulations of the
     // launch share the law table and the species count)
     uint32_t g = 0;
-    if (lane == 0) g = atomicAdd(L.work, 1u);
-    g = __shfl_sync(0xffffffffu, g, 0);
+    if (lane == 0 && tw == 0) g = atomicAdd(L.work, 1u);
+    if (TEAM) {
+      if (lane == 0 && tw == 0) head->item = g;
+      team_sync(bar, 32 * L.team);
+      g = head->item;
+    } else {
+      g = __shfl_sync(0xffffffffu, g, 0);
+    }
     if (g >= total_groups) break;
     int lo_s = 0, hi_s = L.ndesc - 1;
     while (lo_s < hi_s) {
@@ -127,6 +162,7 @@ __global__ void __launch_bounds__((VARD ? kVardWarps : walk_warps(D)) * 32, 1) k
     }
     __syncwarp();
     const uint32_t nnodes = DESC(status)[ST_LEVELS + kMaxLevel + 1];
+    const uint32_t split0 = TEAM ? DESC(status)[ST_LEVELS + L.split] : 0u;   // first node of the level
     const int DR = VARD ? DESC(D) : D;   // species of this item's simulation
     const float rc2 = DESC(rcut_box) * DESC(rcut_box);
     const float rc2_keep = rc2 * 1.0001f;   // margin for FP32 rounding of the offsets
@@ -387,6 +423,10 @@ __global__ void __launch_bounds__((VARD ? kVardWarps : walk_warps(D)) * 32, 1) k
           }
           if (take) cls = 1;
           else cls = lk.y == 0 ? 2 : 3;
+          // above the split level every warp of the team is here: its own
+          // nodes only, unless their children are still above
+          if (TEAM && (uint32_t)node < split0 && cls != 3 && (uint32_t)node % (uint32_t)L.team != (uint32_t)tw)
+            cls = 0;
         }
       }
       // accepted nodes: one record per species with mass
@@ -406,7 +446,15 @@ __global__ void __launch_bounds__((VARD ? kVardWarps : walk_warps(D)) * 32, 1) k
       // rejected internal nodes: push children, in lane order while they
       // fit in `avail`; the remaining opened nodes are pushed back
       {
-        const int nch = cls == 3 ? lk.y : 0;
+        int nch = cls == 3 ? lk.y : 0, step = 1;
+        if (TEAM && cls == 3 && (uint32_t)node < split0 && (uint32_t)lk.x >= split0) {
+          // the team's warps share the children at the split level
+          const int skip = (int)(((uint32_t)tw + (uint32_t)L.team - (uint32_t)lk.x % (uint32_t)L.team) %
+                                 (uint32_t)L.team);
+          nch = lk.y > skip ? (lk.y - 1 - skip) / L.team + 1 : 0;
+          lk.x += skip;
+          step = L.team;
+        }
         int incl = nch;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -418,7 +466,7 @@ __global__ void __launch_bounds__((VARD ? kVardWarps : walk_warps(D)) * 32, 1) k
         const int used = (int)__reduce_max_sync(0xffffffffu, fit ? (unsigned)incl : 0u);
         if (fit) {
           const int base = size + incl - nch;
-          for (int cc = 0; cc < nch; ++cc) ws->stack[base + cc] = lk.x + cc;
+          for (int cc = 0; cc < nch; ++cc) ws->stack[base + cc] = lk.x + cc * step;
         } else if (cls == 3) {
           ws->stack[size + used + __popc(back & lt)] = node;
         }
@@ -454,10 +502,26 @@ __global__ void __launch_bounds__((VARD ? kVardWarps : walk_warps(D)) * 32, 1) k
       __syncwarp();
     }
     __syncwarp();
-    if (overflow) {
-      if (lane == 0) atomicOr(&DESC(status)[ST_FLAGS], (uint32_t)SF_STACK_OVERFLOW);
-      continue;
+    if (overflow && lane == 0) atomicOr(&DESC(status)[ST_FLAGS], (uint32_t)SF_STACK_OVERFLOW);
+    if (TEAM) {
+      // the team's sums to its first warp, in order (an overflow leaves NaN:
+      // the group is not written)
+      Acc* mine = team_part<Acc>(ws);
+      mine[lane] = overflow ? (Acc)NAN : ax;
+      mine[32 + lane] = ay;
+      mine[64 + lane] = az;
+      team_sync(bar, 32 * L.team);
+      if (tw != 0) continue;
+      for (int j = 1; j < L.team; ++j) {
+        const Acc* o = team_part<Acc>(head + j);
+        overflow = overflow || isnan(o[lane]) != 0;
+        ax += o[lane];
+        ay += o[32 + lane];
+        az += o[64 + lane];
+      }
+      overflow = __any_sync(0xffffffffu, overflow && (DESC(status)[ST_FLAGS] & SF_STACK_OVERFLOW) != 0);
     }
+    if (overflow) continue;
     if (active) {
       const Acc sc = (Acc)DESC(out_scale);
       const float fx = (float)(ax * sc), fy = (float)(ay * sc), fz = (float)(az * sc);
@@ -525,29 +589,63 @@ static size_t walk_smem(int tab_count, int nwarps) {
   return tab_bytes + (size_t)nwarps * sizeof(WarpSmem<D, walk_list_cap(D, VARD)>);
 }
 
+template <int D, bool ACC64, bool REL, bool VARD, bool TEAM>
+static int launch_walk_t(ng_ctx* c, cudaStream_t stream, WalkLaunch L, int64_t groups, int nwarps) {
+  auto kernel = k_walk<D, ACC64, REL, VARD, TEAM>;
+  const size_t smem = walk_smem<D, VARD>(L.tab_count, nwarps);
+  // the attribute is a per-function ceiling shared by every thread that
+  // launches the walk: always raise it to the device maximum, never lower it
+  NG_CUDA(c, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c->smem_optin));
+  const int threads = std::max(nwarps, 4) * 32;
+  int per_sm = 0;
+  NG_CUDA(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem));
+  if (per_sm < 1) per_sm = 1;
+  // persistent warps take groups from a counter: no more blocks than the
+  // expected groups need, so small problems leave SMs to concurrent work
+  const int64_t slots = nwarps / L.team;
+  const int64_t want = (std::max<int64_t>(groups, 1) + slots - 1) / slots;
+  const int grid = (int)std::min<int64_t>((int64_t)c->nsm * per_sm, want);
+  L.warps = nwarps;
+  kernel<<<grid, threads, smem, stream>>>(L);
+  c->launches += 1;
+  NG_CUDA(c, cudaGetLastError());
+  return NG_OK;
+}
+
+// Warps per group. With whole groups per warp, a launch of fewer groups than
+// warp slots leaves slots idle, and one of about as many ends with a long
+// tail; a team splits a group's work at the cost of walking the top of the
+// tree once per warp. Passes measured with 1 / 2 / 4 / 8 warps a group: a force
+// on 4096 bodies (0.05 groups per slot) 310 / 262 / 248 / 245 us, on 131k bodies
+// (1.4 per slot) 692 / 682 / 740 / 902 us, a 200k-body step (2.1) 708 / 704 /
+// 767 / 959 us, a 300k-body tree force (4, six species) 1006 / 1110 / 1346 / 1877 us.
+static int walk_team(int64_t groups, int64_t slots) {
+  return groups <= slots / 8 ? 8 : groups <= slots / 2 ? 4 : groups <= 3 * slots ? 2 : 1;
+}
+
 template <int D, bool ACC64, bool REL, bool VARD>
-static int launch_walk_d(ng_ctx* c, cudaStream_t stream, const WalkLaunch& L, int64_t groups) {
+static int launch_walk_d(ng_ctx* c, cudaStream_t stream, WalkLaunch L, int64_t groups) {
   int nwarps = VARD ? kVardWarps : walk_warps(D);
   while (nwarps > 1 && walk_smem<D, VARD>(L.tab_count, nwarps) > c->smem_optin) --nwarps;
   const size_t smem = walk_smem<D, VARD>(L.tab_count, nwarps);
   if (smem > c->smem_optin)
     return fail(c, NG_ENOMEM, "walk needs %zu B shared memory (max %zu)", smem, c->smem_optin);
-  // the attribute is a per-function ceiling shared by every thread that
-  // launches the walk: always raise it to the device maximum, never lower it
-  NG_CUDA(c, cudaFuncSetAttribute(k_walk<D, ACC64, REL, VARD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)c->smem_optin));
-  int per_sm = 0;
-  NG_CUDA(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_walk<D, ACC64, REL, VARD>, nwarps * 32,
-                                                           smem));
-  if (per_sm < 1) per_sm = 1;
-  // persistent warps take groups from a counter: no more blocks than the
-  // expected groups need, so small problems leave SMs to concurrent work
-  const int64_t want = (std::max<int64_t>(groups, 1) + nwarps - 1) / nwarps;
-  const int grid = (int)std::min<int64_t>((int64_t)c->nsm * per_sm, want);
-  k_walk<D, ACC64, REL, VARD><<<grid, nwarps * 32, smem, stream>>>(L);
-  c->launches += 1;
-  NG_CUDA(c, cudaGetLastError());
-  return NG_OK;
+  L.team = 1;
+  if constexpr (!VARD) {
+    int team = walk_team(groups, (int64_t)c->nsm * nwarps);
+    while (team > nwarps) team /= 2;
+    if (team > 1) {
+      L.team = team;
+      // cells of the split level are about 0.7 r_cut wide, so that a group
+      // reaches some tens of them
+      L.split = std::min(std::max((int)std::floor(std::log2(c->L / c->rcut)) + 1, 1), kMaxLevel);
+      // few groups: no more warps per block than spread over the SMs they take
+      const int64_t per = (groups + c->nsm - 1) / c->nsm;
+      nwarps = (int)std::min<int64_t>(nwarps / team, std::max<int64_t>(1, per)) * team;
+      return launch_walk_t<D, ACC64, REL, VARD, true>(c, stream, L, groups, nwarps);
+    }
+  }
+  return launch_walk_t<D, ACC64, REL, VARD, false>(c, stream, L, groups, nwarps);
 }
 
 void fill_walk_desc(ng_ctx* c, float* acc, bool accumulate, WalkDesc* d) {
