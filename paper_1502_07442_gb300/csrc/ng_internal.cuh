@@ -19,16 +19,13 @@ namespace ng {
 constexpr int kMaxD = NG_MAX_SPECIES;
 constexpr int kMaxLevel = 20;           // 20 Morton bits per axis
 constexpr int kCapturedDepthMargin = 2;  // captured steps build this far below the depth seen
-// The top levels of a tree's monopoles are reduced by one cluster of
-// kClusterBlocks blocks with the hardware cluster barrier between levels.
-constexpr int kClusterBlocks = 8;
-constexpr int kMonoWords = 1 + kMaxLevel + 1;   // counters of the monopole stage
-// Monopoles of trees of kBinnedMonoBodies bodies or more are reduced in an
-// order binned by the work of a node: leaves by body count (0..64, one more
-// bin for the larger leaves of a tree stopped at a level cap), internal nodes
-// by level and child count.
+constexpr int kMonoWords = 2;   // counters of the monopole stage
+// Monopoles of trees of kBinnedMonoBodies bodies or more take their leaves and
+// ready internal nodes in an order binned by the work of a node: leaves by body
+// count (0..64, one more bin for the larger leaves of a tree stopped at a level
+// cap), internal nodes by child count.
 constexpr int kLeafBins = 66;
-constexpr int kMonoBins = kLeafBins + (kMaxLevel + 1) * 8;
+constexpr int kMonoBins = kLeafBins + 8;
 constexpr int64_t kBinnedMonoBodies = 1 << 20;
 constexpr int kWarp = 32;
 

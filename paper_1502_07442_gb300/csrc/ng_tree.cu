@@ -1,7 +1,7 @@
 // Tree stage (Sec. 2.2): canonical Morton-prefix octree, all levels at once
 // from the sorted keys (node ranges stay on the device, no host round trip),
 // per-node per-species monopoles reduced in double precision (every leaf in
-// one launch, then the internal nodes by subtrees, bottom-up), and the walk
+// one launch, then the internal nodes bottom-up), and the walk
 // groups.
 //
 // Canonical tree: nodes are the non-empty Morton cells reachable from the
@@ -11,8 +11,6 @@
 // steps stop at a level cap two below the deepest level seen by the step
 // before the capture (their sort then orders fewer key bits); a cell at the
 // cap is then a leaf whatever it holds, and SF_DEPTH says so.
-#include <cooperative_groups.h>
-
 #include "ng_internal.cuh"
 
 namespace ng {
@@ -258,14 +256,8 @@ __global__ void k_tree_nodes(uint32_t* status, int64_t cap, const uint64_t* __re
   }
 }
 
-// Largest subtree of the monopole stage: about n / 2048 bodies, 256 or more.
-constexpr uint32_t kMaxSub = 512;
-static uint32_t mono_sub(int64_t n) { return n <= 256 * 2048 ? 256 : kMaxSub; }
-
-size_t tree_scratch_bytes(int64_t n) {
-  // node counts per level and tile, later the top nodes of the monopoles
-  const int64_t per = std::max<int64_t>((n + kTreeTile - 1) / kTreeTile, n / mono_sub(n) + 1);
-  return (size_t)per * (kMaxLevel + 1) * sizeof(uint32_t);
+size_t tree_scratch_bytes(int64_t n) {   // node counts per level and tile
+  return (size_t)((n + kTreeTile - 1) / kTreeTile) * (kMaxLevel + 1) * sizeof(uint32_t);
 }
 
 int build_octree(ng_ctx* c) {
@@ -353,14 +345,16 @@ constexpr int kTeam = 4 * walk_tab_pad(D);
 // An internal node as its team needs it, loaded ahead of the children's sums.
 struct MonoNode {
   uint32_t k, nch, c0;   // nch = 0: no node
+  uint32_t parent;
   int level;
   uint64_t prefix;
 };
 __device__ __forceinline__ MonoNode mono_load(bool valid, uint32_t k, const MonoArgs& a) {
-  MonoNode v{k, 0u, 0u, 0, 0ull};
+  MonoNode v{k, 0u, 0u, 0u, 0, 0ull};
   if (valid) {
     v.nch = a.nchild[k];
     v.c0 = a.child[k];
+    v.parent = (uint32_t)a.link[k].w;   // left there by k_tree_nodes
     v.level = a.level[k];
     v.prefix = a.prefix[k];
   }
@@ -376,10 +370,12 @@ __device__ __forceinline__ float4 mono_geo(int level, uint64_t prefix) {
                      (float)(2u * morton_compact3(prefix) + 1u) * h, h);
 }
 
-// Sums of internal node v over its children, in child order, by the kTeam<D>
-// lanes of its team. All lanes of the warp call it together.
+// Sum of internal node v over its children by the kTeam<D> lanes of its team:
+// the lane's component of its species, stored for the parent. All lanes of the
+// warp call it together. The additions form a tree (FP64 results come tens of
+// cycles apart, and a path to the root makes them at each of its levels).
 template <int D>
-__device__ __forceinline__ void mono_internal(const MonoNode& v, const MonoArgs& a) {
+__device__ __forceinline__ double mono_sum(const MonoNode& v, const MonoArgs& a) {
   constexpr int P = walk_tab_pad(D);
   const int lane = threadIdx.x & 31, e = lane & 3, q = (lane >> 2) & (P - 1);
   const bool mine = v.nch > 0 && q < D;
@@ -390,24 +386,34 @@ __device__ __forceinline__ void mono_internal(const MonoNode& v, const MonoArgs&
     c[j] = 0.0;
     if (mine && j < (int)v.nch) {
       const size_t r = (size_t)(v.c0 + j) * D + q;
-      c[j] = a.m64[r * 4 + e];
-      if (e == 0) cn += a.cnt[r];
+      c[j] = __ldcg(a.m64 + r * 4 + e);   // of any SM: past this one's L1
+      if (e == 0) cn += __ldcg(a.cnt + r);
     }
   }
   // no further than the longest list of the warp
+  double sum = c[0] + c[1];
   const int most = (int)__reduce_max_sync(0xffffffffu, v.nch);
-  double sum = 0.0;
-#pragma unroll
-  for (int j = 0; j < 8; ++j) {
-    if (j >= most) break;
-    sum += c[j];
+  if (most > 2) sum += c[2] + c[3];
+  if (most > 4) sum += (c[4] + c[5]) + (c[6] + c[7]);
+  if (mine) {
+    const size_t r = (size_t)v.k * D + q;
+    a.m64[r * 4 + e] = sum;
+    if (e == 0) a.cnt[r] = cn;
   }
+  return sum;
+}
+
+// The walk's records of node v from the lanes' sums.
+template <int D>
+__device__ __forceinline__ void mono_node_records(const MonoNode& v, double sum, const MonoArgs& a) {
+  constexpr int P = walk_tab_pad(D);
+  const int lane = threadIdx.x & 31, e = lane & 3, q = (lane >> 2) & (P - 1);
   // over the species (zero in idle lanes), for the node's own centre of mass
   double all = sum;
 #pragma unroll
   for (int o = 4; o < kTeam<D>; o <<= 1) all += __shfl_xor_sync(0xffffffffu, all, o);
   const double m = __shfl_sync(0xffffffffu, sum, 0, 4), mt = __shfl_sync(0xffffffffu, all, 0, 4);
-  if (!mine) return;
+  if (v.nch == 0 || q >= D) return;
   double cen[3], side;
   node_centre(v.level, v.prefix, cen, &side);
   const double ce = e == 1 ? cen[0] : e == 2 ? cen[1] : cen[2];
@@ -415,9 +421,7 @@ __device__ __forceinline__ void mono_internal(const MonoNode& v, const MonoArgs&
   const size_t r = (size_t)v.k * D + q;
   const int at = (e + 3) & 3;
   const float mf = (float)m, f = e == 0 ? mf : (float)fma(-m, ce, sum) * (1.0f / mf);
-  a.m64[r * 4 + e] = sum;
   reinterpret_cast<float*>(a.mono)[r * 4 + at] = m > 0.0 ? f : 0.f;
-  if (e == 0) a.cnt[r] = cn;
   if (q == 0) {
     const float tf = (float)mt, g = e == 0 ? tf : (float)fma(-mt, ce, all) * (1.0f / tf);
     reinterpret_cast<float*>(a.com)[(size_t)v.k * 4 + at] = mt > 0.0 ? g : 0.f;
@@ -428,8 +432,7 @@ __device__ __forceinline__ void mono_internal(const MonoNode& v, const MonoArgs&
 
 // The same sums by the calling lane alone, all species: an FP64 instruction
 // then serves 32 nodes, against 32 / kTeam<D> in teams, for four times as many
-// of them in a row. Taken where the nodes make kLaneLevel rounds of teams.
-constexpr uint32_t kLaneLevel = 4;
+// of them in a row.
 template <int D>
 __device__ __forceinline__ void mono_internal_lane(const MonoNode& v, const MonoArgs& a) {
   if (v.nch == 0) return;
@@ -468,38 +471,39 @@ __device__ __forceinline__ void mono_internal_lane(const MonoNode& v, const Mono
   a.link[v.k] = make_int4((int)v.c0, (int)v.nch, (int)a.first[v.k], (int)a.count[v.k]);
 }
 
-// The internal nodes are reduced by subtrees. A subtree is rooted at an
-// internal node of at most `sub` bodies whose parent holds more (or at such a
-// root of the whole tree); one block reduces all its levels bottom-up, with no
-// launch between levels. The nodes above, fewer than n / sub per level, are
-// listed by level and reduced by one thread-block cluster; sub grows with n so
-// that they stay few thousands.
-// One launch per level (21 of them, each waiting for the slowest warp of a
-// level) took 212 us at 131k bodies and three species, the three launches
-// here 121 us.
+// Internal nodes are summed bottom-up without waiting: a node's link holds, until
+// it is formed, its parent (w, from k_tree_nodes) and how many of its internal
+// children are not formed yet (x). Who forms a node takes one off its parent's
+// count, and who takes the last one forms the parent next. The nodes without
+// internal children are ready at the start.
+// The sums are always over all children in the same order, whoever forms the node.
+// Bound by latency: a level of a path costs two dependent loads, the additions
+// and one counter. Subtrees of 256 bodies by one block each, level by level
+// with barriers, and a cluster of eight blocks for the nodes above took 88 us at
+// 131k bodies and three species, 175 us at 300k and six; this 48 and 59 us. (A
+// 131k-body force 687 -> 651 us, a 300k-body tree force 981 -> 894 us, a
+// 200k-body step 713 -> 660 us, all with the tiles' loads below.)
 //
-// Counters (c->mono_words, zeroed by k_tree_emit): the subtrees and the top
-// nodes per level. Subtree roots are listed in n_tmp, top
-// nodes of level l at top[l * per], top = the tree build's scratch.
-struct MonoLists {
-  uint32_t* words;
-  uint32_t* roots;   // n_tmp
-  uint32_t* top;     // tree_cnt
-  uint32_t sub;      // bodies of the largest subtree
-  uint32_t per;      // top nodes a level can hold
-};
-constexpr int kMlSub = 0, kMlTop = 1;
-static_assert(kMlTop + kMaxLevel + 1 == kMonoWords && kMonoWords <= kTreeThreads, "monopole counters");
+// Counters (c->mono_words, zeroed by k_tree_emit): ready nodes (trees below
+// kBinnedMonoBodies bodies; listed in n_tmp), and nodes listed by k_mono_ready.
+constexpr int kMlReady = 0, kMlNext = 1;
+static_assert(kMlNext + 1 == kMonoWords && kMonoWords <= kTreeThreads, "monopole counters");
 
-// Internal node k into the top list if it is large, into the subtree list if
-// it is small and its parent (left in its link by k_tree_nodes) is not.
-__device__ __forceinline__ void mono_list(uint32_t k, const MonoArgs& a, const MonoLists& m) {
-  if (a.count[k] > m.sub) {
-    const int l = a.level[k];
-    m.top[(size_t)l * m.per + atomicAdd(&m.words[kMlTop + l], 1u)] = k;
-  } else if (k == 0 || a.count[a.link[k].w] > m.sub) {
-    m.roots[atomicAdd(&m.words[kMlSub], 1u)] = k;
-  }
+// Internal children of node k
+__device__ __forceinline__ int mono_pending(uint32_t k, uint32_t nch, const MonoArgs& a) {
+  const uint32_t c0 = nch ? a.child[k] : 0u;
+  int need = 0;
+  for (uint32_t j = 0; j < nch; ++j) need += a.nchild[c0 + j] != 0;
+  return need;
+}
+
+// One internal child of the node with this count is formed: the count before.
+// What this thread (and, past a warp barrier, its warp) has written is seen by
+// whoever finds the count at one, past its own.
+__device__ __forceinline__ int mono_done(int* pending) {
+  int v;
+  asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], -1;" : "=r"(v) : "l"(pending) : "memory");
+  return v;
 }
 
 // Tile: bodies whose leaves start in a block's turn (small, so that a small
@@ -510,45 +514,66 @@ struct LeafSmem {
   double x[3][kLeafLoad];
   float m[kLeafLoad];
   double acc[D][4][kLeafThreads];        // {m, m x, m y, m z} per species, physical units
-  uint32_t start[kLeafTile];             // local start | count class << 16, then in count order
-  uint32_t order[kLeafTile];
+  uint32_t start[kLeafTile];             // per leaf of the tile: local start | count class << 16
+  uint32_t leaf[kLeafTile];              // and its node
+  uint32_t order[kLeafTile];             // leaves in count order
+  uint32_t heads[kLeafTile / 32];        // bodies that start a leaf
   uint32_t bins[kMaxLeaf + 2];
-  uint32_t warp_tot[kLeafThreads / 32], tile_total;
   uint8_t t[kLeafLoad];
 };
 
 // Every leaf and body record, one tile of bodies per block and turn; the
-// internal nodes into their lists.
+// counts of the internal nodes, and the list of those that are ready.
 template <int D>
-__global__ void __launch_bounds__(kLeafThreads) k_mono_tiles(MonoArgs a, MonoLists ml) {
+__global__ void __launch_bounds__(kLeafThreads) k_mono_tiles(MonoArgs a, uint32_t* words, uint32_t* ready) {
   __shared__ LeafSmem<D> sm;
   if (a.status[ST_FLAGS] & SF_NODE_OVERFLOW) return;   // truncated tree: do not read it
   const int tid = threadIdx.x;
   const uint32_t total = levels_of(a.status).start[kMaxLevel + 1];
-  for (uint32_t k = blockIdx.x * blockDim.x + tid; k < total; k += gridDim.x * blockDim.x) {
-    if (a.nchild[k]) mono_list(k, a, ml);
+  for (uint32_t k0 = blockIdx.x * blockDim.x + (tid & ~31); k0 < total; k0 += gridDim.x * blockDim.x) {
+    // warps step together
+    const uint32_t k = k0 + (tid & 31), nch = k < total ? a.nchild[k] : 0u;
+    const int need = mono_pending(k, nch, a);
+    if (nch) a.link[k].x = need;
+    const uint32_t list = __ballot_sync(0xffffffffu, nch != 0 && need == 0);
+    uint32_t at = 0;
+    if ((tid & 31) == 0 && list) at = atomicAdd(&words[kMlReady], (uint32_t)__popc(list));
+    at = __shfl_sync(0xffffffffu, at, 0) + __popc(list & ((1u << (tid & 31)) - 1u));
+    if (nch != 0 && need == 0) ready[at] = k;
   }
   const float invLf = (float)a.invL;
   for (int64_t t0 = (int64_t)blockIdx.x * kLeafTile; t0 < a.n; t0 += (int64_t)gridDim.x * kLeafTile) {
     __syncthreads();   // the previous tile's readers are done
     const int held = (int)min((int64_t)kLeafLoad, a.n - t0), own = min(held, kLeafTile);
     for (int j = tid; j < kMaxLeaf + 2; j += kLeafThreads) sm.bins[j] = 0;
-    uint32_t nleaf = 0;   // leaves that start in the tile (the same in every thread)
-    for (int j0 = 0; j0 < held; j0 += kLeafThreads) {
-      const int j = j0 + tid;
-      bool head = false;
+    constexpr int kRounds = kLeafLoad / kLeafThreads, kOwnRounds = kLeafTile / kLeafThreads;
+    constexpr int kLeafWarps = kLeafThreads / 32;
+    uint32_t leaf[kOwnRounds];
+    bool head[kOwnRounds];
+#pragma unroll
+    for (int r = 0; r < kRounds; ++r) {
+      // no barrier between the rounds: their loads overlap
+      const int j = r * kLeafThreads + tid;
+      const int64_t b = t0 + j;
+      double xp = 0, yp = 0, zp = 0;
+      float m = 0.f;
       if (j < held) {
-        const int64_t b = t0 + j;
-        const double xp = a.spos[b], yp = a.spos[a.n + b], zp = a.spos[2 * a.n + b];
-        const float m = a.smass[b];
+        xp = a.spos[b];
+        yp = a.spos[a.n + b];
+        zp = a.spos[2 * a.n + b];
+        m = a.smass[b];
         sm.x[0][j] = xp;
         sm.x[1][j] = yp;
         sm.x[2][j] = zp;
         sm.m[j] = m;
         sm.t[j] = a.stype[b];
+      }
+      if (r < kOwnRounds) {
+        head[r] = false;
+        leaf[r] = 0;
         if (j < own) {
-          const uint32_t k = a.bleaf[b];
-          head = b == 0 || a.bleaf[b - 1] != k;
+          const uint32_t k = leaf[r] = a.bleaf[b];
+          head[r] = b == 0 || a.bleaf[b - 1] != k;
           double cen[3], side;
           node_centre(a.level[k], a.prefix[k], cen, &side);
           if (!a.unit) {
@@ -559,15 +584,26 @@ __global__ void __launch_bounds__(kLeafThreads) k_mono_tiles(MonoArgs a, MonoLis
           a.body[b] = make_float4((float)(xp - cen[0]) * invLf, (float)(yp - cen[1]) * invLf,
                                   (float)(zp - cen[2]) * invLf, m);
         }
+        const uint32_t heads = __ballot_sync(0xffffffffu, head[r]);
+        if ((tid & 31) == 0) sm.heads[r * kLeafWarps + (tid >> 5)] = heads;
       }
-      const uint32_t inc = block_inclusive_scan<kLeafThreads>(head ? 1u : 0u, sm.warp_tot, &sm.tile_total);
-      if (head) sm.start[nleaf + inc - 1] = (uint32_t)j;
-      nleaf += sm.tile_total;
-      __syncthreads();
     }
+    __syncthreads();
+    uint32_t nleaf = 0;   // leaves that start in the tile (the same in every thread)
+#pragma unroll
+    for (int w = 0; w < kLeafTile / 32; ++w) {
+      const uint32_t heads = sm.heads[w];
+      if (w % kLeafWarps == (tid >> 5) && head[w / kLeafWarps]) {
+        const uint32_t at = nleaf + __popc(heads & ((1u << (tid & 31)) - 1u));
+        sm.start[at] = (uint32_t)(w / kLeafWarps * kLeafThreads + tid);
+        sm.leaf[at] = leaf[w / kLeafWarps];
+      }
+      nleaf += __popc(heads);
+    }
+    __syncthreads();
     // the leaves by body count (one class for those above kMaxLeaf)
     for (uint32_t i = tid; i < nleaf; i += kLeafThreads) {
-      const uint32_t cls = min(a.count[a.bleaf[t0 + sm.start[i]]], (uint32_t)(kMaxLeaf + 1));
+      const uint32_t cls = min(a.count[sm.leaf[i]], (uint32_t)(kMaxLeaf + 1));
       sm.start[i] |= cls << 16;
       atomicAdd(&sm.bins[cls], 1u);
     }
@@ -589,11 +625,12 @@ __global__ void __launch_bounds__(kLeafThreads) k_mono_tiles(MonoArgs a, MonoLis
     }
     __syncthreads();
     for (uint32_t i = tid; i < nleaf; i += kLeafThreads)
-      sm.order[atomicAdd(&sm.bins[sm.start[i] >> 16], 1u)] = sm.start[i] & 0xffffu;
+      sm.order[atomicAdd(&sm.bins[sm.start[i] >> 16], 1u)] = i;
     __syncthreads();
     for (uint32_t i = tid; i < nleaf; i += kLeafThreads) {
-      const int j0 = (int)sm.order[i];
-      const uint32_t k = a.bleaf[t0 + j0], c = a.count[k];
+      const uint32_t at = sm.order[i], k = sm.leaf[at], cls = sm.start[at] >> 16;
+      const uint32_t c = cls <= (uint32_t)kMaxLeaf ? cls : a.count[k];
+      const int j0 = (int)(sm.start[at] & 0xffffu);
       uint32_t sc[D];
 #pragma unroll
       for (int q = 0; q < D; ++q) {
@@ -655,104 +692,37 @@ __global__ void __launch_bounds__(kLeafThreads) k_mono_tiles(MonoArgs a, MonoLis
   }
 }
 
-// One block per subtree: the internal nodes of a level are packed and then
-// summed one per lane where they fill the block's warps, else in teams.
+// The listed nodes and all above them: a team takes a listed node, forms it,
+// and goes on with the parent where that was the last child it waited for, else
+// with its next listed node. Nothing waits: a path from a leaf to the root
+// costs its loads and one counter per level.
 template <int D>
-__global__ void __launch_bounds__(kMonoThreads) k_mono_subtrees(MonoArgs a, MonoLists m) {
-  constexpr int kTeams = kMonoThreads / kTeam<D>;
-  __shared__ uint2 range[kMaxLevel + 1];
-  __shared__ uint32_t packed[kMaxSub / 2];   // a level's internal nodes hold two bodies or more
-  __shared__ uint32_t held[2];
-  __shared__ int deepest;
+__global__ void __launch_bounds__(kMonoThreads) k_mono_up(MonoArgs a, const uint32_t* __restrict__ list,
+                                                          const uint32_t* __restrict__ skip,
+                                                          const uint32_t* __restrict__ listed) {
   if (a.status[ST_FLAGS] & SF_NODE_OVERFLOW) return;
-  const int tid = threadIdx.x, lane = tid & 31;
-  Levels lv = levels_of(a.status);
-  const uint32_t roots = m.words[kMlSub];
-  for (uint32_t i = blockIdx.x; i < roots; i += gridDim.x) {
-    const uint32_t k = m.roots[i];
-    const int l0 = a.level[k];
-    if (tid < 32) {
-      // node range of the subtree per level: children are numbered in node order
-      uint32_t s = k, e = k + 1;
-      int l = l0;
-      while (s < e && l <= kMaxLevel) {
-        if (lane == 0) range[l] = make_uint2(s, e);
-        const uint32_t ns = a.child[s];
-        e = l == kMaxLevel ? ns : e < lv.start[l + 1] ? a.child[e] : lv.start[l + 2];
-        s = ns;
-        ++l;
-      }
-      if (lane == 0) {
-        deepest = l - 1;   // this level holds leaves only
-        held[0] = 0;
-      }
-    }
-    __syncthreads();
-    int turn = 0;
-    for (int x = deepest - 1; x >= l0; --x) {
-      const uint2 r = range[x];
-      for (uint32_t b = r.x; b < r.y; b += kMonoThreads) {
-        const uint32_t node = b + tid;
-        if (node < r.y && a.nchild[node]) packed[atomicAdd(&held[turn], 1u)] = node;
-      }
-      if (tid == 0) held[turn ^ 1] = 0;
-      __syncthreads();
-      const uint32_t cnt = held[turn];
-      turn ^= 1;
-      if (cnt >= kLaneLevel * kTeams) {
-        for (uint32_t j = tid; j < cnt; j += kMonoThreads)
-          mono_internal_lane<D>(mono_load(true, packed[j], a), a);
-      } else {
-        for (uint32_t j0 = 0; j0 < cnt; j0 += kTeams) {
-          const uint32_t j = j0 + tid / kTeam<D>;
-          mono_internal<D>(mono_load(j < cnt, j < cnt ? packed[j] : 0u, a), a);
-        }
-      }
-      __syncthreads();   // this level's sums are read by the next
-    }
-  }
-}
-
-// The nodes above the subtrees, level by level, by one cluster of
-// kClusterBlocks blocks (co-scheduled; its barrier is the hardware cluster
-// barrier, so no block waits on a flag).
-template <int D>
-__global__ void __cluster_dims__(kClusterBlocks, 1, 1) __launch_bounds__(512)
-k_mono_top(int lmax, MonoArgs a, MonoLists m) {
-  // the flag and the counts are the same for every block and not written
-  // here: every block returns, or none does
-  if (a.status[ST_FLAGS] & SF_NODE_OVERFLOW) return;
-  namespace cg = cooperative_groups;
-  cg::cluster_group cluster = cg::this_cluster();
   const int lane = threadIdx.x & 31;
-  const uint32_t team = (blockIdx.x * blockDim.x + threadIdx.x) / kTeam<D>;
-  const uint32_t teams = gridDim.x * blockDim.x / kTeam<D>;
-  const uint32_t counts = m.words[kMlTop + min(lane, kMaxLevel)];   // lane l: level l
-  uint32_t some = __ballot_sync(0xffffffffu, counts != 0 && lane < lmax);   // levels with nodes
-  auto load = [&](int l, uint32_t i, uint32_t cnt) {
-    const bool has = i < cnt;
-    return mono_load(has, has ? m.top[(size_t)l * m.per + i] : 0u, a);
-  };
-  if (!some) return;
-  int l = 31 - __clz(some);
-  uint32_t cnt = __shfl_sync(0xffffffffu, counts, l);
-  MonoNode v = load(l, team, cnt);
-  while (true) {
-    if (cnt >= kLaneLevel * teams) {
-      for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < cnt; i += gridDim.x * blockDim.x)
-        mono_internal_lane<D>(load(l, i, cnt), a);
-    } else {
-      mono_internal<D>(v, a);
-      for (uint32_t i = team + teams; i - lane / kTeam<D> < cnt; i += teams)
-        mono_internal<D>(load(l, i, cnt), a);
+  if (skip) list += *skip;
+  const uint32_t n = *listed, teams = gridDim.x * blockDim.x / kTeam<D>;
+  uint32_t i = (blockIdx.x * blockDim.x + threadIdx.x) / kTeam<D>;
+  MonoNode v = mono_load(i < n, i < n ? list[i] : 0u, a);
+  while (__any_sync(0xffffffffu, v.nch > 0)) {
+    const bool has = v.nch > 0, up = has && v.k != 0;
+    // the parent is read while the children's sums are added
+    const MonoNode p = mono_load(up, up ? v.parent : 0u, a);
+    const double sum = mono_sum<D>(v, a);
+    __syncwarp();   // the team's sums, before its count
+    int left = 0;
+    if (up && lane % kTeam<D> == 0) left = mono_done(&a.link[v.parent].x);
+    mono_node_records<D>(v, sum, a);   // not waited for by the parent
+    left = __shfl_sync(0xffffffffu, left, lane - lane % kTeam<D>);
+    __syncwarp();   // the siblings' sums, after the count
+    if (up && left == 1) {
+      v = p;
+    } else if (has) {
+      i += teams;
+      v = mono_load(i < n, i < n ? list[i] : 0u, a);
     }
-    some &= ~(1u << l);
-    if (!some) break;
-    // the next level's nodes are loaded before its children's sums are awaited
-    l = 31 - __clz(some);
-    cnt = __shfl_sync(0xffffffffu, counts, l);
-    v = load(l, team, cnt);
-    cluster.sync();
   }
 }
 
@@ -764,15 +734,23 @@ k_mono_top(int lmax, MonoArgs a, MonoLists m) {
 // warp instruction costs the same with idle lanes. In Morton order the
 // leaves of a warp hold 1 to leaf_size bodies and a warp ran 2.5 times the
 // iterations its bodies need (2^24 clustered bodies, leaf 32); binned, the
-// threads of a warp have equal loop counts. Each node is still summed by one
-// thread in its own order, so the results do not depend on the binning. At
-// these sizes a level's launch is filled by its nodes, and the subtrees' blocks
-// above wait on memory between their levels instead (3 M bodies, leaf 8,
-// D = 3: tiles and subtrees 701 us, this path 549 us).
+// threads of a warp have equal loop counts. Each leaf is still summed by one
+// thread in its own order, so the results do not depend on the binning.
+// Tiles are the better leaves below (their loads are coalesced and they need no
+// order first), this order above, where it keeps the FP64 pipe's lanes full.
+// Passes with tiles / in this order: a force on 131k bodies 664 / 676 us, a
+// 200k-body step 668 / 698 us, a force on 2 M bodies 5822 / 5755 us, a build of
+// 3 M bodies 1379 / 1182 us.
+// The ready internal nodes are as many again in this order, one per lane (an
+// FP64 instruction serves 32 of them), and what is above them goes to teams. A
+// launch per level (20 of them, most nearly empty, 10 to 20 us each for the
+// lower ones) took 221 us at 3 M bodies and three species; ready nodes, teams
+// and their share of the order take 150 us.
 static_assert(kMonoBins <= 256, "the bin scan takes one bin per thread of a 256-thread block");
 
-__device__ __forceinline__ int mono_bin(uint32_t lvl, uint32_t nch, uint32_t cnt) {
-  return nch == 0 ? (int)min(cnt, (uint32_t)(kLeafBins - 1)) : kLeafBins + (int)lvl * 8 + (int)nch - 1;
+// bin of node k, -1 for an internal node that is not ready (need > 0)
+__device__ __forceinline__ int mono_bin(uint32_t nch, int need, uint32_t cnt) {
+  return nch == 0 ? (int)min(cnt, (uint32_t)(kLeafBins - 1)) : need == 0 ? kLeafBins + (int)nch - 1 : -1;
 }
 
 // bins[0, kMonoBins): nodes per bin (zeroed before the launch)
@@ -783,7 +761,12 @@ __global__ void __launch_bounds__(256) k_mono_hist(MonoArgs a, uint32_t* bins) {
   __syncthreads();
   const uint32_t total = levels_of(a.status).start[kMaxLevel + 1];
   for (uint32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < total; k += gridDim.x * blockDim.x)
-    atomicAdd(&h[mono_bin(a.level[k], a.nchild[k], a.count[k])], 1u);
+  {
+    const uint32_t nch = a.nchild[k];
+    const int need = mono_pending(k, nch, a), bin = mono_bin(nch, need, a.count[k]);
+    if (nch) a.link[k].x = need;
+    if (bin >= 0) atomicAdd(&h[bin], 1u);
+  }
   __syncthreads();
   for (int i = threadIdx.x; i < kMonoBins; i += blockDim.x)
     if (h[i]) atomicAdd(&bins[i], h[i]);
@@ -814,13 +797,21 @@ __global__ void __launch_bounds__(256) k_mono_order(MonoArgs a, uint32_t* bins, 
   const uint32_t total = levels_of(a.status).start[kMaxLevel + 1];
   const uint32_t chunk = (total + gridDim.x - 1) / gridDim.x;
   const uint32_t k0 = min(total, blockIdx.x * chunk), k1 = min(total, k0 + chunk);
-  for (uint32_t k = k0 + tid; k < k1; k += blockDim.x)
-    atomicAdd(&lh[mono_bin(a.level[k], a.nchild[k], a.count[k])], 1u);
+  auto bin_of = [&](uint32_t k) {
+    const uint32_t nch = a.nchild[k];
+    return mono_bin(nch, mono_pending(k, nch, a), a.count[k]);
+  };
+  for (uint32_t k = k0 + tid; k < k1; k += blockDim.x) {
+    const int bin = bin_of(k);
+    if (bin >= 0) atomicAdd(&lh[bin], 1u);
+  }
   __syncthreads();
   if (tid < kMonoBins && lh[tid]) base[tid] += atomicAdd(&bins[kMonoBins + tid], lh[tid]);
   __syncthreads();
-  for (uint32_t k = k0 + tid; k < k1; k += blockDim.x)
-    order[atomicAdd(&base[mono_bin(a.level[k], a.nchild[k], a.count[k])], 1u)] = k;
+  for (uint32_t k = k0 + tid; k < k1; k += blockDim.x) {
+    const int bin = bin_of(k);
+    if (bin >= 0) order[atomicAdd(&base[bin], 1u)] = k;
+  }
 }
 
 // Sums of leaf k: its bodies into the node's FP64 monopoles and FP32 walk
@@ -889,54 +880,57 @@ __global__ void __launch_bounds__(kMonoThreads) k_mono_leaves(MonoArgs a, const 
     mono_leaf<D>(order[i], a, lacc, threadIdx.x);
 }
 
-// The internal nodes of level lvl (their children are done).
+// The ready nodes, one per lane; the parents they complete are listed behind
+// the order for k_mono_up.
 template <int D>
-__global__ void __launch_bounds__(kMonoThreads) k_mono_internal(int lvl, MonoArgs a,
-                                                                const uint32_t* __restrict__ bins,
-                                                                const uint32_t* __restrict__ order) {
+__global__ void __launch_bounds__(kMonoThreads) k_mono_ready(MonoArgs a, const uint32_t* __restrict__ bins,
+                                                             uint32_t* order, uint32_t* words) {
   if (a.status[ST_FLAGS] & SF_NODE_OVERFLOW) return;
-  const uint32_t* start = bins + 2 * kMonoBins + kLeafBins + lvl * 8;
-  const uint32_t s = start[0], e = start[8];
-  for (uint32_t i = s + blockIdx.x * blockDim.x + threadIdx.x; i < e; i += gridDim.x * blockDim.x)
-    mono_internal_lane<D>(mono_load(true, order[i], a), a);
+  const uint32_t s = bins[2 * kMonoBins + kLeafBins], e = bins[3 * kMonoBins];
+  const int lane = threadIdx.x & 31;
+  for (uint32_t i0 = s + blockIdx.x * blockDim.x + (threadIdx.x & ~31); i0 < e; i0 += gridDim.x * blockDim.x) {
+    const bool has = i0 + lane < e;
+    const MonoNode v = mono_load(has, has ? order[i0 + lane] : 0u, a);
+    mono_internal_lane<D>(v, a);
+    const bool last = has && v.k != 0 && mono_done(&a.link[v.parent].x) == 1;
+    const uint32_t m = __ballot_sync(0xffffffffu, last);
+    uint32_t at = 0;
+    if (lane == 0 && m) at = atomicAdd(&words[kMlNext], (uint32_t)__popc(m));
+    at = e + __shfl_sync(0xffffffffu, at, 0) + __popc(m & ((1u << lane) - 1u));
+    if (last) order[at] = v.parent;
+  }
 }
 
 template <int D>
-static int launch_monopoles(ng_ctx* c, const MonoArgs& a, const MonoLists& m, int lmax) {
+static int launch_monopoles(ng_ctx* c, const MonoArgs& a) {
+  uint32_t* words = as<uint32_t>(c->mono_words);
+  uint32_t* order = as<uint32_t>(c->n_tmp);
   if (c->n < kBinnedMonoBodies) {
     const int64_t tiles = (c->n + kLeafTile - 1) / kLeafTile;
-    k_mono_tiles<D><<<(int)std::min<int64_t>((int64_t)c->nsm * 16, tiles), kLeafThreads, 0, c->stream>>>(a, m);
+    k_mono_tiles<D><<<(int)std::min<int64_t>((int64_t)c->nsm * 16, tiles), kLeafThreads, 0, c->stream>>>(a, words, order);
     c->launches += 1;
     if (c->n > c->p.leaf_size) {   // else the root is a leaf
-      // at most eight subtrees under a top node
-      const int64_t subs = 8 * ((c->n + m.sub - 1) / m.sub);
-      k_mono_subtrees<D><<<(int)std::min<int64_t>((int64_t)c->nsm * 16, subs), kMonoThreads, 0, c->stream>>>(a, m);
+      // a ready node holds more than leaf_size bodies
+      const int64_t teams = c->n / (c->p.leaf_size + 1);
+      const int64_t blocks = (teams * kTeam<D> + kMonoThreads - 1) / kMonoThreads;
+      k_mono_up<D><<<(int)std::min<int64_t>((int64_t)c->nsm * 16, blocks), kMonoThreads, 0, c->stream>>>(
+          a, order, nullptr, words + kMlReady);
       c->launches += 1;
-      if (c->n > m.sub) {
-        k_mono_top<D><<<kClusterBlocks, 512, 0, c->stream>>>(lmax, a, m);
-        c->launches += 1;
-      }
     }
     NG_CUDA(c, cudaGetLastError());
     return NG_OK;
   }
-  uint32_t* bins = as<uint32_t>(c->mono_words) + kMonoWords;
-  uint32_t* order = as<uint32_t>(c->n_tmp);
+  uint32_t* bins = words + kMonoWords;
   NG_CUDA(c, cudaMemsetAsync(bins, 0, 2 * kMonoBins * sizeof(uint32_t), c->stream));
   const int64_t cap = std::min<int64_t>(c->cap_nodes, 2 * c->n + 64);
   const int sgrid = work_grid(c, cap, 4);
   k_mono_hist<<<sgrid, 256, 0, c->stream>>>(a, bins);
   k_mono_order<<<sgrid, 256, 0, c->stream>>>(a, bins, order);
-  auto grid = [&](int64_t nodes) {
-    return (int)std::max<int64_t>(
-        1, std::min<int64_t>((int64_t)c->nsm * 16, (nodes + kMonoThreads - 1) / kMonoThreads));
-  };
-  k_mono_leaves<D><<<grid(cap), kMonoThreads, 0, c->stream>>>(a, bins, order);
-  // nodes at level lmax are leaves; a level holds at most 8^l nodes
-  for (int l = lmax - 1; l >= 0; --l)
-    k_mono_internal<D><<<grid(std::min<int64_t>(cap, (int64_t)1 << std::min(3 * l, 40))), kMonoThreads, 0,
-                         c->stream>>>(l, a, bins, order);
-  c->launches += 3 + lmax;
+  const int grid = (int)std::min<int64_t>((int64_t)c->nsm * 16, (cap + kMonoThreads - 1) / kMonoThreads);
+  k_mono_leaves<D><<<grid, kMonoThreads, 0, c->stream>>>(a, bins, order);
+  k_mono_ready<D><<<grid, kMonoThreads, 0, c->stream>>>(a, bins, order, words);
+  k_mono_up<D><<<grid, kMonoThreads, 0, c->stream>>>(a, order, bins + 3 * kMonoBins, words + kMlNext);
+  c->launches += 5;
   NG_CUDA(c, cudaGetLastError());
   return NG_OK;
 }
@@ -965,18 +959,14 @@ int reduce_monopoles(ng_ctx* c) {
   a.invL = 1.0 / c->L;
   a.L = c->L;
   a.unit = c->L == 1.0;
-  // the per-level tree scratch and the node scratch are free once the tree is built
-  MonoLists m{as<uint32_t>(c->mono_words), as<uint32_t>(c->n_tmp), as<uint32_t>(c->tree_cnt),
-              mono_sub(c->n), (uint32_t)(c->n / mono_sub(c->n) + 1)};
-  const int lmax = std::min(std::max(c->level_cap, 0), kMaxLevel);   // deeper levels are empty
   stage_mark(c, NG_STAGE_MONOPOLES);
   switch (c->p.D) {
-    case 1: return launch_monopoles<1>(c, a, m, lmax);
-    case 2: return launch_monopoles<2>(c, a, m, lmax);
-    case 3: return launch_monopoles<3>(c, a, m, lmax);
-    case 4: return launch_monopoles<4>(c, a, m, lmax);
-    case 5: return launch_monopoles<5>(c, a, m, lmax);
-    default: return launch_monopoles<6>(c, a, m, lmax);
+    case 1: return launch_monopoles<1>(c, a);
+    case 2: return launch_monopoles<2>(c, a);
+    case 3: return launch_monopoles<3>(c, a);
+    case 4: return launch_monopoles<4>(c, a);
+    case 5: return launch_monopoles<5>(c, a);
+    default: return launch_monopoles<6>(c, a);
   }
 }
 
