@@ -560,162 +560,109 @@ __global__ void k_gather(GatherArgs g, const uint32_t* __restrict__ perm) {
 
 // ------------------------------------------------------- small problems
 
-// The whole sort stage of up to 1024 * ITEMS bodies in one launch of one
-// block: keys, the radix passes in shared memory, the gather and the
-// type-major order. At these sizes every launch of the general path costs more
-// than its work (4096 bodies: keys, 8 passes, gather and type order 81 us in 11
-// launches, 46 us here). Bodies past n take the largest key and end last.
-constexpr int kSmThreads = 1024, kSmWarps = kSmThreads / 32;
-constexpr int kSmRow = 257;   // words per warp of digit counts (a bank apart per row)
+// The whole sort stage of up to kSmallSort bodies in one launch: a body's
+// sorted place is the number of keys below its own (and of equal keys of lower
+// index, so the order is that of the stable passes), counted by comparing it
+// with every key; its place in the type-major order counts those of its own
+// species. At these sizes a radix pass costs far more than its work: 4096
+// bodies take 81 us of kernels in the 11 launches of the general path, and one
+// block with the passes in shared memory took 44 us on one SM; this takes 20.
+// The n^2 comparisons, five instructions each over the whole chip, set the limit.
+// Each block forms all keys (the bodies are read from L2) and ranks 32 * ITEMS
+// bodies, one per lane and item; its warps share out the keys they are compared with.
+constexpr int kRkThreads = 512, kRkWarps = kRkThreads / 32;
+constexpr int kRkPad = 4 * kRkWarps;   // keys are padded to whole quads per warp
 constexpr int64_t kSmallSort = 8192;
 
-template <int ITEMS>
-struct SmSmem {
-  uint64_t tk[kSmThreads * ITEMS];
-  uint32_t tv[kSmThreads * ITEMS];
-  uint32_t wcnt[kSmWarps * kSmRow];
-  uint32_t wsum[kSmWarps];
-  uint32_t species[8];
-};
+static size_t rank_smem(int64_t n) { return (size_t)((n + kRkPad - 1) / kRkPad * kRkPad) * 12; }
 
 template <int ITEMS, bool RESIDENT>
-__global__ void __launch_bounds__(kSmThreads)
-k_sort_small(KeyArgs a, GatherArgs g, int first, uint64_t* __restrict__ keys,
-             uint32_t* __restrict__ perm, uint32_t* words, uint32_t* __restrict__ tperm) {
-  extern __shared__ __align__(16) unsigned char sm_raw[];
-  SmSmem<ITEMS>& sm = *reinterpret_cast<SmSmem<ITEMS>*>(sm_raw);
+__global__ void __launch_bounds__(kRkThreads)
+k_sort_rank(KeyArgs a, GatherArgs g, int first, uint64_t* __restrict__ keys,
+            uint32_t* __restrict__ perm, uint32_t* words, uint32_t* __restrict__ tperm) {
+  extern __shared__ __align__(16) unsigned char rk_raw[];
+  __shared__ uint32_t rank[32 * ITEMS], trank[32 * ITEMS], species[8];
+  const int n = (int)a.n, npad = (n + kRkPad - 1) / kRkPad * kRkPad;
+  uint64_t* sk = reinterpret_cast<uint64_t*>(rk_raw);          // keys, the sorted digits only
+  uint32_t* st = reinterpret_cast<uint32_t*>(sk + npad);       // species
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-  const uint32_t lt = (1u << lane) - 1u;
-  const int i0 = w * (32 * ITEMS) + lane;   // item it of the thread: body i0 + 32 it
-  uint64_t k[ITEMS];
-  uint32_t v[ITEMS], rank[ITEMS];
+  const int b0 = blockIdx.x * 32 * ITEMS, b1 = b0 + 32 * ITEMS;
+  for (int j = tid; j < 32 * ITEMS; j += kRkThreads) rank[j] = trank[j] = 0;
+  if (tid < 8) species[tid] = 0;
+  __syncthreads();
+#pragma unroll 2
+  for (int j0 = 0; j0 < npad; j0 += kRkThreads) {   // whole warps: npad is a multiple of 64
+    const int j = j0 + tid;
+    if (j0 + (tid & ~31) >= npad) break;
+    uint32_t t = 8;
+    uint64_t k = ~0ull;                             // behind every key
+    if (j < n) {
+      const uint8_t ty = a.type[j];
+      k = body_key(a, j, ty) >> (8 * first);
+      t = stored_type(ty, a.D);
+    }
+    sk[j] = k;
+    st[j] = t;
+    for (int q = 0; q < a.D; ++q) {
+      const uint32_t m = __ballot_sync(0xffffffffu, t == (uint32_t)q);
+      if (lane == 0 && m) atomicAdd(&species[q], (uint32_t)__popc(m));
+    }
+  }
+  __syncthreads();
+  uint64_t key[ITEMS];
+  uint32_t ty[ITEMS], r[ITEMS], tr[ITEMS];
 #pragma unroll
   for (int it = 0; it < ITEMS; ++it) {
-    const int i = i0 + it * 32;
-    v[it] = (uint32_t)i;
-    k[it] = i < a.n ? body_key(a, i, a.type[i]) : ~0ull;
+    const int i = min(b0 + it * 32 + lane, n - 1);
+    key[it] = sk[i];
+    ty[it] = st[i];
+    r[it] = tr[it] = 0;
   }
-  for (int p = first; p < 8; ++p) {
-    const int shift = 8 * p;
-    for (int j = tid; j < kSmWarps * kSmRow; j += kSmThreads) sm.wcnt[j] = 0;
-    __syncthreads();
-    uint32_t* cnt = sm.wcnt + w * kSmRow;
+  // keys j before the block's bodies count when not above, those behind when below
+  auto count = [&](int j, auto below) {
+    const ulonglong2 ka = *reinterpret_cast<const ulonglong2*>(sk + j);
+    const ulonglong2 kb = *reinterpret_cast<const ulonglong2*>(sk + j + 2);
+    const uint4 t = *reinterpret_cast<const uint4*>(st + j);
+    const uint64_t kj[4] = {ka.x, ka.y, kb.x, kb.y};
+    const uint32_t tj[4] = {t.x, t.y, t.z, t.w};
 #pragma unroll
-    for (int h = 0; h < ITEMS; h += 4) {
-      uint32_t peers[4];
+    for (int u = 0; u < 4; ++u)
 #pragma unroll
-      for (int j = 0; j < 4; ++j) peers[j] = digit_peers((uint32_t)(k[h + j] >> shift) & 0xffu, 0xffffffffu);
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const uint32_t d = (uint32_t)(k[h + j] >> shift) & 0xffu;
-        const uint32_t prior = cnt[d];
-        __syncwarp();
-        rank[h + j] = prior + __popc(peers[j] & lt);
-        if ((peers[j] & lt) == 0) cnt[d] = prior + __popc(peers[j]);
-        __syncwarp();
+      for (int it = 0; it < ITEMS; ++it) {
+        const bool lt = kj[u] < below(it, j + u);
+        r[it] += lt ? 1u : 0u;
+        tr[it] += lt && tj[u] == ty[it] ? 1u : 0u;
       }
-    }
-    __syncthreads();
-    {
-      // four threads per digit, eight warps' counts each: the digit's total,
-      // its start (scan over digits) and each warp's place in its run
-      const int d = tid >> 2, seg = tid & 3;
-      uint32_t c[8], sum = 0;
+  };
+  const int per = npad / kRkWarps, js = w * per, je = js + per;   // multiples of 4
+  uint64_t next[ITEMS];   // keys are below 2^63: no overflow
 #pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        c[j] = sm.wcnt[(seg * 8 + j) * kSmRow + d];
-        sum += c[j];
-      }
-      uint32_t incl = sum;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += t;
-      }
-      if (lane == 31) sm.wsum[w] = incl;
-      __syncthreads();
-      uint32_t base = sm.wsum[lane];   // exclusive over the warps
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t t = __shfl_up_sync(0xffffffffu, base, o);
-        if (lane >= o) base += t;
-      }
-      base = __shfl_sync(0xffffffffu, base, w) - sm.wsum[w];
-      uint32_t run = base + incl - sum;
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        sm.wcnt[(seg * 8 + j) * kSmRow + d] = run;
-        run += c[j];
-      }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int it = 0; it < ITEMS; ++it) {
-      const uint32_t at = cnt[(uint32_t)(k[it] >> shift) & 0xffu] + rank[it];
-      sm.tk[at] = k[it];
-      sm.tv[at] = v[it];
-    }
-    __syncthreads();
-#pragma unroll
-    for (int it = 0; it < ITEMS; ++it) {
-      k[it] = sm.tk[i0 + it * 32];
-      v[it] = sm.tv[i0 + it * 32];
-    }
-  }
-  if (tid < 8) sm.species[tid] = 0;
-  uint32_t* chunk = sm.wcnt;   // [8][32 ITEMS]: bodies per species and chunk, then positions
-  constexpr int kChunks = 32 * ITEMS;
-  __syncthreads();
-  int ty[ITEMS];
+  for (int it = 0; it < ITEMS; ++it) next[it] = key[it] + 1;
+#pragma unroll 2
+  for (int j = js; j < min(je, b0); j += 4) count(j, [&](int it, int) { return next[it]; });
+  for (int j = max(js, b0); j < min(je, b1); j += 4)
+    count(j, [&](int it, int jj) { return jj < b0 + it * 32 + lane ? next[it] : key[it]; });
+#pragma unroll 2
+  for (int j = max(js, b1); j < je; j += 4) count(j, [&](int it, int) { return key[it]; });
 #pragma unroll
   for (int it = 0; it < ITEMS; ++it) {
-    const int i = i0 + it * 32;
-    ty[it] = -1;
-    if (i < a.n) {
-      keys[i] = k[it];
-      perm[i] = v[it];
-      if (RESIDENT) gather_resident(g, i, v[it]);
-      else gather_plain(g, i, v[it]);
-      ty[it] = (int)stored_type(a.type[v[it]], a.D);
-    }
-    rank[it] = 0;
-    for (int t = 0; t < a.D; ++t) {
-      const uint32_t m = __ballot_sync(0xffffffffu, ty[it] == t);
-      if (ty[it] == t) rank[it] = __popc(m & lt);
-      if (lane == 0) chunk[t * kChunks + w * ITEMS + it] = __popc(m);
-    }
+    atomicAdd(&rank[it * 32 + lane], r[it]);
+    atomicAdd(&trank[it * 32 + lane], tr[it]);
   }
   __syncthreads();
-  uint32_t c[ITEMS], incl = 0, sum = 0;
-  if (w < a.D) {   // warp w: species w, chunks in order
-#pragma unroll
-    for (int j = 0; j < ITEMS; ++j) {
-      c[j] = chunk[w * kChunks + lane * ITEMS + j];
-      sum += c[j];
-    }
-    incl = sum;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += t;
-    }
-    if (lane == 31) sm.species[w] = incl;
+  for (int b = tid; b < 32 * ITEMS; b += kRkThreads) {
+    const int i = b0 + b;
+    if (i >= n) break;
+    const uint32_t k = rank[b], t = st[i];
+    keys[k] = body_key(a, i, a.type[i]);
+    perm[k] = (uint32_t)i;
+    if (RESIDENT) gather_resident(g, k, (uint32_t)i);
+    else gather_plain(g, k, (uint32_t)i);
+    uint32_t at = trank[b];
+    for (uint32_t q = 0; q < t; ++q) at += species[q];
+    tperm[at] = k;
   }
-  __syncthreads();
-  if (w < a.D) {
-    uint32_t run = incl - sum;
-    for (int t = 0; t < w; ++t) run += sm.species[t];
-#pragma unroll
-    for (int j = 0; j < ITEMS; ++j) {
-      chunk[w * kChunks + lane * ITEMS + j] = run;
-      run += c[j];
-    }
-  }
-  if (tid < 8) words[kSwTypes + tid] = sm.species[tid];
-  __syncthreads();
-#pragma unroll
-  for (int it = 0; it < ITEMS; ++it)
-    if (ty[it] >= 0) tperm[chunk[ty[it] * kChunks + w * ITEMS + it] + rank[it]] = (uint32_t)(i0 + it * 32);
+  if (blockIdx.x == 0 && tid < 8) words[kSwTypes + tid] = species[tid];
 }
 
 int work_grid(ng_ctx* c, int64_t items, int per_sm) {
@@ -746,11 +693,12 @@ int reserve_sort(ng_ctx* c, int64_t n) {
 }
 
 template <int ITEMS, bool RESIDENT>
-static int sort_small(ng_ctx* c, const KeyArgs& a, const GatherArgs& g, int first) {
-  const size_t smem = sizeof(SmSmem<ITEMS>);
-  NG_CUDA(c, cudaFuncSetAttribute(k_sort_small<ITEMS, RESIDENT>,
-                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  k_sort_small<ITEMS, RESIDENT><<<1, kSmThreads, smem, c->stream>>>(
+static int sort_rank(ng_ctx* c, const KeyArgs& a, const GatherArgs& g, int first) {
+  const size_t smem = rank_smem(a.n);
+  NG_CUDA(c, cudaFuncSetAttribute(k_sort_rank<ITEMS, RESIDENT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)rank_smem(kSmallSort)));
+  const int grid = (int)((a.n + 32 * ITEMS - 1) / (32 * ITEMS));
+  k_sort_rank<ITEMS, RESIDENT><<<grid, kRkThreads, smem, c->stream>>>(
       a, g, first, as<uint64_t>(c->keys_a), as<uint32_t>(c->vals_a), as<uint32_t>(c->sort_words),
       as<uint32_t>(c->tperm));
   c->launches += 1;
@@ -782,7 +730,8 @@ static int sort_stage(ng_ctx* c, const GatherArgs& g) {
   const KeyArgs a{n, g.pos, g.type, g.L, g.invL, g.pow2, g.pow2 ? std::ilogb(c->L) : 0, c->p.D};
   if (n <= kSmallSort) {
     stage_mark(c, NG_STAGE_KEYS);
-    return n <= 4 * kSmThreads ? sort_small<4, RESIDENT>(c, a, g, first) : sort_small<8, RESIDENT>(c, a, g, first);
+    // at most 128 blocks: one round on the SMs
+    return n <= kSmallSort / 2 ? sort_rank<1, RESIDENT>(c, a, g, first) : sort_rank<2, RESIDENT>(c, a, g, first);
   }
   const int64_t lbw = rs_lb_words(n), lbt = 8 * to_tiles(n);
   uint64_t* lb = as<uint64_t>(c->lookback);

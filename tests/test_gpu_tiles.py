@@ -83,3 +83,29 @@ def test_state_returns_to_caller_order(ng, n):
     assert np.array_equal(pos.cpu().numpy(), x - np.floor(x))
     assert np.array_equal(vel.cpu().numpy(), v0)
     assert np.all(acc.cpu().numpy() == 0)
+
+
+@pytest.mark.parametrize("n,D", [(31, 1), (32, 6), (33, 2), (63, 3), (65, 4), (2047, 6), (4095, 1), (4096, 3),
+                                 (8191, 2), (8192, 6), (8193, 5)])
+def test_small_sort_at_its_edges(ng, n, D):
+    """Sorts by counting (up to 8192 bodies, in blocks of 32 or 64) and the
+    first size past them: duplicates keep their order."""
+    import torch
+    w = small_clustered(n, D, 500 + n)
+    w["pos"][:, ::3] = w["pos"][:, :1]          # a third of the bodies in one place
+    prm = w["params"]
+    pos, typ, mass = device_arrays(w)
+    sim = ng.Simulation(ng_params(prm))
+    keys = torch.empty(n, dtype=torch.int64, device=pos.device)
+    perm = torch.empty(n, dtype=torch.int32, device=pos.device)
+    order = torch.empty(n, dtype=torch.int32, device=pos.device)
+    ng.ng_build_tree(sim.ctx, pos, typ, mass, keys, perm)
+    offs = ng.ng_type_order(sim.ctx, D, order)
+    sim.close()
+    k_ref = oracle.keys(w["pos"], w["type"])
+    p_ref = np.argsort(k_ref, kind="stable").astype(np.uint32)
+    assert np.array_equal(perm.cpu().numpy().view(np.uint32), p_ref)
+    assert np.array_equal(keys.cpu().numpy().view(np.uint64), k_ref[p_ref])
+    assert np.array_equal(order.cpu().numpy().view(np.uint32),
+                          p_ref[np.argsort(w["type"][p_ref], kind="stable")])
+    assert np.array_equal(offs, np.concatenate([[0], np.cumsum(np.bincount(w["type"], minlength=D))]))
