@@ -367,6 +367,8 @@ int build_checked(ng_ctx* c, int64_t n, const double* pos, const uint8_t* type,
   c->built = false;
   NG_TRY(alloc_bodies(c, n));
   NG_CUDA(c, cudaMemsetAsync(c->status.p, 0, ST_COUNT * 4, c->stream));
+  // records of the sort (not needed for it: without them it gathers unpacked)
+  if (n >= kPackBodies && ensure(c, c->rpack, (size_t)n * 32) != NG_OK) c->err.clear();
   NG_TRY(sort_bodies(c, n, pos, type, mass));
   return tree_checked(c);
 }

@@ -27,6 +27,7 @@ constexpr int kMonoWords = 2;   // counters of the monopole stage
 constexpr int kLeafBins = 66;
 constexpr int kMonoBins = kLeafBins + 8;
 constexpr int64_t kBinnedMonoBodies = 1 << 20;
+constexpr int64_t kPackBodies = 1 << 17;   // sorts gather packed records (ng_sort.cu)
 constexpr int kWarp = 32;
 
 // Status words in device memory (ctx->status).

@@ -109,3 +109,29 @@ def test_small_sort_at_its_edges(ng, n, D):
     assert np.array_equal(order.cpu().numpy().view(np.uint32),
                           p_ref[np.argsort(w["type"][p_ref], kind="stable")])
     assert np.array_equal(offs, np.concatenate([[0], np.cumsum(np.bincount(w["type"], minlength=D))]))
+
+
+@pytest.mark.parametrize("n", [300, 20000, 131071, 131072, 131101])
+def test_bodies_outside_the_box_and_bad_species(ng, n):
+    """Every path of the sort (counting, radix passes, packed records from 131072
+    bodies) wraps positions as the keys do and refuses a species out of range,
+    after which the context takes good input."""
+    import torch
+    w = small_clustered(n, 3, 600 + n % 101)
+    rng = inputs.rng_for(n + 1)
+    w["pos"] = w["pos"] + rng.integers(-2, 3, w["pos"].shape)
+    pos, typ, mass = device_arrays(w)
+    bad = typ.clone()
+    bad[n // 2] = 3
+    sim = ng.Simulation(ng_params(w["params"]))
+    keys = torch.empty(n, dtype=torch.int64, device=pos.device)
+    with pytest.raises(ng.NgError):
+        ng.ng_build_tree(sim.ctx, pos, bad, mass)
+    ng.ng_build_tree(sim.ctx, pos, typ, mass, keys)
+    T = ng.ng_tree_export(sim.ctx, 3)
+    sim.close()
+    assert np.array_equal(keys.cpu().numpy().view(np.uint64), np.sort(oracle.keys(w["pos"], w["type"])))
+    R = oracle.tree(oracle_params(w["params"]), w["pos"], w["type"], w["mass"])
+    assert np.array_equal(T["cnt"], R["cnt"].astype(T["cnt"].dtype))
+    bound = 2.0 ** -53 * 4 * (R["cnt"].astype(np.float64) + 2)
+    assert np.all(np.abs(T["com"] - R["com"]).max(axis=2) <= bound)
