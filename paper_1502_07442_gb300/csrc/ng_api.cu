@@ -306,6 +306,8 @@ int alloc_bodies(ng_ctx* c, int64_t n) {
   NG_TRY(ensure(c, c->bleaf, n * 4));
   NG_TRY(ensure(c, c->groups, n * 8));
   NG_TRY(ensure(c, c->tree_cnt, tree_scratch_bytes(n)));
+  NG_TRY(ensure(c, c->gsize, (size_t)n * sizeof(uint32_t)));
+  NG_TRY(ensure(c, c->group_lb, group_lookback_bytes(n)));
   if (c->p.pure_tree) NG_TRY(ensure(c, c->exact_body, n * 32));
   NG_TRY(ensure(c, c->status, ST_COUNT * 4));
   NG_TRY(ensure(c, c->counter, 8));
@@ -320,7 +322,6 @@ int reserve(ng_ctx* c, int64_t n) {
   NG_TRY(alloc_nodes(c, std::max<int64_t>(c->cap_nodes, n + 1024)));
   NG_TRY(reserve_sort(c, n));
   NG_TRY(ensure(c, c->gsize, (size_t)n * sizeof(uint32_t)));
-  NG_TRY(ensure(c, c->grank, (size_t)n * sizeof(uint32_t)));
   NG_TRY(ensure(c, c->walk_desc, sizeof(WalkDesc)));
   NG_TRY(ensure(c, c->walk_prefix, 4 * sizeof(uint32_t)));
   if (c->p.opening == NG_OPEN_RELATIVE) NG_TRY(ensure(c, c->aold, (size_t)n * sizeof(float)));
@@ -801,7 +802,7 @@ int ng_destroy(ng_ctx* c) {
                     &c->tperm, &c->scan_part, &c->n_level, &c->n_prefix, &c->n_first,
                     &c->n_count, &c->n_child, &c->n_nchild, &c->n_tmp, &c->n_m64,
                     &c->n_cnt, &c->n_geo, &c->n_com, &c->n_link, &c->n_mono, &c->exact_node, &c->exact_body, &c->mono_words,
-                    &c->tree_cnt, &c->groups, &c->gsize, &c->grank,
+                    &c->tree_cnt, &c->groups, &c->gsize, &c->group_lb,
                     &c->status, &c->counter, &c->aold, &c->io_pos, &c->io_vel, &c->io_type, &c->io_mass,
                     &c->io_acc, &c->lattice, &c->rho, &c->rhok, &c->phi,
                     &c->walk_desc, &c->walk_prefix, &c->spos_alt, &c->smass_alt, &c->stype_alt,

@@ -19,7 +19,7 @@ namespace ng {
 constexpr int kMaxD = NG_MAX_SPECIES;
 constexpr int kMaxLevel = 20;           // 20 Morton bits per axis
 constexpr int kCapturedDepthMargin = 2;  // captured steps build this far below the depth seen
-constexpr int kMonoWords = 2;   // counters of the monopole stage
+constexpr int kMonoWords = 3;   // counters of the monopole stage, ticket of the group stage
 // Monopoles of trees of kBinnedMonoBodies bodies or more take their leaves and
 // ready internal nodes in an order binned by the work of a node: leaves by body
 // count (0..64, one more bin for the larger leaves of a tree stopped at a level
@@ -289,7 +289,7 @@ struct ng_ctx {
   ng::DevBuf mono_words;   // uint32[kMonoWords + 3 kMonoBins + 1]: counters and bins of the monopole stage
   ng::DevBuf tree_cnt;    // uint32[levels][tiles]: node counts of the tree build
   ng::DevBuf groups;
-  ng::DevBuf gsize, grank;          // group size at its first body, rank of each group start
+  ng::DevBuf gsize, group_lb;       // group size at its first body, look-back state of the group list
   ng::DevBuf status;     // uint32[ST_COUNT]
   ng::DevBuf walk_desc, walk_prefix;
   ng::DevBuf counter;    // unsigned long long
@@ -375,7 +375,6 @@ inline T* as(const DevBuf& b) { return static_cast<T*>(b.p); }
 // Device-wide exclusive scan of uint32 values; len read from *d_len when
 // d_len != nullptr (then len is an upper bound), total written to *d_total
 // when non-null. Needs ctx->scan_part scratch.
-int scan_u32_flags(ng_ctx* c, const uint32_t* in, uint32_t* out, int64_t len, uint32_t* d_total);
 int scan_u32(ng_ctx* c, const uint32_t* in, uint32_t* out, int64_t len,
              const uint32_t* d_len, uint32_t* d_total);
 
@@ -397,6 +396,7 @@ int resident_store(ng_ctx* c, int64_t n, double* pos, float* vel, float* acc);
 int resident_step_once(ng_ctx* c, int64_t n, double dt, bool checked);
 int build_octree(ng_ctx* c);                  // needs sorted bodies
 size_t tree_scratch_bytes(int64_t n);         // tree_cnt for n bodies
+size_t group_lookback_bytes(int64_t n);       // group_lb for n bodies
 int reduce_monopoles(ng_ctx* c);              // needs octree
 int build_groups(ng_ctx* c);                  // needs octree
 int launch_walk(ng_ctx* c, float* acc, bool accumulate, bool count);
@@ -499,6 +499,49 @@ __device__ __forceinline__ uint32_t block_inclusive_scan(uint32_t v, uint32_t* w
   __syncthreads();
   if (wid > 0) v += warp_tot[wid - 1];
   return v;
+}
+
+// Look-back over tiles that a launch works through in ticket order: each tile
+// publishes its count, then its prefix. State of a tile: 0, or a flag in the
+// top bits and a count below (64 bits: counts up to the largest n).
+constexpr uint64_t kLbAggregate = 1ull << 62, kLbPrefix = 2ull << 62, kLbCount = (1ull << 62) - 1;
+
+__device__ __forceinline__ uint64_t lb_load(const uint64_t* p) {
+  uint64_t v;
+  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ void lb_store(uint64_t* p, uint64_t v) {
+  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+// Polls of one state before a tile stops waiting and counts what lies before it
+// from the input itself. Tiles are numbered by ticket, so the tile waited
+// for always runs and never waits for this one; the limit only bounds the wait.
+constexpr int kLbPolls = 1 << 20;
+
+// Count of all tiles before `tile`, by one warp (32 states per load); the state
+// of tile t at lb[t * stride]. recount: the calling lane's share of that count,
+// taken from the input.
+template <class Recount>
+__device__ __forceinline__ uint64_t lb_before(const uint64_t* lb, int stride, int64_t tile,
+                                              Recount recount) {
+  const int lane = threadIdx.x & 31;
+  uint64_t before = 0;
+  int polls = 0;
+  for (int64_t t = tile - 1; t >= 0;) {
+    // lane j: the state of tile t - j; add up to the nearest prefix
+    const uint64_t s = t - lane >= 0 ? lb_load(&lb[(t - lane) * stride]) : kLbPrefix;
+    const uint32_t pre = __ballot_sync(0xffffffffu, (s & kLbPrefix) != 0);
+    const uint32_t use = pre ? (pre & -pre) | ((pre & -pre) - 1u) : 0xffffffffu;
+    const bool wait = (__ballot_sync(0xffffffffu, s == 0) & use) != 0;
+    if (wait && ++polls < kLbPolls) continue;
+    uint64_t add = wait ? recount() : (use >> lane & 1u) ? s & kLbCount : 0;
+    for (int o = 16; o; o >>= 1) add += __shfl_xor_sync(0xffffffffu, add, o);
+    before = wait ? add : before + add;
+    if (wait || pre) break;
+    t -= 32;
+  }
+  return before;
 }
 
 // Blocks of 256 threads for a grid-stride kernel over `items` items: enough

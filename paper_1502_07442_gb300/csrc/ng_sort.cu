@@ -20,13 +20,13 @@ __device__ __forceinline__ int64_t scan_len(int64_t bound, const uint32_t* d_len
 
 __global__ void __launch_bounds__(kScanThreads)
 k_scan_partial(const uint32_t* __restrict__ in, int64_t bound, const uint32_t* d_len,
-               uint32_t* part, int as_flags) {
+               uint32_t* part) {
   const int64_t len = scan_len(bound, d_len);
   const int64_t chunk = (len + gridDim.x - 1) / gridDim.x;
   const int64_t b0 = (int64_t)blockIdx.x * chunk;
   const int64_t b1 = b0 + chunk < len ? b0 + chunk : len;
   uint32_t s = 0;
-  for (int64_t i = b0 + threadIdx.x; i < b1; i += blockDim.x) s += as_flags ? (in[i] != 0u) : in[i];
+  for (int64_t i = b0 + threadIdx.x; i < b1; i += blockDim.x) s += in[i];
 #pragma unroll
   for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
   __shared__ uint32_t ws[32];
@@ -42,7 +42,7 @@ k_scan_partial(const uint32_t* __restrict__ in, int64_t bound, const uint32_t* d
 
 __global__ void __launch_bounds__(kScanThreads)
 k_scan_final(const uint32_t* in, uint32_t* out, int64_t bound, const uint32_t* d_len,
-             const uint32_t* __restrict__ part, uint32_t* d_total, int as_flags) {
+             const uint32_t* __restrict__ part, uint32_t* d_total) {
   __shared__ uint32_t warp_tot[32];
   __shared__ uint32_t tile_total;
   __shared__ uint32_t off;
@@ -61,8 +61,7 @@ k_scan_final(const uint32_t* in, uint32_t* out, int64_t bound, const uint32_t* d
   uint32_t carry = off;
   for (int64_t base = b0; base < b1; base += kScanThreads) {
     const int64_t i = base + threadIdx.x;
-    uint32_t v = i < b1 ? in[i] : 0u;
-    if (as_flags) v = v != 0u;
+    const uint32_t v = i < b1 ? in[i] : 0u;
     const uint32_t inc = block_inclusive_scan<kScanThreads>(v, warp_tot, &tile_total);
     if (i < b1) out[i] = carry + inc - v;
     __syncthreads();
@@ -84,21 +83,8 @@ int scan_u32(ng_ctx* c, const uint32_t* in, uint32_t* out, int64_t len, const ui
   // blocks for at most 4 tiles each; both kernels split the range by gridDim
   const int blocks = scan_blocks(len);
   // one block needs no partial sums (its offset is zero)
-  if (blocks > 1) k_scan_partial<<<blocks, kScanThreads, 0, c->stream>>>(in, len, d_len, part, 0);
-  k_scan_final<<<blocks, kScanThreads, 0, c->stream>>>(in, out, len, d_len, part, d_total, 0);
-  c->launches += blocks > 1 ? 2 : 1;
-  NG_CUDA(c, cudaGetLastError());
-  return NG_OK;
-}
-
-// Exclusive scan of the flags (in[i] != 0): out[i] = number of non-zero
-// entries before i; *d_total = number of non-zero entries.
-int scan_u32_flags(ng_ctx* c, const uint32_t* in, uint32_t* out, int64_t len, uint32_t* d_total) {
-  NG_TRY(ensure(c, c->scan_part, kScanBlocks * sizeof(uint32_t)));
-  uint32_t* part = as<uint32_t>(c->scan_part);
-  const int blocks = scan_blocks(len);
-  if (blocks > 1) k_scan_partial<<<blocks, kScanThreads, 0, c->stream>>>(in, len, nullptr, part, 1);
-  k_scan_final<<<blocks, kScanThreads, 0, c->stream>>>(in, out, len, nullptr, part, d_total, 1);
+  if (blocks > 1) k_scan_partial<<<blocks, kScanThreads, 0, c->stream>>>(in, len, d_len, part);
+  k_scan_final<<<blocks, kScanThreads, 0, c->stream>>>(in, out, len, d_len, part, d_total);
   c->launches += blocks > 1 ? 2 : 1;
   NG_CUDA(c, cudaGetLastError());
   return NG_OK;
@@ -139,23 +125,6 @@ __device__ __forceinline__ uint32_t stored_type(uint8_t t, int D) { return t < D
 // the species counts (kept until the next sort: the starts of the type-major
 // order), and one tile ticket per pass and for the type order.
 constexpr int kSwTypes = 8 * 256, kSwTickets = kSwTypes + 8, kSortWords = kSwTickets + 9;
-
-// Look-back state of one (tile, digit): 0, or a flag in the top bits and a
-// body count below (64 bits: counts up to the largest n).
-constexpr uint64_t kLbAggregate = 1ull << 62, kLbPrefix = 2ull << 62, kLbCount = (1ull << 62) - 1;
-
-__device__ __forceinline__ uint64_t lb_load(const uint64_t* p) {
-  uint64_t v;
-  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-  return v;
-}
-__device__ __forceinline__ void lb_store(uint64_t* p, uint64_t v) {
-  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
-}
-// Polls of one state before a tile stops waiting and counts the digits before
-// it from the input itself. Tiles are numbered by ticket, so the tile waited
-// for always runs and never waits for this one; the limit only bounds the wait.
-constexpr int kLbPolls = 1 << 20;
 
 // Keys of all bodies, the digit histograms of passes first..7 and the species
 // counts; clears the look-back state of the first pass and of the type order.
@@ -476,26 +445,11 @@ k_type_order(int64_t n, int D, const uint8_t* __restrict__ stype, uint32_t* word
     }
     const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
     if (lane == 0) lb_store(&lb[tile * 8 + w], (tile == 0 ? kLbPrefix : kLbAggregate) | total);
-    uint64_t before = 0;
-    int polls = 0;
-    for (int64_t t = tile - 1; t >= 0;) {
-      // lane j: the state of tile t - j; add up to the nearest prefix
-      const uint64_t s = t - lane >= 0 ? lb_load(&lb[(t - lane) * 8 + w]) : kLbPrefix;
-      const uint32_t pre = __ballot_sync(0xffffffffu, (s & kLbPrefix) != 0);
-      const uint32_t use = pre ? (pre & -pre) | ((pre & -pre) - 1u) : 0xffffffffu;
-      if (__ballot_sync(0xffffffffu, s == 0) & use) {
-        if (++polls < kLbPolls) continue;
-        before = 0;   // count the species before this tile instead
-        for (int64_t i = lane; i < t0; i += 32) before += stype[i] == w;
-        for (int o = 16; o; o >>= 1) before += __shfl_xor_sync(0xffffffffu, before, o);
-        break;
-      }
-      uint64_t add = (use >> lane & 1u) ? s & kLbCount : 0;
-      for (int o = 16; o; o >>= 1) add += __shfl_xor_sync(0xffffffffu, add, o);
-      before += add;
-      if (pre) break;
-      t -= 32;
-    }
+    const uint64_t before = lb_before(lb + w, 8, tile, [&] {
+      uint64_t c = 0;
+      for (int64_t i = lane; i < t0; i += 32) c += stype[i] == w;
+      return c;
+    });
     if (lane == 0 && tile > 0) lb_store(&lb[tile * 8 + w], kLbPrefix | (before + total));
     uint32_t run = (uint32_t)before + incl - sum;
     for (int s = 0; s < w; ++s) run += words[kSwTypes + s];
