@@ -20,8 +20,8 @@ constexpr int kMaxD = NG_MAX_SPECIES;
 constexpr int kMaxLevel = 20;           // 20 Morton bits per axis
 constexpr int kCapturedDepthMargin = 2;  // captured steps build this far below the depth seen
 constexpr int kMonoWords = 3;   // counters of the monopole stage, ticket of the group stage
-// Monopoles of trees of kBinnedMonoBodies bodies or more take their leaves and
-// ready internal nodes in an order binned by the work of a node: leaves by body
+// Monopoles of trees of kBinnedMonoBodies bodies or more (leaf sizes above 8)
+// take their leaves and ready internal nodes in an order binned by the work of a node: leaves by body
 // count (0..64, one more bin for the larger leaves of a tree stopped at a level
 // cap), internal nodes by child count.
 constexpr int kLeafBins = 66;

@@ -41,8 +41,8 @@ __device__ __forceinline__ Levels levels_of(uint32_t* status) {
 // flags laid out level-major, which k_tree_count sums per tile, one device
 // scan turns into offsets, and k_tree_emit completes inside the tile.
 //
-// Bound by reading the keys twice (8 B a body each) and by the launches: four
-// or five for any size, where one launch triple per level took 81 (131k
+// Bound by reading the keys twice (8 B a body each) and by the launches: three
+// to five for any size, where one launch triple per level took 81 (131k
 // bodies: about 340 -> 33 us of kernels; 3 M: 560 -> 95 us), and a cluster of
 // eight blocks walking the levels of a small tree 92 us at 4096 bodies (now 26).
 constexpr int kTreeThreads = 256;
@@ -365,7 +365,7 @@ struct MonoArgs {
   bool unit;               // L == 1: physical and box units are the same
 };
 
-// Below kBinnedMonoBodies bodies, leaves are summed from tiles of consecutive
+// Below kBinnedMonoBodies bodies, and for small leaves, leaves are summed from tiles of consecutive
 // bodies in shared memory: the body arrays are read once, coalesced, and every
 // body's record (offset from its leaf's centre, subtracted in FP64 in physical
 // units, scaled to box units in FP32) is written coalesced. A leaf is then summed by one thread
@@ -537,9 +537,9 @@ __device__ __forceinline__ void mono_internal_lane(const MonoNode& v, const Mono
 // 131k-body force 687 -> 651 us, a 300k-body tree force 981 -> 894 us, a
 // 200k-body step 713 -> 660 us, all with the tiles' loads below.)
 //
-// Counters (c->mono_words, zeroed by k_tree_emit): ready nodes (trees below
-// kBinnedMonoBodies bodies; listed in n_tmp), nodes listed by k_mono_ready, and
-// the tiles of the group list.
+// Counters (c->mono_words, zeroed by k_tree_emit): ready nodes (trees whose
+// leaves go by tiles; listed in n_tmp), nodes listed by k_mono_ready, and the
+// tiles of the group list.
 constexpr int kMlReady = 0, kMlNext = 1, kGroupTicket = 2;
 static_assert(kGroupTicket + 1 == kMonoWords && kMonoWords <= kTreeThreads, "counters");
 
@@ -780,9 +780,9 @@ __global__ void __launch_bounds__(kMonoThreads) k_mono_up(MonoArgs a, const uint
   }
 }
 
-// Trees of kBinnedMonoBodies bodies or more: the leaves one thread each, all
-// in one launch, then the internal nodes one thread each, one launch per
-// level, bottom-up, both in an order binned by the node's work. A leaf loops
+// Other trees of kBinnedMonoBodies bodies or more: the leaves one thread each, all
+// in one launch, then the ready internal nodes one thread each, both in an
+// order binned by the node's work. A leaf loops
 // over its bodies and an internal node over its children, so a warp runs as
 // long as its longest loop; FP64 issues at 1/64 of the FP32 rate here and a
 // warp instruction costs the same with idle lanes. In Morton order the
@@ -790,16 +790,17 @@ __global__ void __launch_bounds__(kMonoThreads) k_mono_up(MonoArgs a, const uint
 // iterations its bodies need (2^24 clustered bodies, leaf 32); binned, the
 // threads of a warp have equal loop counts. Each leaf is still summed by one
 // thread in its own order, so the results do not depend on the binning.
-// Tiles are the better leaves below (their loads are coalesced and they need no
-// order first), this order above, where it keeps the FP64 pipe's lanes full.
-// Passes with tiles / in this order: a force on 131k bodies 664 / 676 us, a
-// 200k-body step 668 / 698 us, a force on 2 M bodies 5822 / 5755 us, a build of
-// 3 M bodies 1379 / 1182 us.
-// The ready internal nodes are as many again in this order, one per lane (an
-// FP64 instruction serves 32 of them), and what is above them goes to teams. A
+// Tiles take no order first and read the bodies coalesced; this order keeps the
+// FP64 pipe's lanes full, which a tile's few leaves do not when leaves are
+// large. Passes with tiles / in this order: a force on 131k bodies 664 / 676 us,
+// a 200k-body step 668 / 698 us, a build of 3 M bodies in leaves of 8 1053 /
+// 1114 us, two steps of 2^24 bodies in leaves of 32 145.5 / 144.3 ms: tiles
+// below kBinnedMonoBodies bodies and for leaves up to kTileLeaf.
+// From kBinnedMonoBodies bodies the ready nodes are taken one per lane (an FP64
+// instruction serves 32 of them), and what is above them goes to teams. A
 // launch per level (20 of them, most nearly empty, 10 to 20 us each for the
-// lower ones) took 221 us at 3 M bodies and three species; ready nodes, teams
-// and their share of the order take 150 us.
+// lower ones) took 221 us at 3 M bodies and three species; this takes 140 us.
+constexpr int kTileLeaf = 8;
 static_assert(kMonoBins <= 256, "the bin scan takes one bin per thread of a 256-thread block");
 
 // bin of node k, -1 for an internal node that is not ready (need > 0)
@@ -934,13 +935,15 @@ __global__ void __launch_bounds__(kMonoThreads) k_mono_leaves(MonoArgs a, const 
     mono_leaf<D>(order[i], a, lacc, threadIdx.x);
 }
 
-// The ready nodes, one per lane; the parents they complete are listed behind
-// the order for k_mono_up.
+// The ready nodes order[*skip, *end), one per lane; the parents they complete
+// are listed behind them for k_mono_up.
 template <int D>
-__global__ void __launch_bounds__(kMonoThreads) k_mono_ready(MonoArgs a, const uint32_t* __restrict__ bins,
-                                                             uint32_t* order, uint32_t* words) {
+__global__ void __launch_bounds__(kMonoThreads) k_mono_ready(MonoArgs a, uint32_t* order,
+                                                             const uint32_t* __restrict__ skip,
+                                                             const uint32_t* __restrict__ end,
+                                                             uint32_t* words) {
   if (a.status[ST_FLAGS] & SF_NODE_OVERFLOW) return;
-  const uint32_t s = bins[2 * kMonoBins + kLeafBins], e = bins[3 * kMonoBins];
+  const uint32_t s = skip ? *skip : 0u, e = *end;
   const int lane = threadIdx.x & 31;
   for (uint32_t i0 = s + blockIdx.x * blockDim.x + (threadIdx.x & ~31); i0 < e; i0 += gridDim.x * blockDim.x) {
     const bool has = i0 + lane < e;
@@ -959,11 +962,18 @@ template <int D>
 static int launch_monopoles(ng_ctx* c, const MonoArgs& a) {
   uint32_t* words = as<uint32_t>(c->mono_words);
   uint32_t* order = as<uint32_t>(c->n_tmp);
-  if (c->n < kBinnedMonoBodies) {
+  const int64_t cap = std::min<int64_t>(c->cap_nodes, 2 * c->n + 64);
+  const int grid = (int)std::min<int64_t>((int64_t)c->nsm * 16, (cap + kMonoThreads - 1) / kMonoThreads);
+  const bool large = c->n >= kBinnedMonoBodies;
+  if (!large || c->p.leaf_size <= kTileLeaf) {
     const int64_t tiles = (c->n + kLeafTile - 1) / kLeafTile;
-    k_mono_tiles<D><<<(int)std::min<int64_t>((int64_t)c->nsm * 16, tiles), kLeafThreads, 0, c->stream>>>(a, words, order);
+    k_mono_tiles<D><<<(int)std::min<int64_t>((int64_t)c->nsm * 64, tiles), kLeafThreads, 0, c->stream>>>(a, words, order);
     c->launches += 1;
-    if (c->n > c->p.leaf_size) {   // else the root is a leaf
+    if (large) {
+      k_mono_ready<D><<<grid, kMonoThreads, 0, c->stream>>>(a, order, nullptr, words + kMlReady, words);
+      k_mono_up<D><<<grid, kMonoThreads, 0, c->stream>>>(a, order, words + kMlReady, words + kMlNext);
+      c->launches += 2;
+    } else if (c->n > c->p.leaf_size) {   // else the root is a leaf
       // a ready node holds more than leaf_size bodies
       const int64_t teams = c->n / (c->p.leaf_size + 1);
       const int64_t blocks = (teams * kTeam<D> + kMonoThreads - 1) / kMonoThreads;
@@ -976,13 +986,12 @@ static int launch_monopoles(ng_ctx* c, const MonoArgs& a) {
   }
   uint32_t* bins = words + kMonoWords;
   NG_CUDA(c, cudaMemsetAsync(bins, 0, 2 * kMonoBins * sizeof(uint32_t), c->stream));
-  const int64_t cap = std::min<int64_t>(c->cap_nodes, 2 * c->n + 64);
   const int sgrid = work_grid(c, cap, 4);
   k_mono_hist<<<sgrid, 256, 0, c->stream>>>(a, bins);
   k_mono_order<<<sgrid, 256, 0, c->stream>>>(a, bins, order);
-  const int grid = (int)std::min<int64_t>((int64_t)c->nsm * 16, (cap + kMonoThreads - 1) / kMonoThreads);
   k_mono_leaves<D><<<grid, kMonoThreads, 0, c->stream>>>(a, bins, order);
-  k_mono_ready<D><<<grid, kMonoThreads, 0, c->stream>>>(a, bins, order, words);
+  k_mono_ready<D><<<grid, kMonoThreads, 0, c->stream>>>(a, order, bins + 2 * kMonoBins + kLeafBins,
+                                                          bins + 3 * kMonoBins, words);
   k_mono_up<D><<<grid, kMonoThreads, 0, c->stream>>>(a, order, bins + 3 * kMonoBins, words + kMlNext);
   c->launches += 5;
   NG_CUDA(c, cudaGetLastError());

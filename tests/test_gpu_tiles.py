@@ -135,3 +135,9 @@ def test_bodies_outside_the_box_and_bad_species(ng, n):
     assert np.array_equal(T["cnt"], R["cnt"].astype(T["cnt"].dtype))
     bound = 2.0 ** -53 * 4 * (R["cnt"].astype(np.float64) + 2)
     assert np.all(np.abs(T["com"] - R["com"]).max(axis=2) <= bound)
+
+
+@pytest.mark.parametrize("n,D,leaf", [(1048576, 2, 8), (1048577, 3, 1), (1048577, 6, 9)])
+def test_large_trees_of_small_leaves(ng, n, D, leaf):
+    """From 2^20 bodies: leaves by tiles up to 8 bodies, binned above."""
+    test_sort_and_tree_at_tile_edges(ng, n, D, leaf)
