@@ -126,7 +126,8 @@ def stage_bytes(n, D, mesh, passes=8):
     keys 24 B position + 1 B species read, 8 B key + 4 B index written; each
     radix pass (8 for a full sort, fewer when the step's tree stops at a level
     cap) 8 B key read by the histogram, 12 B key + index read and 12 B written
-    by the scatter; type-major order 4 B index written,
+    by the scatter (the bytes of a pass in three launches, kept so that lines of
+    different builds compare; a pass in one launch moves 24 B); type-major order 4 B index written,
     then one 32 B radix pass; deposit 33 B per body read plus the D mesh
     clears; FFTs and k-space one read and one write of the D real meshes or
     half spectra; interpolation 24 B position + 1 B species + 4 B index read,
