@@ -368,8 +368,14 @@ int build_checked(ng_ctx* c, int64_t n, const double* pos, const uint8_t* type,
   c->built = false;
   NG_TRY(alloc_bodies(c, n));
   NG_CUDA(c, cudaMemsetAsync(c->status.p, 0, ST_COUNT * 4, c->stream));
-  // records of the sort (not needed for it: without them it gathers unpacked)
-  if (n >= kPackBodies && ensure(c, c->rpack, (size_t)n * 32) != NG_OK) c->err.clear();
+  // records of the sort, which gathers unpacked without them: taken only
+  // where they are a small part of the free memory, so that no call runs out
+  // of it for their sake
+  if (n >= kPackBodies && c->rpack.bytes < (size_t)n * 32) {
+    size_t free_bytes = 0, all = 0;
+    NG_CUDA(c, cudaMemGetInfo(&free_bytes, &all));
+    if ((size_t)n * 32 <= free_bytes / 64 && ensure(c, c->rpack, (size_t)n * 32) != NG_OK) c->err.clear();
+  }
   NG_TRY(sort_bodies(c, n, pos, type, mass));
   return tree_checked(c);
 }
@@ -645,6 +651,23 @@ __global__ void k_scatter_f32(int64_t n, const uint32_t* __restrict__ idx,
     out[idx[k]] = in[k];
 }
 
+// Without the records' memory: straight to the caller's arrays.
+__global__ void k_resident_scatter(int64_t n, const uint32_t* __restrict__ rorig,
+                                   const double* __restrict__ rpos, const float* __restrict__ rvel,
+                                   const float* __restrict__ racc, double* __restrict__ pos,
+                                   float* __restrict__ vel, float* __restrict__ acc) {
+  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n;
+       k += (int64_t)gridDim.x * blockDim.x) {
+    const uint32_t i = rorig[k];
+#pragma unroll
+    for (int e = 0; e < 3; ++e) {
+      pos[e * n + i] = rpos[e * n + k];
+      vel[e * n + i] = rvel[e * n + k];
+      acc[e * n + i] = racc[e * n + k];
+    }
+  }
+}
+
 int reserve_resident(ng_ctx* c, int64_t n) {
   NG_TRY(reserve(c, n));
   NG_TRY(ensure(c, c->spos_alt, (size_t)n * 24));
@@ -656,7 +679,8 @@ int reserve_resident(ng_ctx* c, int64_t n) {
   NG_TRY(ensure(c, c->rorig_alt, (size_t)n * 4));
   NG_TRY(ensure(c, c->racc, (size_t)n * 12));
   NG_TRY(ensure(c, c->rtmp, (size_t)n * 4));
-  NG_TRY(ensure(c, c->rpack, (size_t)n * 64));
+  // (last: without its records the state is scattered back directly)
+  if (ensure(c, c->rpack, (size_t)n * 64) != NG_OK) c->err.clear();
   return NG_OK;
 }
 
@@ -688,12 +712,18 @@ int resident_load(ng_ctx* c, int64_t n, const double* pos, const float* vel,
 // bodies of the last step to caller indices, as after ng_build_tree, and the
 // relative criterion's |a_old| returns to caller order.
 int resident_store(ng_ctx* c, int64_t n, double* pos, float* vel, float* acc) {
-  const int grid = (int)((n + kPackTile - 1) / kPackTile);
-  k_resident_pack<<<grid, kPackTile, 0, c->stream>>>(n, as<uint32_t>(c->rorig), as<double>(c->spos),
-                                                     as<float>(c->rvel), as<float>(c->racc),
-                                                     as<uint4>(c->rpack));
-  k_resident_unpack<<<grid, kPackTile, 0, c->stream>>>(n, as<uint4>(c->rpack), pos, vel, acc);
-  c->launches += 2;
+  if (c->rpack.bytes >= (size_t)n * 64) {
+    const int grid = (int)((n + kPackTile - 1) / kPackTile);
+    k_resident_pack<<<grid, kPackTile, 0, c->stream>>>(n, as<uint32_t>(c->rorig), as<double>(c->spos),
+                                                       as<float>(c->rvel), as<float>(c->racc),
+                                                       as<uint4>(c->rpack));
+    k_resident_unpack<<<grid, kPackTile, 0, c->stream>>>(n, as<uint4>(c->rpack), pos, vel, acc);
+    c->launches += 2;
+  } else {
+    k_resident_scatter<<<work_grid(c, n, 8), 256, 0, c->stream>>>(
+        n, as<uint32_t>(c->rorig), as<double>(c->spos), as<float>(c->rvel), as<float>(c->racc), pos, vel, acc);
+    c->launches += 1;
+  }
   NG_CUDA(c, cudaGetLastError());
   NG_CUDA(c, cudaMemcpyAsync(c->vals_a.p, c->rorig.p, (size_t)n * 4, cudaMemcpyDeviceToDevice,
                              c->stream));
