@@ -23,12 +23,14 @@ int fail(ng_ctx* c, int code, const char* fmt, ...) {
   return code;
 }
 
+// Growing frees the old buffer first, so its contents and its address are gone
+// whether or not the new one is had: captured steps are told by alloc_gen, and
+// callers whose state stands on the buffer give that state up.
 int ensure(ng_ctx* c, DevBuf& b, size_t bytes) {
   if (bytes == 0) bytes = 16;
   if (b.bytes >= bytes) return NG_OK;
-  if (b.p) cudaFree(b.p);
-  b.p = nullptr;
-  b.bytes = 0;
+  release(b);
+  if (c) c->alloc_gen++;
   void* p = nullptr;
   const cudaError_t e = cudaMalloc(&p, bytes);
   if (e != cudaSuccess) {
@@ -37,7 +39,6 @@ int ensure(ng_ctx* c, DevBuf& b, size_t bytes) {
   }
   b.p = p;
   b.bytes = bytes;
-  if (c) c->alloc_gen++;
   return NG_OK;
 }
 

@@ -331,7 +331,7 @@ struct ng_ctx {
   // (fork after the type-major order, join before the walk)
   cudaStream_t pm_stream = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
-  uint64_t alloc_gen = 0;          // bumped whenever a device buffer is (re)allocated
+  uint64_t alloc_gen = 0;          // bumped whenever a device buffer is replaced or lost
   uint64_t graph_gen = 0;
   cudaGraphExec_t step_exec = nullptr;
   int64_t graph_n = -1;

@@ -1,0 +1,90 @@
+"""What the library's host code makes of device memory that runs out, without a
+GPU: it runs against a stand-in CUDA runtime (fake_cudart.c), in which kernels
+do nothing and any allocation can be made to fail. A failed call frees the
+buffers it was growing, so nothing that stood on them may be used afterwards:
+no tree, no node capacity, no captured step."""
+import ctypes
+import json
+import os
+import subprocess
+import sys
+
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+ROOT = os.path.dirname(HERE)
+
+PRELUDE = """
+import ctypes, json, sys
+sys.path.insert(0, {root!r})
+from paper_1502_07442_gb300 import binding as ng
+F = ctypes.CDLL({fake!r})
+F.fake_set_limit.argtypes = [ctypes.c_size_t]
+F.fake_fail_at.argtypes = [ctypes.c_long]
+for f in ("fake_in_use", "fake_live", "fake_mallocs", "fake_captures", "fake_replays"):
+    getattr(F, f).restype = ctypes.c_size_t
+L = ng.lib()
+vp, i64 = ctypes.c_void_p, ctypes.c_int64
+def params(leaf=8):
+    p = ng.NgParams()
+    p.D, p.box, p.eps, p.asmth, p.rcut_over_rs = 1, 1.0, 1e-4, 0.02, 4.5
+    p.theta, p.leaf_size, p.G[0][0] = 0.5, leaf, 1.0
+    return p
+def context(**k):
+    c = vp()
+    p = params(**k)
+    assert L.ng_create(ctypes.byref(c), ctypes.byref(p), None) == ng.NG_OK
+    return c
+def state(n):
+    # "device" arrays: pos, vel, type, mass, acc
+    return [ctypes.cast(ctypes.create_string_buffer(max(1, b * n)), vp) for b in (24, 12, 1, 4, 12)]
+def build(c, n, s):
+    return L.ng_build_tree(c, i64(n), s[0], s[2], s[3], None, None)
+def step(c, n, s, valid, k):
+    return L.ng_step(c, i64(n), s[0], s[1], s[2], s[3], s[4], valid, k, ctypes.c_double(0.25))
+"""
+
+
+@pytest.fixture(scope="module")
+def run(tmp_path_factory):
+    from paper_1502_07442_gb300 import build
+    build.build()
+    d = tmp_path_factory.mktemp("fake")
+    fake = str(d / "fake_cudart.so")
+    subprocess.check_call(["gcc", "-O1", "-shared", "-fPIC", os.path.join(HERE, "fake_cudart.c"), "-o", fake])
+
+    def go(body):
+        script = d / "case.py"
+        script.write_text(PRELUDE.format(root=ROOT, fake=fake) + body)
+        r = subprocess.run([sys.executable, str(script)], capture_output=True, text=True, timeout=120,
+                           env=dict(os.environ, LD_PRELOAD=fake))
+        assert r.returncode == 0, r.stderr[-2000:]
+        return json.loads(r.stdout.splitlines()[-1])
+    return go
+
+
+@pytest.mark.parametrize("k", [0, 1, 5, 12])
+def test_a_failed_batch_step_drops_the_captured_one(run, k):
+    """A larger batch step whose k-th allocation fails has freed buffers that the
+    step captured before reads: the next step at the old sizes is captured anew."""
+    out = run(f"""
+S, n = 2, 1000
+b = vp()
+P = (ng.NgParams * S)(params(), params())
+assert L.ng_batch_create(ctypes.byref(b), S, P, None) == ng.NG_OK
+st, big = [state(n), state(n)], [state(60000), state(n)]
+def go(ns, states, valid, steps):
+    arr = [(vp * S)(*[x[j].value for x in states]) for j in range(5)]
+    return L.ng_batch_step(b, (i64 * S)(*ns), arr[0], arr[1], arr[2], arr[3], arr[4], valid, steps,
+                           ctypes.c_double(0.25))
+assert go([n, n], st, 0, 3) == ng.NG_OK
+c1 = F.fake_captures()
+assert go([n, n], st, 1, 3) == ng.NG_OK
+c2 = F.fake_captures()
+F.fake_fail_at({k})
+r = go([60000, n], big, 0, 3)
+F.fake_fail_at(-1)
+assert go([n, n], st, 1, 3) == ng.NG_OK
+print(json.dumps(dict(reused=c2 == c1, failed=r == ng.NG_ENOMEM, anew=F.fake_captures() > c2)))
+""")
+    assert out == dict(reused=True, failed=True, anew=True)
