@@ -261,6 +261,7 @@ __global__ void k_amag(int64_t n, const float* __restrict__ acc, float* __restri
 }
 
 static int set_aold(ng_ctx* c, int64_t n, const float* acc) {
+  c->aold_n = -1;   // until the new ones are written
   NG_TRY(ensure(c, c->aold, (size_t)n * sizeof(float)));
   k_amag<<<work_grid(c, n, 8), 256, 0, c->stream>>>(n, acc, as<float>(c->aold));
   c->launches += 1;
@@ -282,6 +283,8 @@ static size_t node_bytes(int D) {
 
 int alloc_nodes(ng_ctx* c, int64_t cap) {
   const int D = c->p.D;
+  if (cap > c->cap_nodes) c->built = false;   // arrays are replaced
+  c->cap_nodes = 0;                           // until every one is had
   NG_TRY(ensure(c, c->n_level, cap));
   NG_TRY(ensure(c, c->n_prefix, cap * 8));
   NG_TRY(ensure(c, c->n_first, cap * 4));
@@ -325,7 +328,10 @@ int reserve(ng_ctx* c, int64_t n) {
   NG_TRY(ensure(c, c->gsize, (size_t)n * sizeof(uint32_t)));
   NG_TRY(ensure(c, c->walk_desc, sizeof(WalkDesc)));
   NG_TRY(ensure(c, c->walk_prefix, 4 * sizeof(uint32_t)));
-  if (c->p.opening == NG_OPEN_RELATIVE) NG_TRY(ensure(c, c->aold, (size_t)n * sizeof(float)));
+  if (c->p.opening == NG_OPEN_RELATIVE) {
+    if (c->aold.bytes < (size_t)n * sizeof(float)) c->aold_n = -1;
+    NG_TRY(ensure(c, c->aold, (size_t)n * sizeof(float)));
+  }
   if (c->p.pm_mesh > 0 && !c->pm_stream) {
     if (cudaStreamCreateWithFlags(&c->pm_stream, cudaStreamNonBlocking) != cudaSuccess ||
         cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
@@ -1041,7 +1047,11 @@ int ng_step(ng_ctx* c, int64_t n, double* pos, float* vel, const uint8_t* type,
   }
   // the state stays on the device in the previous step's sorted order
   c->n = n;
-  NG_TRY(reserve_resident(c, n));
+  const int reserved = reserve_resident(c, n);
+  if (reserved != NG_OK) {
+    c->built = false;   // buffers of an earlier tree may be gone
+    return reserved;
+  }
   NG_CUDA(c, cudaMemsetAsync(c->status.p, 0, sizeof(uint32_t), c->stream));
   NG_TRY(resident_load(c, n, pos, vel, type, mass, acc));
   int r = NG_OK;

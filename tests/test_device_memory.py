@@ -63,6 +63,32 @@ def run(tmp_path_factory):
     return go
 
 
+def test_a_failed_step_leaves_no_tree_and_no_capacity(run):
+    """Every allocation of a larger step fails in turn: the tree of the build
+    before is then refused, and the next build holds all of its buffers again."""
+    out = run("""
+s, big = state(1000), state(50000)
+rows = []
+for k in range(200):
+    c = context()
+    assert build(c, 1000, s) == ng.NG_OK and L.ng_tree_force(c, s[4], None) == ng.NG_OK
+    live = F.fake_live()
+    F.fake_fail_at(k)
+    r = step(c, 50000, big, 1, 1)
+    F.fake_fail_at(-1)
+    if r == ng.NG_OK:
+        break
+    refused = L.ng_tree_force(c, s[4], None)
+    again = build(c, 1000, s), L.ng_tree_force(c, s[4], None)
+    rows.append([r, refused, again[0], again[1], F.fake_live() >= live])
+    L.ng_destroy(c)
+print(json.dumps(dict(rows=rows, enomem=ng.NG_ENOMEM, estate=ng.NG_ESTATE)))
+""")
+    assert len(out["rows"]) > 30
+    for k, r in enumerate(out["rows"]):
+        assert r == [out["enomem"], out["estate"], 0, 0, True], (k, r)
+
+
 @pytest.mark.parametrize("k", [0, 1, 5, 12])
 def test_a_failed_batch_step_drops_the_captured_one(run, k):
     """A larger batch step whose k-th allocation fails has freed buffers that the
