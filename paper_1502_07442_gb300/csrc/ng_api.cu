@@ -160,7 +160,6 @@ int build_tables(ng_ctx* c) {
     return fail(c, NG_EINVAL, "box too large relative to the table spacing (box/dr = %.3g)",
                 c->L / c->dr_phys);
   std::vector<float> h = walk_table(c, ncut, c->dr_phys);
-  c->h_tab = h;
   NG_TRY(ensure(c, c->d_tab, h.size() * sizeof(float)));
   // upload through the context's pinned staging copy: wait until the stream
   // has consumed the previous contents, then copy without a pageable stall
@@ -186,6 +185,7 @@ int build_tables(ng_ctx* c) {
     }
     NG_TRY(build_lattice(c, (int)laws.size(), kinds.data(), as.data(), ls.data()));
   }
+  c->h_tab = std::move(h);
   return NG_OK;
 }
 
@@ -551,6 +551,7 @@ void normalize_params(ng_params* p) {
 int ctx_configure(ng_ctx* c, const ng_params* p) {
   NG_TRY(validate(c, p));
   c->p = *p;
+  c->h_tab.clear();   // until the tables of these parameters are had
   normalize_params(&c->p);
   c->L = p->box;
   c->rs = p->pm_mesh > 0 ? p->asmth * p->box / p->pm_mesh : p->asmth * p->box;

@@ -114,3 +114,30 @@ assert go([n, n], st, 1, 3) == ng.NG_OK
 print(json.dumps(dict(reused=c2 == c1, failed=r == ng.NG_ENOMEM, anew=F.fake_captures() > c2)))
 """)
     assert out == dict(reused=True, failed=True, anew=True)
+
+
+def test_a_slot_without_tables_is_configured_again(run):
+    """A served request whose law tables could not be had fails; the next one with
+    the same parameters does not run on what is left of them."""
+    out = run("""
+s = vp()
+assert L.ng_serve_create(ctypes.byref(s), 1, ctypes.c_size_t(1 << 32)) == ng.NG_OK
+n = 1000
+a = state(n)
+q = ng.NgRequest()
+q.kind, q.n, q.params = 0, n, params()
+q.params.D = 5                      # a larger table than the slot's first one
+q.pos, q.type, q.mass, q.acc_out = [x.value for x in (a[0], a[2], a[3], a[4])]
+res = (ng.NgResult * 1)()
+def serve():
+    assert L.ng_serve(s, ctypes.byref(q), res, 1, None, ctypes.c_double(30.0)) == ng.NG_OK
+    return res[0].status
+F.fake_fail_at(0)
+first = serve()
+F.fake_fail_at(-1)
+second = serve()
+reconf = i64()
+L.ng_serve_stats(s, None, None, None, ctypes.byref(reconf))
+print(json.dumps(dict(first=first == ng.NG_ENOMEM, second=second, configured=reconf.value)))
+""")
+    assert out == dict(first=True, second=0, configured=1)
