@@ -32,7 +32,8 @@ int ensure(ng_ctx* c, DevBuf& b, size_t bytes) {
   release(b);
   if (c) c->alloc_gen++;
   void* p = nullptr;
-  const cudaError_t e = cudaMalloc(&p, bytes);
+  cudaError_t e = cudaMalloc(&p, bytes);
+  if (e != cudaSuccess && give_back_records(c)) e = cudaMalloc(&p, bytes);
   if (e != cudaSuccess) {
     cudaGetLastError();
     return fail(c, NG_ENOMEM, "cudaMalloc of %zu bytes failed: %s", bytes, cudaGetErrorString(e));
@@ -46,6 +47,36 @@ void release(DevBuf& b) {
   if (b.p) cudaFree(b.p);
   b.p = nullptr;
   b.bytes = 0;
+}
+
+// Records of the sort (32 bytes a body) and of the return of a stepped state
+// (64 bytes) make these passes faster; both work without. They are taken only
+// where kRecordRoom bytes a body are free, 3 % of the free memory at most, a
+// buffer at hand stays until the larger one is had, and they are given back
+// when an allocation that a call needs fails.
+constexpr size_t kRecordRoom = 2048;
+
+void take_records(ng_ctx* c, int64_t n, size_t bytes) {
+  if (c->rpack.bytes >= bytes) return;
+  size_t free_bytes = 0, all = 0;
+  DevBuf b;
+  if (cudaMemGetInfo(&free_bytes, &all) != cudaSuccess || free_bytes / kRecordRoom < (size_t)n ||
+      cudaMalloc(&b.p, bytes) != cudaSuccess) {
+    cudaGetLastError();
+    return;
+  }
+  b.bytes = bytes;
+  release(c->rpack);
+  c->rpack = b;
+  c->alloc_gen++;
+}
+
+bool give_back_records(ng_ctx* c) {
+  if (!c || !c->rpack.p) return false;
+  cudaGetLastError();   // of the allocation that failed
+  release(c->rpack);
+  c->alloc_gen++;
+  return true;
 }
 
 // ------------------------------------------------------ short-range laws
@@ -375,14 +406,7 @@ int build_checked(ng_ctx* c, int64_t n, const double* pos, const uint8_t* type,
   c->built = false;
   NG_TRY(alloc_bodies(c, n));
   NG_CUDA(c, cudaMemsetAsync(c->status.p, 0, ST_COUNT * 4, c->stream));
-  // records of the sort, which gathers unpacked without them: taken only
-  // where they are a small part of the free memory, so that no call runs out
-  // of it for their sake
-  if (n >= kPackBodies && c->rpack.bytes < (size_t)n * 32) {
-    size_t free_bytes = 0, all = 0;
-    NG_CUDA(c, cudaMemGetInfo(&free_bytes, &all));
-    if ((size_t)n * 32 <= free_bytes / 64 && ensure(c, c->rpack, (size_t)n * 32) != NG_OK) c->err.clear();
-  }
+  if (n >= kPackBodies) take_records(c, n, (size_t)n * 32);   // without: unpacked
   NG_TRY(sort_bodies(c, n, pos, type, mass));
   return tree_checked(c);
 }
@@ -687,8 +711,7 @@ int reserve_resident(ng_ctx* c, int64_t n) {
   NG_TRY(ensure(c, c->rorig_alt, (size_t)n * 4));
   NG_TRY(ensure(c, c->racc, (size_t)n * 12));
   NG_TRY(ensure(c, c->rtmp, (size_t)n * 4));
-  // (last: without its records the state is scattered back directly)
-  if (ensure(c, c->rpack, (size_t)n * 64) != NG_OK) c->err.clear();
+  take_records(c, n, (size_t)n * 64);   // without: scattered back directly
   return NG_OK;
 }
 
@@ -1114,7 +1137,8 @@ int ng_step(ng_ctx* c, int64_t n, double* pos, float* vel, const uint8_t* type,
           r = fail(c, NG_ECUDA, "step capture failed: %s", cudaGetErrorString(e));
           break;
         }
-        const cudaError_t ei = cudaGraphInstantiate(slot, g, 0);
+        cudaError_t ei = cudaGraphInstantiate(slot, g, 0);
+        if (ei == cudaErrorMemoryAllocation && give_back_records(c)) ei = cudaGraphInstantiate(slot, g, 0);
         cudaGraphDestroy(g);
         if (ei != cudaSuccess) r = fail(c, NG_ECUDA, "graph instantiate failed: %s", cudaGetErrorString(ei));
       }

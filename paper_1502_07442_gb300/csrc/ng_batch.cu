@@ -113,6 +113,17 @@ bool join_class(WalkClass& k, const ng_ctx* rep, const ng_ctx* c, int ncut, doub
   return true;
 }
 
+// A stage of a step that allocates (and can be run again): out of memory, it
+// runs again without the optional records of all members.
+template <class Stage>
+int with_room(ng_batch* b, Stage stage) {
+  int r = stage();
+  if (r != NG_ENOMEM) return r;
+  bool some = false;
+  for (ng_ctx* c : b->sims) some = give_back_records(c) || some;
+  return some ? stage() : r;
+}
+
 uint64_t alloc_gen(const ng_batch* b) {
   uint64_t g = 0;
   for (const ng_ctx* c : b->sims) g += c->alloc_gen;
@@ -331,8 +342,8 @@ int ng_batch_step(ng_batch* b, const int64_t* n, double* const* pos, float* cons
     for (int i = 0; i < S; ++i) {
       ng_ctx* c = b->sims[i];
       c->stream = b->stream;
-      int r = build_checked(c, n[i], pos[i], type[i], mass[i]);
-      if (r == NG_OK) r = force_stages(c, acc[i]);
+      int r = with_room(b, [&] { return build_checked(c, n[i], pos[i], type[i], mass[i]); });
+      if (r == NG_OK) r = with_room(b, [&] { return force_stages(c, acc[i]); });
       if (r != NG_OK) return from_sim(b, i, r);
     }
   }
@@ -361,12 +372,12 @@ int ng_batch_step(ng_batch* b, const int64_t* n, double* const* pos, float* cons
       ng_ctx* c = b->sims[i];
       c->stream = b->stream;
       int r = launch_kick_drift(c, n[i], vel[i], acc[i], 0.5 * dt, 1, pos[i], dt);
-      if (r == NG_OK) r = build_checked(c, n[i], pos[i], type[i], mass[i]);
-      if (r == NG_OK) r = force_stages(c, acc[i]);
+      if (r == NG_OK) r = with_room(b, [&] { return build_checked(c, n[i], pos[i], type[i], mass[i]); });
+      if (r == NG_OK) r = with_room(b, [&] { return force_stages(c, acc[i]); });
       if (r == NG_OK) r = launch_kick(c, n[i], vel[i], acc[i], 0.5 * dt);
       if (r == NG_OK && c->cap_nodes < c->nnodes + c->nnodes / 4 + 1024) {
         if (cudaStreamSynchronize(b->stream) != cudaSuccess) return bfail(b, NG_ECUDA, "sync");
-        r = alloc_nodes(c, c->nnodes + c->nnodes / 4 + 1024);
+        r = with_room(b, [&] { return alloc_nodes(c, c->nnodes + c->nnodes / 4 + 1024); });
       }
       if (r != NG_OK) return from_sim(b, i, r);
     }
@@ -381,8 +392,10 @@ int ng_batch_step(ng_batch* b, const int64_t* n, double* const* pos, float* cons
           for (int tt = 0; tt < kMaxD; ++tt) k.h[j].tabid[ss][tt] = m[ss * kMaxD + tt];
       }
       ng_ctx* rep = b->sims[k.members[0]];
-      int r = ensure(rep, k.d, k.h.size() * sizeof(WalkDesc));
-      if (r == NG_OK) r = ensure(rep, k.pre, (k.h.size() + 2) * sizeof(uint32_t));
+      const int r = with_room(b, [&] {
+        NG_TRY(ensure(rep, k.d, k.h.size() * sizeof(WalkDesc)));
+        return ensure(rep, k.pre, (k.h.size() + 2) * sizeof(uint32_t));
+      });
       if (r != NG_OK) return from_sim(b, k.members[0], r);
     }
     if (cudaStreamSynchronize(b->stream) != cudaSuccess) return bfail(b, NG_ECUDA, "sync failed");

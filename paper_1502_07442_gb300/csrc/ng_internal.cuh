@@ -368,6 +368,10 @@ int fail(ng_ctx* c, int code, const char* fmt, ...);
 // Ensure buf holds at least bytes (grows, contents not kept).
 int ensure(ng_ctx* c, DevBuf& buf, size_t bytes);
 void release(DevBuf& buf);
+// Optional records of n bodies (c->rpack): taken where memory is ample; given
+// back (true: there were some) when a call runs out of it.
+void take_records(ng_ctx* c, int64_t n, size_t bytes);
+bool give_back_records(ng_ctx* c);
 
 template <class T>
 inline T* as(const DevBuf& b) { return static_cast<T*>(b.p); }

@@ -245,11 +245,18 @@ static int pm_setup(ng_ctx* c) {
   int dims[3] = {N, N, N};
   ng_ctx::Plan pl{N, D, 0, 0};
   std::lock_guard<std::mutex> lock(g_fft_plan_lock);
-  if (cufftPlanMany(&pl.r2c, 3, dims, nullptr, 1, (int)N3, nullptr, 1, (int)modes,
-                    CUFFT_R2C, D) != CUFFT_SUCCESS ||
-      cufftPlanMany(&pl.c2r, 3, dims, nullptr, 1, (int)modes, nullptr, 1, (int)N3,
-                    CUFFT_C2R, D) != CUFFT_SUCCESS) {
+  auto make_plans = [&] {
+    if (cufftPlanMany(&pl.r2c, 3, dims, nullptr, 1, (int)N3, nullptr, 1, (int)modes,
+                      CUFFT_R2C, D) == CUFFT_SUCCESS &&
+        cufftPlanMany(&pl.c2r, 3, dims, nullptr, 1, (int)modes, nullptr, 1, (int)N3,
+                      CUFFT_C2R, D) == CUFFT_SUCCESS)
+      return true;
     if (pl.r2c) cufftDestroy(pl.r2c);
+    pl.r2c = pl.c2r = 0;
+    cudaGetLastError();
+    return false;
+  };
+  if (!make_plans() && !(give_back_records(c) && make_plans())) {
     return fail(c, NG_ECUDA, "cuFFT plan creation failed for a %d^3 mesh, batch %d", N, D);
   }
   c->plans.push_back(pl);

@@ -141,3 +141,62 @@ L.ng_serve_stats(s, None, None, None, ctypes.byref(reconf))
 print(json.dumps(dict(first=first == ng.NG_ENOMEM, second=second, configured=reconf.value)))
 """)
     assert out == dict(first=True, second=0, configured=1)
+
+
+def test_records_are_given_back_before_a_call_runs_out(run):
+    """A step on 131072 bodies keeps its optional records (64 bytes a body); a later
+    build that fits only without them gets their memory, and so does a batch
+    member from another's."""
+    out = run("""
+n1, n2 = 131072, 4000000
+s1, s2 = state(n1), state(n2)
+def single(limit):
+    F.fake_set_limit(limit)
+    c = context()
+    assert step(c, n1, s1, 1, 2) == ng.NG_OK
+    held = F.fake_in_use()
+    r = build(c, n2, s2), L.ng_tree_force(c, s2[4], None)
+    top = F.fake_in_use()
+    L.ng_destroy(c)
+    return held, r, top
+def batch(limit):
+    F.fake_set_limit(limit)
+    b = vp()
+    P = (ng.NgParams * 2)(params(), params())
+    assert L.ng_batch_create(ctypes.byref(b), 2, P, None) == ng.NG_OK
+    def go(ns, states):
+        arr = [(vp * 2)(*[x[j].value for x in states]) for j in range(5)]
+        return L.ng_batch_step(b, (i64 * 2)(*ns), arr[0], arr[1], arr[2], arr[3], arr[4], 0, 2, ctypes.c_double(0.25))
+    small = state(1000)
+    assert go([n1, 1000], [s1, small]) == ng.NG_OK
+    held = F.fake_in_use()
+    r = [go([n1, n2], [s1, s2])]
+    top = F.fake_in_use()
+    L.ng_batch_destroy(b)
+    return held, r, top
+rows = []
+for f, records in ((single, 64 * n1), (batch, 32 * n1)):
+    held, r, top = f(1 << 30)
+    tight = f(top - records // 2)
+    rows.append([list(r), list(tight[1]), tight[0] == held, top - tight[2] == records])
+print(json.dumps(rows))
+""")
+    assert out == [[[0, 0], [0, 0], True, True], [[0], [0], True, True]]
+
+
+@pytest.mark.parametrize("call,size", [("build(c, n, s)", 32), ("step(c, n, s, 1, 1)", 64)])
+def test_records_are_a_small_part_of_the_free_memory(run, call, size):
+    """Taken only where 2048 bytes a body are free: 3 % of it at most."""
+    out = run(f"""
+n = 150000
+s = state(n)
+use = []
+for limit in (1 << 33, 1 << 28):
+    F.fake_set_limit(limit)
+    c = context()
+    assert {call} == ng.NG_OK
+    use.append(F.fake_in_use())
+    L.ng_destroy(c)
+print(json.dumps(use[0] - use[1]))
+""")
+    assert out == size * 150000
