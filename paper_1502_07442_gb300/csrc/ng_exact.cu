@@ -7,8 +7,10 @@
 // per-particle count (geometric or relative, decisions in FP64 as there),
 // a node per lane, and evaluates every accepted species monopole and every
 // body of an opened leaf, a term per lane, with the pair's law in FP32
-// (offsets of positions held as two floats each, rounded to FP32 as the FP64
-// difference would be; the cut-off decided as in FP64):
+// (offsets and |d|^2 + eps^2 from positions held as two floats each, correct
+// to 2^-30 of |d| before their one rounding to FP32, and from the FP64
+// positions where the pair is closer than that allows; the cut-off decided as
+// in FP64):
 //   Newton         f = 1
 //   Yukawa (C=1)   f = 1 + a (1 + r/l) e^{-r/l}
 //   pure Yukawa    f = a (1 + r/l) e^{-r/l}
@@ -71,7 +73,8 @@ struct ExactArgs {
   uint32_t* status;
   bool unit;               // L == 1
   float Lh, Ll;            // L = Lh + Ll
-  float theta32, eps2f;
+  float theta32;
+  float eps2h, eps2l;      // eps2 = eps2h + eps2l
   float cut_lo2, cut_hi2;  // node cut-off^2 (box units) less and plus the FP32 margin
   float rc2f;              // rcut2, for the terms' FP32 decision
 };
@@ -246,27 +249,67 @@ __device__ __forceinline__ int exact_decide32(const ExactArgs& a, const float4 g
   return -1;
 }
 
-// Whether a term at q64 = |d|^2 + eps^2 (FP64, the count's operation order)
-// lies within the cut-off: for the terms FP32 cannot tell.
-__device__ __noinline__ bool exact_within64(const ExactArgs& a, const double p[3], int64_t k) {
+// Bodies closer than this (box units, largest component) take their offset from
+// the FP64 positions: two floats hold a position to 2^-50 and leave an offset
+// uncertain by 2^-47 with the roundings of their difference, 2^-31 of |d| here.
+constexpr float kExactNear = 1.f / 65536.f;
+
+// A term in FP64, in the operation order of the count: offset (physical) and
+// |d|^2 + eps^2 of node species record or body src from body k, each rounded
+// once; w < 0: beyond the cut-off.
+__device__ __noinline__ float4 exact_pair64(const ExactArgs& a, bool mono, uint32_t src, int64_t k) {
   double d[3];
+  const double* m = a.m64 + (size_t)src * 4;
 #pragma unroll
-  for (int e = 0; e < 3; ++e)
-    d[e] = nearest_image_unit(__dsub_rn(p[e], a.spos[e * a.n + k] * a.invL)) * a.L;
+  for (int e = 0; e < 3; ++e) {
+    const double p = mono ? m[1 + e] / m[0] : a.spos[e * a.n + src] * a.invL;
+    d[e] = nearest_image_unit(__dsub_rn(p, a.spos[e * a.n + k] * a.invL)) * a.L;
+  }
   const double r2 = __dadd_rn(__dadd_rn(__dmul_rn(d[0], d[0]), __dmul_rn(d[1], d[1])),
                               __dmul_rn(d[2], d[2]));
-  return __dadd_rn(r2, a.eps2) < a.rcut2;
+  const double q = __dadd_rn(r2, a.eps2);
+  return make_float4((float)d[0], (float)d[1], (float)d[2], q < a.rcut2 ? (float)q : -1.f);
 }
 
-// Offset of two-float position (ph, pl) from (xh, xl): the difference of the
-// high parts with its rounding error (Knuth's two-sum), wrapped exactly, plus
-// the low parts; times L. One rounding, up to terms of 2^-48.
-__device__ __forceinline__ float exact_offset(const ExactArgs& a, float ph, float pl, float xh, float xl) {
+// Offset of two-float position (ph, pl) from (xh, xl) as two floats: the
+// difference of the high parts with its rounding error (Knuth's two-sum),
+// wrapped exactly, plus the low parts; times L. x: the offset rounded to FP32,
+// y: what the rounding left. far: the largest |component| so far, box units.
+__device__ __forceinline__ float2 exact_offset(const ExactArgs& a, float ph, float pl, float xh, float xl,
+                                               float& far) {
   const float s = __fsub_rn(ph, xh);
   const float bb = __fsub_rn(s, ph);
   const float err = __fsub_rn(__fsub_rn(ph, __fsub_rn(s, bb)), __fadd_rn(xh, bb));
-  const float w = image32(s), low = __fadd_rn(err, __fsub_rn(pl, xl));
-  return a.unit ? __fadd_rn(w, low) : fmaf(w, a.Lh, fmaf(w, a.Ll, low * a.Lh));
+  float w = image32(s), low = __fadd_rn(err, __fsub_rn(pl, xl));
+  far = fmaxf(far, fabsf(w));
+  if (!a.unit) {
+    const float p = __fmul_rn(w, a.Lh);
+    low = fmaf(w, a.Ll, fmaf(low, a.Lh, fmaf(w, a.Lh, -p)));
+    w = p;
+  }
+  const float h = __fadd_rn(w, low);
+  return make_float2(h, __fsub_rn(low, __fsub_rn(h, w)));
+}
+
+// |d|^2 + eps^2 of two-float offsets: squares with their rounding errors,
+// summed with the errors of the sum (Knuth's two-sum), so that only the last
+// rounding is left, as from an FP64 sum.
+__device__ __forceinline__ float exact_q(const ExactArgs& a, float2 x, float2 y, float2 z) {
+  const float px = __fmul_rn(x.x, x.x), py = __fmul_rn(y.x, y.x), pz = __fmul_rn(z.x, z.x);
+  const float ex = fmaf(x.x + x.x, x.y, fmaf(x.x, x.x, -px));
+  const float ey = fmaf(y.x + y.x, y.y, fmaf(y.x, y.x, -py));
+  const float ez = fmaf(z.x + z.x, z.y, fmaf(z.x, z.x, -pz));
+  float low = (ex + ey) + (ez + a.eps2l);
+  float sum = px;
+  const float add[3] = {py, pz, a.eps2h};
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    const float s = __fadd_rn(sum, add[j]);
+    const float bb = __fsub_rn(s, sum);
+    low += __fadd_rn(__fsub_rn(sum, __fsub_rn(s, bb)), __fsub_rn(add[j], bb));
+    sum = s;
+  }
+  return __fadd_rn(sum, low);
 }
 
 constexpr int kExactWarps = 4;
@@ -285,9 +328,11 @@ struct ExactWarp {
 // rate) the decisions and offsets kept that pipe 85 % busy; they are now made
 // in FP32 with error bounds, in FP64 only where FP32 cannot tell, with the same
 // outcome. 30011 bodies, two species, leaf 8: 11.4 ms with a thread per body,
-// 3.4 ms with a warp per body in FP64, 0.52 ms now. The terms and their number
-// are those of the per-particle count; each lane sums its terms in FP32, the
-// lanes' sums are added at the end.
+// 3.4 ms with a warp per body in FP64, 0.52 ms with FP32 throughout; offsets and
+// |d|^2 with the digits of FP64 cost 6 % (30011 bodies in 8 spheres: a tree force
+// 782 -> 832 us; at 72 and 80 registers, with less spilled, 862 and 901). The terms
+// and their number are those of the per-particle count; each lane sums its terms
+// in FP32, the lanes' sums are added at the end.
 __global__ void __launch_bounds__(32 * kExactWarps, 8) k_walk_exact(ExactArgs a) {
   __shared__ ExactWarp sm[kExactWarps];
   if (a.status[ST_FLAGS] & SF_NODE_OVERFLOW) return;
@@ -411,20 +456,20 @@ __global__ void __launch_bounds__(32 * kExactWarps, 8) k_walk_exact(ExactArgs a)
           pl = a.brec[2 * (size_t)src + 1];
           t = __float_as_int(pl.w);
         }
-        const float dx = exact_offset(a, ph.x, pl.x, xh[0], bl.x);
-        const float dy = exact_offset(a, ph.y, pl.y, xh[1], bl.y);
-        const float dz = exact_offset(a, ph.z, pl.z, xh[2], bl.z);
-        const float q = fmaf(dx, dx, fmaf(dy, dy, fmaf(dz, dz, a.eps2f)));
-        // q is within 4e-7 of its FP64 value
+        float far = 0.f;
+        const float2 x2 = exact_offset(a, ph.x, pl.x, xh[0], bl.x, far);
+        const float2 y2 = exact_offset(a, ph.y, pl.y, xh[1], bl.y, far);
+        const float2 z2 = exact_offset(a, ph.z, pl.z, xh[2], bl.z, far);
+        float dx = x2.x, dy = y2.x, dz = z2.x, q = exact_q(a, x2, y2, z2);
         bool within = q < a.rc2f;
-        if (fabsf(q - a.rc2f) <= 2e-6f * a.rc2f && a.rc2f < 3.0e38f) {
-          double p[3];
-#pragma unroll
-          for (int e = 0; e < 3; ++e) {
-            const double* m = a.m64 + (size_t)src * 4;
-            p[e] = mono ? m[1 + e] / m[0] : a.spos[e * a.n + src] * a.invL;
-          }
-          within = exact_within64(a, p, k);
+        // where two floats or FP32 cannot tell (both rare)
+        if (far < kExactNear || (fabsf(q - a.rc2f) <= 2e-6f * a.rc2f && a.rc2f < 3.0e38f)) {
+          const float4 d = exact_pair64(a, mono, src, k);
+          dx = d.x;
+          dy = d.y;
+          dz = d.z;
+          q = d.w;
+          within = q >= 0.f;
         }
         if (within) exact_term(a, s, t, ph.w, np, mp, dx, dy, dz, q, ax, ay, az);
         ++terms;
@@ -508,7 +553,8 @@ int launch_walk_exact(ng_ctx* c, float* acc, bool accumulate, bool count) {
   a.Lh = (float)c->L;
   a.Ll = (float)(c->L - (double)a.Lh);
   a.theta32 = (float)a.theta;
-  a.eps2f = (float)a.eps2;
+  a.eps2h = (float)a.eps2;
+  a.eps2l = (float)(a.eps2 - (double)a.eps2h);
   a.rc2f = (float)a.rcut2;
   a.cut_lo2 = (float)((rc - 2e-6) * (rc - 2e-6) * 0.999999);
   a.cut_hi2 = (float)((rc + 2e-6) * (rc + 2e-6) * 1.000001);
