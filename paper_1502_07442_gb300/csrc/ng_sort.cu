@@ -554,7 +554,7 @@ __global__ void k_gather(GatherArgs g, const uint32_t* __restrict__ perm) {
 
 // ------------------------------------------------------- small problems
 
-// The whole sort stage of up to kSmallSort bodies in one launch: a body's
+// The whole sort stage of few bodies in one launch: a body's
 // sorted place is the number of keys below its own (and of equal keys of lower
 // index, so the order is that of the stable passes), counted by comparing it
 // with every key; its place in the type-major order counts those of its own
@@ -564,9 +564,14 @@ __global__ void k_gather(GatherArgs g, const uint32_t* __restrict__ perm) {
 // The n^2 comparisons, five instructions each over the whole chip, set the limit.
 // Each block forms all keys (the bodies are read from L2) and ranks 32 * ITEMS
 // bodies, one per lane and item; its warps share out the keys they are compared with.
+// In a box that is a power of two a key is integer work, and a build takes 129 us
+// at 4096 bodies and 153 at 8192 (general path: 186 and 193). In other boxes it is
+// six FP64 divisions, formed again by every block: 195 / 253 / 299 us at 4096 /
+// 6144 / 8192 bodies against 223 / 226 / 229, so there the general path takes over
+// where the two meet, at 5120.
 constexpr int kRkThreads = 512, kRkWarps = kRkThreads / 32;
 constexpr int kRkPad = 4 * kRkWarps;   // keys are padded to whole quads per warp
-constexpr int64_t kSmallSort = 8192;
+constexpr int64_t kSmallSort = 8192, kSmallSortAnyBox = 5120;
 
 static size_t rank_smem(int64_t n) { return (size_t)((n + kRkPad - 1) / kRkPad * kRkPad) * 12; }
 
@@ -722,7 +727,7 @@ static int sort_stage(ng_ctx* c, GatherArgs g) {
   c->sort_passes = 8 - first;
   c->typed = false;
   KeyArgs a{n, g.pos, g.type, g.L, g.invL, g.pow2, g.pow2 ? std::ilogb(c->L) : 0, c->p.D, g.mass, nullptr};
-  if (n <= kSmallSort) {
+  if (n <= (g.pow2 ? kSmallSort : kSmallSortAnyBox)) {
     stage_mark(c, NG_STAGE_KEYS);
     // at most 128 blocks: one round on the SMs
     return n <= kSmallSort / 2 ? sort_rank<1, RESIDENT>(c, a, g, first) : sort_rank<2, RESIDENT>(c, a, g, first);
