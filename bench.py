@@ -121,20 +121,20 @@ def measured_peaks():
 
 
 def stage_bytes(n, D, mesh, passes=8):
-    """Algorithmic DRAM bytes of the memory-bound stages of one force
-    evaluation (reads + writes of the arrays each stage must touch once):
+    """Byte counts by which lines of all builds are compared (reads + writes of
+    the arrays of each memory-bound stage of one force evaluation):
     keys 24 B position + 1 B species read, 8 B key + 4 B index written; each
     radix pass (8 for a full sort, fewer when the step's tree stops at a level
-    cap) 8 B key read by the histogram, 12 B key + index read and 12 B written
-    by the scatter (the bytes of a pass in three launches, kept so that lines of
-    different builds compare; a pass in one launch moves 24 B); type-major order 4 B index written,
+    cap) 8 B key read by a histogram, 12 B key + index read and 12 B written
+    by a scatter; type-major order 4 B index written,
     then one 32 B radix pass; deposit 33 B per body read plus the D mesh
     clears; FFTs and k-space one read and one write of the D real meshes or
     half spectra; interpolation 24 B position + 1 B species + 4 B index read,
     12 B acceleration written, and one read of the D potential meshes. The
     gather of a step (ng_step keeps the state in the previous step's sorted
     order) reads and writes 24 B position, 12 B velocity, 4 B mass, 1 B
-    species, 4 B caller index and reads the 4 B permutation."""
+    species, 4 B caller index and reads the 4 B permutation. Stages whose
+    launches move other bytes by now: see moved_bytes."""
     real = 4 * D * mesh ** 3
     spec = 8 * D * mesh * mesh * (mesh // 2 + 1)
     b = {"keys": 37 * n, "radix": passes * 32 * n, "gather": (2 * 45 + 4) * n, "type_order": 36 * n,
@@ -144,16 +144,35 @@ def stage_bytes(n, D, mesh, passes=8):
     return b
 
 
+def moved_bytes(n, passes=8):
+    """Bytes that the launches of the sort move where these differ from
+    stage_bytes: keys write no index (25 B in, 8 B out); a radix pass is one
+    launch that reads and writes 12 B a body, and the first forms its index
+    instead of reading it; the type-major order reads a species and writes an
+    index."""
+    return {"keys": 33 * n, "radix": (passes * 24 - 4) * n if passes else 0, "type_order": 5 * n}
+
+
 def hbm_block(times, n, D, mesh, passes=8):
+    """Per stage: bytes, rate and fraction of the measured copy bandwidth. Where
+    the launches move other bytes than the basis that lines of all builds share,
+    moved_* are the figures of what they move; the type-major order, whose basis
+    is seven times that, has those alone."""
     peak, src = measured_peaks()
     out = {"peak_gbs": peak, "peak_source": f"{src} copy bandwidth (MEASURED_PEAKS.json hbm_gbs)",
            "radix_passes": passes}
+    moved = moved_bytes(n, passes)
     for k, nbytes in stage_bytes(n, D, mesh, passes).items():
         ms = times.get(k, 0.0)
         if ms > 0:
-            gbs = nbytes / (ms / 1e3) / 1e9
-            out[k] = {"ms": round(ms, 4), "bytes": int(nbytes), "gbs": round(gbs, 1),
-                      "frac": round(gbs / peak, 4)}
+            def rate(b, pre=""):
+                gbs = b / (ms / 1e3) / 1e9
+                return {pre + "bytes": int(b), pre + "gbs": round(gbs, 1), pre + "frac": round(gbs / peak, 4)}
+            out[k] = {"ms": round(ms, 4)}
+            if k != "type_order":
+                out[k].update(rate(nbytes))
+            if k in moved:
+                out[k].update(rate(moved[k], "moved_"))
     for k in ("octree", "monopoles", "groups", "walk"):
         if times.get(k, 0.0) > 0:
             out[k] = {"ms": round(times[k], 4), "bound": "latency / FP64" if k != "walk" else "FP32"}
