@@ -308,10 +308,6 @@ int update_aold(ng_ctx* c, const float* acc) {
 
 // ------------------------------------------------------------ pipeline
 
-static size_t node_bytes(int D) {
-  return 1 + 8 + 4 + 4 + 4 + 1 + 4 + (size_t)D * 32 + (size_t)D * 4 + 16 * 3 + (size_t)D * 16;
-}
-
 int alloc_nodes(ng_ctx* c, int64_t cap) {
   const int D = c->p.D;
   if (cap > c->cap_nodes) c->built = false;   // arrays are replaced
@@ -332,7 +328,6 @@ int alloc_nodes(ng_ctx* c, int64_t cap) {
   NG_TRY(ensure(c, c->mono_words, (kMonoWords + 3 * kMonoBins + 1) * sizeof(uint32_t)));
   if (c->p.pure_tree) NG_TRY(ensure(c, c->exact_node, cap * (2 * D + 1) * 16));
   c->cap_nodes = cap;
-  (void)node_bytes;
   return NG_OK;
 }
 
@@ -393,7 +388,6 @@ int check_flags(ng_ctx* c, uint32_t flags) {
   flags &= ~(uint32_t)SF_DEPTH;   // a capped tree is valid (see SF_DEPTH)
   if (flags & SF_NODE_OVERFLOW) return fail(c, NG_ENOMEM, "tree node capacity exceeded");
   if (flags & SF_STACK_OVERFLOW) return fail(c, NG_ENOMEM, "walk stack capacity exceeded");
-  if (flags & SF_GROUP_OVERFLOW) return fail(c, NG_ENOMEM, "walk group capacity exceeded");
   if (flags & SF_BAD_TYPE) return fail(c, NG_EINVAL, "a species value is >= D");
   if (flags) return fail(c, NG_ECUDA, "device status flags 0x%x", flags);
   return NG_OK;

@@ -42,7 +42,6 @@ enum StatusSlot {
 enum StatusFlag {
   SF_NODE_OVERFLOW = 1,
   SF_STACK_OVERFLOW = 2,
-  SF_GROUP_OVERFLOW = 4,
   SF_BAD_TREE = 8,
   SF_BAD_TYPE = 16,
   // not an error: a build with a level cap (captured steps) kept a node at
@@ -376,11 +375,9 @@ bool give_back_records(ng_ctx* c);
 template <class T>
 inline T* as(const DevBuf& b) { return static_cast<T*>(b.p); }
 
-// Device-wide exclusive scan of uint32 values; len read from *d_len when
-// d_len != nullptr (then len is an upper bound), total written to *d_total
+// Device-wide exclusive scan of len uint32 values, total written to *d_total
 // when non-null. Needs ctx->scan_part scratch.
-int scan_u32(ng_ctx* c, const uint32_t* in, uint32_t* out, int64_t len,
-             const uint32_t* d_len, uint32_t* d_total);
+int scan_u32(ng_ctx* c, const uint32_t* in, uint32_t* out, int64_t len, uint32_t* d_total);
 
 // Stages of the pipeline (each enqueues on c->stream, no host sync).
 int sort_bodies(ng_ctx* c, int64_t n, const double* pos, const uint8_t* type,

@@ -12,16 +12,8 @@ namespace ng {
 constexpr int kScanThreads = 1024;
 constexpr int kScanBlocks = 256;
 
-__device__ __forceinline__ int64_t scan_len(int64_t bound, const uint32_t* d_len) {
-  if (!d_len) return bound;
-  const int64_t l = (int64_t)*d_len;
-  return l < bound ? l : bound;
-}
-
 __global__ void __launch_bounds__(kScanThreads)
-k_scan_partial(const uint32_t* __restrict__ in, int64_t bound, const uint32_t* d_len,
-               uint32_t* part) {
-  const int64_t len = scan_len(bound, d_len);
+k_scan_partial(const uint32_t* __restrict__ in, int64_t len, uint32_t* part) {
   const int64_t chunk = (len + gridDim.x - 1) / gridDim.x;
   const int64_t b0 = (int64_t)blockIdx.x * chunk;
   const int64_t b1 = b0 + chunk < len ? b0 + chunk : len;
@@ -41,12 +33,11 @@ k_scan_partial(const uint32_t* __restrict__ in, int64_t bound, const uint32_t* d
 }
 
 __global__ void __launch_bounds__(kScanThreads)
-k_scan_final(const uint32_t* in, uint32_t* out, int64_t bound, const uint32_t* d_len,
-             const uint32_t* __restrict__ part, uint32_t* d_total) {
+k_scan_final(const uint32_t* in, uint32_t* out, int64_t len, const uint32_t* __restrict__ part,
+             uint32_t* d_total) {
   __shared__ uint32_t warp_tot[32];
   __shared__ uint32_t tile_total;
   __shared__ uint32_t off;
-  const int64_t len = scan_len(bound, d_len);
   const int64_t chunk = (len + gridDim.x - 1) / gridDim.x;
   const int64_t b0 = (int64_t)blockIdx.x * chunk;
   const int64_t b1 = b0 + chunk < len ? b0 + chunk : len;
@@ -76,15 +67,14 @@ static int scan_blocks(int64_t len) {
       1, std::min<int64_t>(kScanBlocks, (len + 4 * kScanThreads - 1) / (4 * kScanThreads)));
 }
 
-int scan_u32(ng_ctx* c, const uint32_t* in, uint32_t* out, int64_t len, const uint32_t* d_len,
-             uint32_t* d_total) {
+int scan_u32(ng_ctx* c, const uint32_t* in, uint32_t* out, int64_t len, uint32_t* d_total) {
   NG_TRY(ensure(c, c->scan_part, kScanBlocks * sizeof(uint32_t)));
   uint32_t* part = as<uint32_t>(c->scan_part);
   // blocks for at most 4 tiles each; both kernels split the range by gridDim
   const int blocks = scan_blocks(len);
   // one block needs no partial sums (its offset is zero)
-  if (blocks > 1) k_scan_partial<<<blocks, kScanThreads, 0, c->stream>>>(in, len, d_len, part);
-  k_scan_final<<<blocks, kScanThreads, 0, c->stream>>>(in, out, len, d_len, part, d_total);
+  if (blocks > 1) k_scan_partial<<<blocks, kScanThreads, 0, c->stream>>>(in, len, part);
+  k_scan_final<<<blocks, kScanThreads, 0, c->stream>>>(in, out, len, part, d_total);
   c->launches += blocks > 1 ? 2 : 1;
   NG_CUDA(c, cudaGetLastError());
   return NG_OK;

@@ -324,7 +324,7 @@ int build_octree(ng_ctx* c) {
   // up to kSumTiles tiles, adding their counts up again in every block costs
   // less than a scan's launch (4096 bodies: 3.6 us; 131k: 5.5 us)
   const bool sum = tiles <= kSumTiles;
-  if (!sum) NG_TRY(scan_u32(c, cnt, cnt, (int64_t)tiles * (lmax + 1), nullptr, st + ST_NODES_NEEDED));
+  if (!sum) NG_TRY(scan_u32(c, cnt, cnt, (int64_t)tiles * (lmax + 1), st + ST_NODES_NEEDED));
   (sum ? k_tree_emit<true> : k_tree_emit<false>)<<<tiles, kTreeThreads, 0, c->stream>>>(
       keys, n, leaf, lmax, cnt, st, cap, as<uint8_t>(c->n_level), as<uint64_t>(c->n_prefix),
       as<uint32_t>(c->n_first), as<uint32_t>(c->n_child),
