@@ -410,9 +410,11 @@ int ng_serve_stats(const ng_server* s, size_t* held_bytes, size_t* peak_held_byt
 
 /*
  * Stages of one force evaluation, in execution order (ng_stage_times):
- * Morton+type keys, the 8 radix passes, the gather into sorted order, the
- * octree levels, the monopoles, the walk groups, the type-major order, the
- * PM deposit (mesh clear + CIC), forward FFTs, k-space kernels, inverse
+ * Morton+type keys, the radix passes, the gather into sorted order, the
+ * octree, the monopoles, the walk groups, the type-major order (up to 8192
+ * bodies, 5120 in a box that is not a power of two, one launch does all of the
+ * sort: its time is NG_STAGE_KEYS, and the passes, the gather and the
+ * type-major order report 0), the PM deposit (mesh clear + CIC), forward FFTs, k-space kernels, inverse
  * FFTs, gradient + interpolation, and the short-range tree force.
  */
 enum {
@@ -446,10 +448,11 @@ int ng_stage_times(ng_ctx* ctx, int64_t n, double* pos, float* vel, const uint8_
 int ng_launch_count(const ng_ctx* ctx, uint64_t* out);
 
 /*
- * Radix passes (8 key bits each) of the context's last key sort: 8 for a
- * canonical build; fewer in steps whose trees stop at a level cap (captured
- * steps, served integrations), which sort only the Morton bits of their
- * levels. Sizes the sort's bytes in per-stage bandwidth figures.
+ * 8-bit digits that the context's last key sort ordered, a radix pass each
+ * where it ran in passes (see the stages above): 8 for a canonical build; fewer
+ * in steps whose trees stop at a level cap (captured steps, served
+ * integrations), which sort only the Morton bits of their levels. Sizes the
+ * sort's bytes in per-stage bandwidth figures.
  */
 int ng_sort_passes(const ng_ctx* ctx, int32_t* out);
 

@@ -28,7 +28,6 @@ constexpr int kLeafBins = 66;
 constexpr int kMonoBins = kLeafBins + 8;
 constexpr int64_t kBinnedMonoBodies = 1 << 20;
 constexpr int64_t kPackBodies = 1 << 17;   // sorts gather packed records (ng_sort.cu)
-constexpr int kWarp = 32;
 
 // Status words in device memory (ctx->status).
 enum StatusSlot {
@@ -61,10 +60,7 @@ struct DevBuf {
 // Walk tuning constants.
 constexpr int kStackCap = 384;          // node stack entries per warp
 constexpr int kStackReserve = 7 * kMaxLevel + 8 + 32;   // depth-first descent + push-backs
-constexpr int kWalkMaxWarps = 32;
-// Warps per walk block by species count: as many as the per-warp lists and a
-// 64 KB law table leave room for in 227 KB of shared memory; the register
-// budget follows (65536 / threads).
+
 // Every third bit of v, from bit 0, packed into the low 21 bits: one axis
 // of a Morton key or node prefix (x from v >> 2, y from v >> 1, z from v).
 __device__ __forceinline__ uint32_t morton_compact3(uint64_t v) {
@@ -178,6 +174,9 @@ __host__ __device__ constexpr int walk_tab_shift(int D) { return D <= 1 ? 0 : D 
 // Warps per walk block (one block per SM): registers and the per-warp lists
 // bound them. The variable-species instance of batches, laid out for six
 // species, runs 24 warps when its law table is small (a few distinct laws).
+// Warps per walk block by species count: as many as the per-warp lists and a
+// 64 KB law table leave room for in 227 KB of shared memory; the register
+// budget follows (65536 / threads).
 __host__ __device__ constexpr int walk_warps(int D) { return D <= 3 ? 24 : D == 4 ? 24 : D == 5 ? 20 : 16; }
 constexpr int kVardWarps = 24;
 // Records per species list per warp: as many as fit beside the default law

@@ -140,7 +140,7 @@ constexpr double kFirstTreeWait = 120.0;
 // was prepared by prepare_slot). For an integration the thread waits (bounded)
 // for the first tree only, while the first force runs: the trees of the steps
 // then stop two levels below its depth (cells at the cap stay leaves, a valid
-// tree; see SF_DEPTH), which saves the launches of the empty deeper levels.
+// tree; see SF_DEPTH), and their sorts skip the key passes below.
 int launch_request(ng_server* s, Slot& sl, Req& q) {
   ng_ctx* c = sl.ctx;
   c->stream = sl.stream;

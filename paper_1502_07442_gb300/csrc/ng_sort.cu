@@ -98,7 +98,7 @@ struct KeyArgs {
 // which has the positions in hand, writes them wrapped, with mass and species,
 // as one 32-byte record, and the gather reads one sector (3 M bodies: keys 34 ->
 // 47 us, gather 108 -> 46 us; a build 1161 -> 1118 us). At 131k bodies, all in L2,
-// it is still 5 us of a 650 us force; below it would cost more memory for less.
+// it is still 5 us of a 650 us force; smaller sizes were not tried.
 __device__ __forceinline__ double4_32a pack_body(double x, double y, double z, float mass, uint8_t type) {
   const uint64_t mt = (uint64_t)type << 32 | __float_as_uint(mass);
   return make_double4_32a(x, y, z, __longlong_as_double((long long)mt));
@@ -165,7 +165,8 @@ k_keys(KeyArgs a, int first, uint64_t* __restrict__ keys, uint32_t* words,
 constexpr int kRsThreads = 256;
 constexpr int kRsWarps = kRsThreads / 32;
 constexpr int kRsItemsSmall = 4, kRsItemsLarge = 16;
-// two tiles of the larger kind per SM
+// two tiles of the larger kind per SM of a GB300. (Fixed, since the look-back state
+// is sized by it: fewer bodies than this can need more of it than more bodies do.)
 constexpr int64_t kRsLarge = (int64_t)2 * 152 * kRsThreads * kRsItemsLarge;
 
 // Look-back state of one pass. Tiles form groups of kRsGroup: a tile adds up

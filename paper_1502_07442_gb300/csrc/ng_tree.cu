@@ -529,7 +529,9 @@ __device__ __forceinline__ void mono_internal_lane(const MonoNode& v, const Mono
 // children are not formed yet (x). Who forms a node takes one off its parent's
 // count, and who takes the last one forms the parent next. The nodes without
 // internal children are ready at the start.
-// The sums are always over all children in the same order, whoever forms the node.
+// Which sum a node takes, pairwise in a team (mono_sum) or child by child in a
+// lane (mono_internal_lane: the nodes without internal children of trees of
+// kBinnedMonoBodies bodies or more), is set by the tree, so results repeat.
 // Bound by latency: a level of a path costs two dependent loads, the additions
 // and one counter. Subtrees of 256 bodies by one block each, level by level
 // with barriers, and a cluster of eight blocks for the nodes above took 88 us at
@@ -792,7 +794,7 @@ __global__ void __launch_bounds__(kMonoThreads) k_mono_up(MonoArgs a, const uint
 // thread in its own order, so the results do not depend on the binning.
 // Tiles take no order first and read the bodies coalesced; this order keeps the
 // FP64 pipe's lanes full, which a tile's few leaves do not when leaves are
-// large. Passes with tiles / in this order: a force on 131k bodies 664 / 676 us,
+// large (leaf sizes 9 to 31 from kBinnedMonoBodies bodies were not timed). Passes with tiles / in this order: a force on 131k bodies 664 / 676 us,
 // a 200k-body step 668 / 698 us, a build of 3 M bodies in leaves of 8 1053 /
 // 1114 us, two steps of 2^24 bodies in leaves of 32 145.5 / 144.3 ms: tiles
 // below kBinnedMonoBodies bodies and for leaves up to kTileLeaf.

@@ -619,6 +619,8 @@ static int launch_walk_t(ng_ctx* c, cudaStream_t stream, WalkLaunch L, int64_t g
 // on 4096 bodies (0.05 groups per slot) 310 / 262 / 248 / 245 us, on 131k bodies
 // (1.4 per slot) 692 / 682 / 740 / 902 us, a 200k-body step (2.1) 708 / 704 /
 // 767 / 959 us, a 300k-body tree force (4, six species) 1006 / 1110 / 1346 / 1877 us.
+// Batches keep whole groups per warp: one queue holds the groups of all members.
+// Teams were not tried there.
 static int walk_team(int64_t groups, int64_t slots) {
   return groups <= slots / 8 ? 8 : groups <= slots / 2 ? 4 : groups <= 3 * slots ? 2 : 1;
 }
