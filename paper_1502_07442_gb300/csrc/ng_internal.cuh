@@ -171,12 +171,11 @@ __device__ __forceinline__ uint64_t sort_key(double x, double y, double z, uint8
 __host__ __device__ constexpr int walk_tab_pad(int D) { return D <= 1 ? 1 : D == 2 ? 2 : D <= 4 ? 4 : 8; }
 __host__ __device__ constexpr int walk_tab_shift(int D) { return D <= 1 ? 0 : D == 2 ? 1 : D <= 4 ? 2 : 3; }
 
-// Warps per walk block (one block per SM): registers and the per-warp lists
-// bound them. The variable-species instance of batches, laid out for six
-// species, runs 24 warps when its law table is small (a few distinct laws).
-// Warps per walk block by species count: as many as the per-warp lists and a
+// Warps per walk block (one block per SM): as many as the per-warp lists and a
 // 64 KB law table leave room for in 227 KB of shared memory; the register
-// budget follows (65536 / threads).
+// budget follows (65536 / threads). The variable-species instance of batches,
+// laid out for six species, runs 24 warps when its law table is small (a few
+// distinct laws).
 __host__ __device__ constexpr int walk_warps(int D) { return D <= 3 ? 24 : D == 4 ? 24 : D == 5 ? 20 : 16; }
 constexpr int kVardWarps = 24;
 // Records per species list per warp: as many as fit beside the default law
