@@ -17,3 +17,8 @@ def test_moved_bytes_beside_the_shared_basis(monkeypatch):
     assert "frac" not in h["type_order"]         # its basis is seven times what it moves
     assert h["keys"]["bytes"] == 37 * n and h["radix"]["bytes"] == 6 * 32 * n
     assert "moved_bytes" not in bench.hbm_block({"gather": 1.0}, n, 4, 0)["gather"]
+
+
+def test_passes_are_those_of_the_reported_radix_time():
+    calls = [({"radix": 1.3, "keys": 0.2}, 8), ({"radix": 1.0, "keys": 0.3}, 6), ({"radix": 1.4, "keys": 0.1}, 8)]
+    assert bench.best_stages(calls) == ({"radix": 1.0, "keys": 0.1}, 6)
